@@ -1,7 +1,7 @@
 // exact64.cuh -- FP64 results without the FP64 pipe.  An SM of this GPU issues about two
 // FP64 operations per clock (conversions to and from FP64 included) against 64 integer and
 // 128 FP32 ones, so the boundary kernels, which hand FP32 and FP16 states out as FP64
-// arrays, are bound by that pipe and not by memory when they add and divide in FP64.
+// arrays, are bound by that pipe and not by memory when they convert, add and divide in FP64.
 // Everything here gives the value that the FP64 instruction sequence gives.
 #pragma once
 
@@ -9,6 +9,16 @@
 #include <cuda_runtime.h>
 
 namespace kss {
+
+// double(x): a normal number's sign, exponent (rebiased by 1023 - 127 = 896) and fraction
+// move to their FP64 places; zero, subnormals, infinities and NaN take the conversion.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t b = __float_as_uint(x);
+  if (((b + 0x00800000u) & 0x7f000000u) == 0u) return double(x);  // exponent field 0 or 255
+  return __hiloint2double(int((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))),
+                          int(b << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
 
 // The rounded quotient j / r of two integers, |j| and 0 < r below 2^53 (jd, rd: the
 // magnitudes scaled into [1, 2), yd about 1 / rd): q0 = jd yd, then one correction by the

@@ -13,6 +13,13 @@ inline dim3 helper_grid(int nx, long long rows) {
   return dim3((unsigned)((nx + 255) / 256), (unsigned)(rows < 65535 ? rows : 65535));
 }
 
+// Columns per thread of the kernels between pitched planes and a dense FP64 array: two
+// where every pair of columns of every row is 16-byte aligned there.  (Rows of the planes
+// always are: their pitch is a multiple of 128 bytes.)
+inline int dense_vec(const void* dense, int nx) {
+  return (nx % 2 == 0 && reinterpret_cast<uintptr_t>(dense) % 16 == 0) ? 2 : 1;
+}
+
 // Let `kernel` take DYN bytes of dynamic shared memory on the current device (beyond the
 // default 48 KB of static plus dynamic memory an opt-in is needed), once per device.
 // Threads that race here at most repeat the (idempotent) attribute call.
@@ -357,8 +364,10 @@ template <>
 cudaError_t launch_pops_to_dense<KSS_T>(const KSS_T* src, long long plane, int pitch, int nx,
                                         int ny, double* dst, const codec_t<KSS_T>& codec,
                                         cudaStream_t stream) {
-  pops_to_dense_kernel<KSS_T><<<helper_grid(nx, ny), 256, 0, stream>>>(
-      src, plane, pitch, nx, ny, dst, codec);
+  if (dense_vec(dst, nx) == 2)
+    pops_to_dense_kernel<KSS_T, 2><<<helper_grid((nx + 1) / 2, ny), 256, 0, stream>>>(src, plane, pitch, nx, ny, dst, codec);
+  else
+    pops_to_dense_kernel<KSS_T, 1><<<helper_grid(nx, ny), 256, 0, stream>>>(src, plane, pitch, nx, ny, dst, codec);
   return cudaGetLastError();
 }
 
@@ -366,8 +375,10 @@ template <>
 cudaError_t launch_dense_to_pops<KSS_T>(const double* src, long long plane, int pitch, int nx,
                                         int ny, KSS_T* dst, const codec_t<KSS_T>& codec,
                                         cudaStream_t stream) {
-  dense_to_pops_kernel<KSS_T><<<helper_grid(nx, ny), 256, 0, stream>>>(
-      src, plane, pitch, nx, ny, dst, codec);
+  if (dense_vec(src, nx) == 2)
+    dense_to_pops_kernel<KSS_T, 2><<<helper_grid((nx + 1) / 2, ny), 256, 0, stream>>>(src, plane, pitch, nx, ny, dst, codec);
+  else
+    dense_to_pops_kernel<KSS_T, 1><<<helper_grid(nx, ny), 256, 0, stream>>>(src, plane, pitch, nx, ny, dst, codec);
   return cudaGetLastError();
 }
 
@@ -375,16 +386,20 @@ cudaError_t launch_dense_to_pops<KSS_T>(const double* src, long long plane, int 
 template <>
 cudaError_t launch_pitched_to_dense<KSS_T>(const KSS_T* src, long long plane, int pitch, int nx,
                                            int ny, int nplanes, double* dst, cudaStream_t stream) {
-  pitched_to_dense_kernel<KSS_T><<<helper_grid(nx, ny), 256, 0, stream>>>(
-      src, plane, pitch, nx, ny, nplanes, dst);
+  if (dense_vec(dst, nx) == 2)
+    pitched_to_dense_kernel<KSS_T, 2><<<helper_grid((nx + 1) / 2, ny), 256, 0, stream>>>(src, plane, pitch, nx, ny, nplanes, dst);
+  else
+    pitched_to_dense_kernel<KSS_T, 1><<<helper_grid(nx, ny), 256, 0, stream>>>(src, plane, pitch, nx, ny, nplanes, dst);
   return cudaGetLastError();
 }
 
 template <>
 cudaError_t launch_dense_to_pitched<KSS_T>(const double* src, long long plane, int pitch, int nx,
                                            int ny, int nplanes, KSS_T* dst, cudaStream_t stream) {
-  dense_to_pitched_kernel<KSS_T><<<helper_grid(nx, ny), 256, 0, stream>>>(
-      src, plane, pitch, nx, ny, nplanes, dst);
+  if (dense_vec(src, nx) == 2)
+    dense_to_pitched_kernel<KSS_T, 2><<<helper_grid((nx + 1) / 2, ny), 256, 0, stream>>>(src, plane, pitch, nx, ny, nplanes, dst);
+  else
+    dense_to_pitched_kernel<KSS_T, 1><<<helper_grid(nx, ny), 256, 0, stream>>>(src, plane, pitch, nx, ny, nplanes, dst);
   return cudaGetLastError();
 }
 #endif  // KSS_STORAGE_HALF

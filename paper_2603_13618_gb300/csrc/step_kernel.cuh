@@ -2461,54 +2461,101 @@ __global__ void moments_kernel(const S* __restrict__ f, long long plane, int pit
   }
 }
 
+// ---- pitched planes <-> dense FP64 arrays ----
+// A thread moves V columns of a row, all planes of a group at once so that their loads are
+// in flight together: V = 2 (16-byte accesses of the dense array) where the dense pointer is
+// 16-byte aligned and nx even, V = 1 elsewhere (dense_vec).  FP32 values are widened in
+// integer arithmetic (exact64.cuh), off the FP64 pipe.  4096^2 FP32 lattice, into device
+// memory: populations 0.41 -> 0.31 ms (their 108 bytes per cell alone take 0.27 ms), a
+// sensor field 0.107 -> 0.077 ms.  (Narrowing in integer arithmetic too, with its rounding
+// and the branch for special values, made kss_set_populations slower: 0.36 -> 0.57 ms.)
+template <class S, int V>
+struct alignas(sizeof(S) * V) ColVec {
+  S v[V];
+};
+
 // The nine population planes (decoded) <-> dense double planes [9][ny][nx].
-template <class S>
+template <class S, int V>
 __global__ void pops_to_dense_kernel(const S* __restrict__ src, long long plane, int pitch,
                                      int nx, int ny, double* __restrict__ dst,
                                      const codec_t<S> codec) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  using In = ColVec<S, V>;
+  using Out = ColVec<double, V>;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) * V;
   if (i >= nx) return;
+  for (int j = blockIdx.y; j < ny; j += gridDim.y) {
+    In a[9];
 #pragma unroll
-  for (int q = 0; q < 9; ++q)
-    for (int j = blockIdx.y; j < ny; j += gridDim.y)
-      dst[((long long)q * ny + j) * nx + i] =
-          double(decode<S>(src[q * plane + (long long)j * pitch + i], q, codec));
+    for (int q = 0; q < 9; ++q)
+      a[q] = *reinterpret_cast<const In*>(src + q * plane + (long long)j * pitch + i);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+      Out o;
+#pragma unroll
+      for (int k = 0; k < V; ++k) o.v[k] = widen(decode<S>(a[q].v[k], q, codec));
+      *reinterpret_cast<Out*>(dst + ((long long)q * ny + j) * nx + i) = o;
+    }
+  }
 }
 
-template <class S>
+template <class S, int V>
 __global__ void dense_to_pops_kernel(const double* __restrict__ src, long long plane,
                                      int pitch, int nx, int ny, S* __restrict__ dst,
                                      const codec_t<S> codec) {
   using T = arith_t<S>;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  using In = ColVec<double, V>;
+  using Out = ColVec<S, V>;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) * V;
   if (i >= nx) return;
+  for (int j = blockIdx.y; j < ny; j += gridDim.y) {
+    In a[9];
 #pragma unroll
-  for (int q = 0; q < 9; ++q)
-    for (int j = blockIdx.y; j < ny; j += gridDim.y)
-      dst[q * plane + (long long)j * pitch + i] =
-          encode<S>(T(src[((long long)q * ny + j) * nx + i]), q, codec);
+    for (int q = 0; q < 9; ++q)
+      a[q] = *reinterpret_cast<const In*>(src + ((long long)q * ny + j) * nx + i);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+      Out o;
+#pragma unroll
+      for (int k = 0; k < V; ++k) o.v[k] = encode<S>(T(a[q].v[k]), q, codec);
+      *reinterpret_cast<Out*>(dst + q * plane + (long long)j * pitch + i) = o;
+    }
+  }
 }
 
 // nplanes pitched T planes <-> dense double planes (sensor fields, weights).
-template <class T>
+template <class T, int V>
 __global__ void pitched_to_dense_kernel(const T* __restrict__ src, long long plane, int pitch,
                                         int nx, int ny, int nplanes, double* __restrict__ dst) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  using In = ColVec<T, V>;
+  using Out = ColVec<double, V>;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) * V;
   if (i >= nx) return;
   for (int q = 0; q < nplanes; ++q)
-    for (int j = blockIdx.y; j < ny; j += gridDim.y)
-      dst[((long long)q * ny + j) * nx + i] = double(src[q * plane + (long long)j * pitch + i]);
+    for (int j = blockIdx.y; j < ny; j += gridDim.y) {
+      const In a = *reinterpret_cast<const In*>(src + q * plane + (long long)j * pitch + i);
+      Out o;
+#pragma unroll
+      for (int k = 0; k < V; ++k) o.v[k] = widen(a.v[k]);
+      *reinterpret_cast<Out*>(dst + ((long long)q * ny + j) * nx + i) = o;
+    }
 }
 
-template <class T>
+template <class T, int V>
 __global__ void dense_to_pitched_kernel(const double* __restrict__ src, long long plane,
                                         int pitch, int nx, int ny, int nplanes,
                                         T* __restrict__ dst) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  using In = ColVec<double, V>;
+  using Out = ColVec<T, V>;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) * V;
   if (i >= nx) return;
   for (int q = 0; q < nplanes; ++q)
-    for (int j = blockIdx.y; j < ny; j += gridDim.y)
-      dst[q * plane + (long long)j * pitch + i] = T(src[((long long)q * ny + j) * nx + i]);
+    for (int j = blockIdx.y; j < ny; j += gridDim.y) {
+      const In a = *reinterpret_cast<const In*>(src + ((long long)q * ny + j) * nx + i);
+      Out o;
+#pragma unroll
+      for (int k = 0; k < V; ++k) o.v[k] = T(a.v[k]);
+      *reinterpret_cast<Out*>(dst + q * plane + (long long)j * pitch + i) = o;
+    }
 }
 
 }  // namespace kss
