@@ -184,10 +184,24 @@ static_assert(opp(1) == 3 && opp(2) == 4 && opp(3) == 1 && opp(4) == 2 && opp(5)
 //   KL = |sum f^eq phi(x)|,  HR = |sum f^neq L + sum f^eq phi(x)|,
 //   sigma_H = (sum f^neq L + sum f^neq ln(1+x)) / tau,
 //   sigma_KL = sum f^neq ln(1+x) / tau,   L_q = ln(f^eq_q / (w_q rho)).
+//
+// need (MODE_FULL): the sensors that are read (bit s: sensor s), uniform over the launch.
+// Groups of sensors that nothing reads are skipped, so the entries of o.sv outside `need`
+// may be left unset.  The costly parts are the 18 logarithms (of 1 + x for sigma_H and
+// sigma_KL, of f^eq / (w rho) for HR and sigma_H) and the alpha polynomial: a 2048^2 FP32
+// step took 212 us whatever it needed; with the groups skipped, in the same kernel, 99 us
+// for the strain sensor S, 108 us for alpha, 122 us for sigma_KL, 166 us for HR and KL.
 template <class T, int MODE, bool COLLIDE, bool AAR = false>
 __device__ __forceinline__ void cell_update(const T (&ft)[9], T omega, T tau, T (&fo)[9],
                                             CellOut<T>& o, const Trt<T>& trt = Trt<T>{},
-                                            bool sw = false) {
+                                            bool sw = false, uint32_t need = ~0u) {
+  constexpr uint32_t kRatio = (1u << S_KN) | (1u << S_KL) | (1u << S_HR) | (1u << S_SIGMA_H) |
+                              (1u << S_SIGMA_KL);
+  constexpr uint32_t kPhi = (1u << S_KL) | (1u << S_HR);
+  constexpr uint32_t kTensor = (1u << S_TAU_NS) | (1u << S_C) | (1u << S_S) | (1u << S_E) |
+                               (1u << S_QH);
+  constexpr uint32_t kLin = (1u << S_HR) | (1u << S_SIGMA_H);
+  constexpr uint32_t kSig = (1u << S_SIGMA_H) | (1u << S_SIGMA_KL);
   const T rho = ((ft[0] + ft[1]) + (ft[2] + ft[3])) + ((ft[4] + ft[5]) + (ft[6] + ft[7])) + ft[8];
   const T jx = (ft[1] + ft[5] + ft[8]) - (ft[3] + ft[6] + ft[7]);
   const T jy = (ft[2] + ft[5] + ft[6]) - (ft[4] + ft[7] + ft[8]);
@@ -223,10 +237,23 @@ __device__ __forceinline__ void cell_update(const T (&ft)[9], T omega, T tau, T 
   for (int q = 0; q < 9; ++q) {
     fneq[q] = ft[q] - feq[q];
     nonpos |= (ft[q] <= T(0)) | (feq[q] <= T(0));
-    x[q] = fneq[q] * Num<T>::rcp(feq[q]);
-    kn += fabs(x[q]);
     neq += fabs(fneq[q]);
-    kl = fma(feq[q], phi<T>(x[q]), kl);
+    if (MODE != MODE_FULL) {
+      x[q] = fneq[q] * Num<T>::rcp(feq[q]);
+      kn += fabs(x[q]);
+      kl = fma(feq[q], phi<T>(x[q]), kl);
+    }
+  }
+  if (MODE == MODE_FULL && (need & kRatio)) {
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+      x[q] = fneq[q] * Num<T>::rcp(feq[q]);
+      kn += fabs(x[q]);
+    }
+    if (need & kPhi) {
+#pragma unroll
+      for (int q = 0; q < 9; ++q) kl = fma(feq[q], phi<T>(x[q]), kl);
+    }
   }
   const T kInf = Num<T>::inf();
   o.nonpos = nonpos;
@@ -243,19 +270,19 @@ __device__ __forceinline__ void cell_update(const T (&ft)[9], T omega, T tau, T 
   if (MODE != MODE_FULL) return;
 
   // ---- class 1: the non-equilibrium pressure tensor P^neq = sum c c f^neq ----
-  const T diag = (fneq[5] + fneq[6]) + (fneq[7] + fneq[8]);
-  const T pxx = (fneq[1] + fneq[3]) + diag;
-  const T pyy = (fneq[2] + fneq[4]) + diag;
-  const T pxy = (fneq[5] - fneq[6]) + (fneq[7] - fneq[8]);
-  const T mu = rho * (tau * T(1.0 / 3.0));  // mu = rho c_s^2 tau, lambda = 0, eta = mu
-  const T inv_mu = Num<T>::rcp(mu);
-  const T norm_p = Num<T>::sqrt_(fma(pxx, pxx, fma(pyy, pyy, T(2) * pxy * pxy)));
-  const T half_dev = T(0.5) * (pyy - pxx);  // tr P / 2 - P_xx
-  o.sv[S_TAU_NS] = norm_p;
-  o.sv[S_C] = T(1.4142135623730951) * fabs(pxx + pyy) * (T(0.5) * inv_mu);
-  o.sv[S_S] = Num<T>::sqrt_(T(2) * fma(half_dev, half_dev, pxy * pxy)) * inv_mu;
-  o.sv[S_E] = norm_p * (T(0.5) * inv_mu);
-  {
+  if (need & kTensor) {
+    const T diag = (fneq[5] + fneq[6]) + (fneq[7] + fneq[8]);
+    const T pxx = (fneq[1] + fneq[3]) + diag;
+    const T pyy = (fneq[2] + fneq[4]) + diag;
+    const T pxy = (fneq[5] - fneq[6]) + (fneq[7] - fneq[8]);
+    const T mu = rho * (tau * T(1.0 / 3.0));  // mu = rho c_s^2 tau, lambda = 0, eta = mu
+    const T inv_mu = Num<T>::rcp(mu);
+    const T norm_p = Num<T>::sqrt_(fma(pxx, pxx, fma(pyy, pyy, T(2) * pxy * pxy)));
+    const T half_dev = T(0.5) * (pyy - pxx);  // tr P / 2 - P_xx
+    o.sv[S_TAU_NS] = norm_p;
+    o.sv[S_C] = T(1.4142135623730951) * fabs(pxx + pyy) * (T(0.5) * inv_mu);
+    o.sv[S_S] = Num<T>::sqrt_(T(2) * fma(half_dev, half_dev, pxy * pxy)) * inv_mu;
+    o.sv[S_E] = norm_p * (T(0.5) * inv_mu);
     const T qx = fma(ux, pxx, uy * pxy), qy = fma(ux, pxy, uy * pyy);
     o.sv[S_QH] = Num<T>::sqrt_(fma(qx, qx, qy * qy));
   }
@@ -263,7 +290,7 @@ __device__ __forceinline__ void cell_update(const T (&ft)[9], T omega, T tau, T 
   // ---- entropy-based sensors ----
   // L_q = ln(f^eq_q / (w_q rho)) = ln(1 + 3 c.u + 9/2 (c.u)^2 - 3/2 u.u)
   T lin = T(0), sig = T(0);
-  {
+  if (need & kLin) {
     const T usq15 = T(1.5) * fma(ux, ux, uy * uy);
     const T s = ux + uy, d = uy - ux;
     T arg[9];
@@ -277,10 +304,11 @@ __device__ __forceinline__ void cell_update(const T (&ft)[9], T omega, T tau, T 
     arg[6] = fma(T(4.5) * d, d, fma(T(3), d, -usq15));
     arg[8] = fma(T(4.5) * d, d, fma(T(-3), d, -usq15));
 #pragma unroll
-    for (int q = 0; q < 9; ++q) {
-      lin = fma(fneq[q], Num<T>::log1p_(arg[q]), lin);
-      sig = fma(fneq[q], Num<T>::log1p_(x[q]), sig);
-    }
+    for (int q = 0; q < 9; ++q) lin = fma(fneq[q], Num<T>::log1p_(arg[q]), lin);
+  }
+  if (need & kSig) {
+#pragma unroll
+    for (int q = 0; q < 9; ++q) sig = fma(fneq[q], Num<T>::log1p_(x[q]), sig);
   }
   const T inv_tau = omega;  // 1 / tau
   o.sv[S_HR] = nonpos ? kInf : fabs(lin + kl);
@@ -290,7 +318,7 @@ __device__ __forceinline__ void cell_update(const T (&ft)[9], T omega, T tau, T 
   // ---- entropic estimate: literal polynomial with f^neq = f - f^eq ----
   // a_n = (-1)^(n-1)/(n(n+1)) sum (f^neq)^(n+1)/f^n ;  |2 - alpha| =
   // |4 r2 - 16 r2^2 + 8 r3 - 80 r2 r3 + 80 r2^3 + 16 r4|, r_n = a_n / a_1.
-  {
+  if (need & (1u << S_ALPHA)) {
     T s1 = T(0), s2 = T(0), s3 = T(0), s4 = T(0);
 #pragma unroll
     for (int q = 0; q < 9; ++q) {

@@ -214,7 +214,8 @@ cudaError_t launch_eval(kss_lattice* L, int sensor, bool keep) {
     p.rec_slot[sensor] = 0;
     extra = 1u << sensor;
   }
-  return kss::launch_step<S>(p, mode_for(needed_mask(L, extra)), pull, false, L->stream);
+  p.need = needed_mask(L, extra);
+  return kss::launch_step<S>(p, mode_for(p.need), pull, false, L->stream);
 }
 
 // A device word that nothing ever writes: the bounded wait of kss_testing_expire_wait

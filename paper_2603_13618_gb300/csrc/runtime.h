@@ -202,6 +202,7 @@ kss::StepParams<S> make_params(const kss_lattice* L, const void* src, void* dst)
   p.refine_s = L->cfg.refine_sensor;
   p.switch_s = L->cfg.switch_sensor;
   for (int s = 0; s < KSS_S_COUNT; ++s) p.rec_slot[s] = L->rec_slot[s];
+  p.need = needed_mask(L, L->cfg.record_mask);
   p.codec = codec_of<S>(L);
   p.region = L->region;
   if (L->cfg.tau2 > 0.0) {

@@ -54,8 +54,12 @@ namespace kss {
 //                        CTAs (80 registers).
 //   KSS_F16_MIN_BLOCKS   FP16-deviation {Kn, KL, neq} steps: three (0.659 ms per 8192^2 step
 //                        against 0.706 ms at two: its 8-byte rows need more warps in flight).
-//   KSS_FULL_MIN_BLOCKS  the all-sensor steps (much more per-cell state): two CTAs (at most
-//                        128 registers) against one (158 registers).
+//   KSS_FULL_MIN_BLOCKS  the all-sensor steps with FP32 arithmetic: four CTAs at 64 registers
+//                        (2048^2 FP32, all of Table 1: 217 / 189 / 179 / 195 us at two /
+//                        three / four / five; the strain sensor alone: 114 / 96 / 80 / 86 us).
+//                        FP64 ones keep two: the FP64 pipe bounds them (8.0 ms at two and at
+//                        four), and so do batches, whose members with the {Kn, KL, neq} set
+//                        share the kernel and spill below 128 registers.
 #ifndef KSS_F32_MIN_BLOCKS
 #define KSS_F32_MIN_BLOCKS 2
 #endif
@@ -63,7 +67,7 @@ namespace kss {
 #define KSS_STEP_MIN_BLOCKS 3
 #endif
 #ifndef KSS_FULL_MIN_BLOCKS
-#define KSS_FULL_MIN_BLOCKS 2
+#define KSS_FULL_MIN_BLOCKS 4
 #endif
 #ifndef KSS_F16_MIN_BLOCKS
 #define KSS_F16_MIN_BLOCKS KSS_STEP_MIN_BLOCKS
@@ -81,7 +85,7 @@ namespace kss {
 // The knob of a step kernel with storage S and sensor set MODE.
 template <class S, int MODE>
 __host__ __device__ constexpr int step_min_blocks() {
-  return MODE == MODE_FULL ? KSS_FULL_MIN_BLOCKS
+  return MODE == MODE_FULL ? (std::is_same<S, double>::value ? 2 : KSS_FULL_MIN_BLOCKS)
          : std::is_same<S, float>::value ? KSS_F32_MIN_BLOCKS
          : (std::is_same<S, __half>::value && MODE == MODE_STD) ? KSS_F16_MIN_BLOCKS
                                                                 : KSS_STEP_MIN_BLOCKS;
@@ -239,6 +243,7 @@ struct StepParams {
   T zero;                // 0, read at run time (see product2): every builder value-initialises
   int slab;              // 0: periodic in y; 1: a y-slab of a decomposed lattice, whose rows
                          // -1 and ny are halo rows held next to its own (kss_slab_create)
+  uint32_t need;         // all-sensor steps: the sensors recorded or tagged (cell_update)
   int rec_slot[S_COUNT];  // plane index of each recorded sensor, -1 if not recorded
   codec_t<S> codec;      // FP16 deviation codec (empty for float / double storage)
   uint8_t* region;       // two-relaxation region [ny][pitch], a byte per cell (AAR steps):
@@ -1215,51 +1220,8 @@ __device__ __forceinline__ uint32_t fused_row(const StepParams<S>& p,
   constexpr bool OUT = MODE != MODE_PLAIN;
   const long long off = (long long)j * p.pitch + i0;
   uint32_t fbits = 0;
-  if constexpr (MODE == MODE_FULL) {
-    // ---- all sensors of Table 1: cell-major, generic per-cell arithmetic ----
-    T fo[9][V];
-#pragma unroll
-    for (int k = 0; k < V; ++k) {
-      T c[9], o9[9];
-#pragma unroll
-      for (int q = 0; q < 9; ++q) c[q] = ft[q][k];
-      CellOut<T> co;
-      cell_update<T, MODE, STORE, AAR>(c, p.omega, p.tau, o9, co, p.trt,
-                                       ((mbits >> (8 * k)) & 0xffu) != 0u);
-      const bool valid = cv && (i0 + k < p.nx);
-      if (STORE) {
-#pragma unroll
-        for (int q = 0; q < 9; ++q) fo[q][k] = o9[q];
-      }
-      if (valid) {
-        a_rho.add(co.rho);
-        a_jx.add(co.jx);
-        a_jy.add(co.jy);
-      }
-      const bool r = valid && (pick<T>(co.sv, p.refine_s) > p.thr_r);
-      const bool sw = valid && p.switch_on && (pick<T>(co.sv, p.switch_s) > p.thr_s);
-      const bool np = valid && co.nonpos;
-      fbits |= (uint32_t(r) | (uint32_t(sw) << 1) | (uint32_t(np) << 7)) << (8 * k);
-      // recorded sensors: one value per cell as soon as it is known (the lanes of a warp
-      // still cover contiguous bytes), so no sensor values stay live across the cells
-      if (valid) {
-#pragma unroll
-        for (int sid = 0; sid < S_COUNT; ++sid) {
-          const int slot = p.rec_slot[sid];
-          if (slot >= 0) p.rec[slot * p.plane + off + k] = co.sv[sid];
-        }
-      }
-    }
-    if (STORE && cv) {
-#pragma unroll
-      for (int q = 0; q < 9; ++q) pop_vstore<S>(p.dst + q * p.plane + off, fo[q], q, p.codec);
-    }
-    if (cv) {
-      store_flags<V>(p.flags + off, fbits);
-      if (AAR && STORE && p.region) store_flags<V>(p.region + off, (fbits >> 1) & 0x01010101u);
-    }
-  } else if constexpr (KSS_ROW_PAIRED && std::is_same<T, float>::value && V == 4 &&
-                       !(AAR && MULTI)) {
+  static_assert(MODE != MODE_FULL, "all-sensor rows: full_row");
+  if constexpr (KSS_ROW_PAIRED && std::is_same<T, float>::value && V == 4 && !(AAR && MULTI)) {
     // ---- the same row in paired instructions (fused_row_paired) ----
     F2 f[9][2];
 #pragma unroll
@@ -1681,6 +1643,100 @@ __device__ __forceinline__ void pull_row(const StepParams<S>& p, int j, int i0, 
   assemble_from_right<T>(ft[7], h7, i0, p.nx, lane);
 }
 
+// ---------------------------------------------------------------- all sensors ----
+// One row of an all-sensor step: the warp's 32 V columns as V passes of one cell per lane,
+// with the generic per-cell arithmetic (cell_update).  One cell per lane keeps one copy of
+// that arithmetic (18 logarithms, about 1250 instructions) in the loop: with V cells
+// unrolled it overflowed the instruction cache (1.5 to 3 of the 5.8 to 8 stall cycles per
+// issue) and held 128 registers at 21 % occupancy.  Its loads and stores are 32 consecutive
+// elements per warp, recorded sensors included.  2048^2 FP32: all of Table 1 recorded
+// 246 -> 179 us per step, the strain sensor alone 99 -> 80 us (its bytes: 48 us).
+//
+// The flags and moments of a pass go through the warp's row in shared memory, so that lane
+// L then holds cells V L .. V L + V - 1 as in the other rows: the same flag word, and sums
+// added in the same order.
+template <class S>
+struct FullRow {
+  static constexpr int kCells = 32 * Vec<S>::N;
+  arith_t<S> m[3][kCells];  // rho, jx, jy
+  uint8_t flags[kCells];
+};
+
+template <class S, bool PULL, bool STORE, bool AAR, bool CG>
+__device__ __forceinline__ uint32_t full_row(const StepParams<S>& p, FullRow<S>& row, int c0,
+                                             int j, int lane, Acc<arith_t<S>>& a_rho,
+                                             Acc<arith_t<S>>& a_jx, Acc<arith_t<S>>& a_jy) {
+  using T = arith_t<S>;
+  constexpr int V = Vec<S>::N;
+  constexpr int cx[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
+  constexpr int cy[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+  long long up, dn;  // rows j - 1 and j + 1
+  row_neighbours(p, j, up, dn);
+  const S* const src = p.src + (long long)j * p.pitch;
+#pragma unroll 1
+  for (int c = 0; c < V; ++c) {
+    const int t = 32 * c + lane, i = c0 + t;
+    const bool ok = i < p.nx;
+    T f[9], fo[9];
+    uint32_t switched = 0;
+    if (ok) {
+      const int l = i == 0 ? p.nx - 1 : i - 1, r = i + 1 == p.nx ? 0 : i + 1;
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        const int col = !PULL || cx[q] == 0 ? i : (cx[q] > 0 ? l : r);
+        const long long off = !PULL || cy[q] == 0 ? 0 : (cy[q] > 0 ? up : dn);
+        f[q] = decode<S>(ld_pop<CG>(src + q * p.plane + off + col), q, p.codec);
+      }
+      // (in a batch, a member without the model has no region: it steps as BGK)
+      if (AAR && STORE && p.region) switched = p.region[(long long)j * p.pitch + i];
+    } else {
+#pragma unroll
+      for (int q = 0; q < 9; ++q) f[q] = T(1);  // finite; nothing of it is stored or added
+    }
+    CellOut<T> co;
+    cell_update<T, MODE_FULL, STORE, AAR>(f, p.omega, p.tau, fo, co, p.trt, switched != 0u,
+                                          p.need);
+    const long long off = (long long)j * p.pitch + i;
+    if (ok) {
+      if (STORE) {
+#pragma unroll
+        for (int q = 0; q < 9; ++q)
+          __stcs(p.dst + q * p.plane + off, encode<S>(fo[q], q, p.codec));
+      }
+#pragma unroll
+      for (int sid = 0; sid < S_COUNT; ++sid) {
+        const int slot = p.rec_slot[sid];
+        if (slot >= 0) p.rec[slot * p.plane + off] = co.sv[sid];
+      }
+    }
+    const bool rf = ok && (pick<T>(co.sv, p.refine_s) > p.thr_r);
+    const bool sw = ok && p.switch_on && (pick<T>(co.sv, p.switch_s) > p.thr_s);
+    row.flags[t] = uint8_t(uint32_t(rf) | (uint32_t(sw) << 1) | (uint32_t(ok && co.nonpos) << 7));
+    row.m[0][t] = co.rho;
+    row.m[1][t] = co.jx;
+    row.m[2][t] = co.jy;
+  }
+  __syncwarp();
+  uint32_t fbits = 0;
+#pragma unroll
+  for (int k = 0; k < V; ++k) {
+    const int t = lane * V + k;
+    fbits |= uint32_t(row.flags[t]) << (8 * k);
+    if (c0 + t < p.nx) {
+      a_rho.add(row.m[0][t]);
+      a_jx.add(row.m[1][t]);
+      a_jy.add(row.m[2][t]);
+    }
+  }
+  __syncwarp();  // the row is rewritten by the warp's next row
+  if (c0 + lane * V < p.nx) {
+    const long long off = (long long)j * p.pitch + c0 + lane * V;
+    store_flags<V>(p.flags + off, fbits);
+    if (AAR && STORE && p.region) store_flags<V>(p.region + off, (fbits >> 1) & 0x01010101u);
+  }
+  return fbits;
+}
+
 // ---------------------------------------------------------------- the fused step ----
 // MODE:  MODE_PLAIN (stream + collide only), MODE_STD / MODE_FULL (plus sensors,
 //        flags, tile counts, sums).
@@ -1725,6 +1781,9 @@ __device__ __forceinline__ void step_block(const StepParams<S>& p, const int bx,
   __shared__ uint32_t s_cx[3];                   // their tags (refine, switch, nonpos)
   __shared__ Red<T> s_sum[NW][3];
   __shared__ uint32_t s_cnt[NW][3];
+  struct NoRow {};
+  __shared__ typename std::conditional<MODE == MODE_FULL, FullRow<S>, NoRow>::type
+      s_row[MODE == MODE_FULL ? NW : 1];
   if (OUT) {
     for (int t = threadIdx.x; t < 2 * kMaxBands * 32; t += NT) (&s_tiles[0][0][0])[t] = 0;
     if (threadIdx.x < 3) s_cx[threadIdx.x] = 0;
@@ -1832,6 +1891,9 @@ __device__ __forceinline__ void step_block(const StepParams<S>& p, const int bx,
       }
       assemble_half_row(p, i0, lane, w, h, f);
       fbits = fused_row_paired<S, MODE, STORE>(p, f, i0, j, cv, a_rho, a_jx, a_jy);
+    } else if constexpr (MODE == MODE_FULL) {
+      fbits = full_row<S, PULL, STORE, AAR, CG>(p, s_row[warp], bx * 32 * V, j, lane, a_rho,
+                                                a_jx, a_jy);
     } else {
     T ft[9][V];
     const S* base = p.src + (long long)j * p.pitch;
@@ -2242,7 +2304,7 @@ struct BatchItem {
 // AAR: members with a region take the two-relaxation collision there (members without
 // one step as BGK).
 template <class S, int MODE, bool AAR = false>
-__global__ void __launch_bounds__(kThreads, step_min_blocks<S, MODE>())
+__global__ void __launch_bounds__(kThreads, MODE == MODE_FULL ? 2 : step_min_blocks<S, MODE>())
 batch_step_kernel(const StepParams<S>* __restrict__ table, const BatchItem* __restrict__ items,
                   int nitems) {
   static_assert(sizeof(StepParams<S>) % 8 == 0, "parameter copy in 8-byte words");
