@@ -325,6 +325,14 @@ int steps_graph(kss_lattice* L, int nsteps) {
   return KSS_OK;
 }
 
+// Do this lattice's output steps share each block out to several CTAs?  (Then a run of them
+// is a graph of one-step launches, not one multi-step launch.)
+bool splits(const kss_lattice* L) {
+  return with_storage(L->cfg.precision, [&](auto tag) {
+    return kss::split_ranks<typename decltype(tag)::type>(L->nblocks, L->cfg.tile * L->bands) > 0;
+  });
+}
+
 int ensure_staging(kss_lattice* L, size_t elems) {
   if (L->staging_elems >= elems) return KSS_OK;
   if (L->staging) {
@@ -799,7 +807,7 @@ int kss_step(kss_lattice* L, int32_t nsteps) {
       every == 1 ? mode_for(needed_mask(L, L->cfg.record_mask), L->region != nullptr) : MODE_PLAIN;
   if (KSS_MULTISTEP && nsteps >= 2 && every == 1 && mode == MODE_STD &&
       (KSS_MULTISTEP_F16 || L->cfg.precision != KSS_FP16DEV) &&
-      (L->region || !use_tma(L, mode)) &&
+      (L->region || !use_tma(L, mode)) && !splits(L) &&
       (long long)nsteps * L->nblocks < (1LL << 30)) {
     KSS_CUDA(L, with_storage(L->cfg.precision, [&](auto tag) {
                return launch_multi<typename decltype(tag)::type>(L, mode, nsteps);

@@ -39,6 +39,17 @@ template <class T>
 cudaError_t launch_step(const StepParams<T>& p, int mode, bool pull, bool store,
                         cudaStream_t stream);
 
+// CTAs (ranks) that share each block of an output step or evaluation pass of `nblocks`
+// blocks of `rows` rows (step_kernel_split), or 0 where a block is one CTA's.  Blocks are
+// shared where the ranks, at one row per warp of eight, all fit on the GPU at once (two CTAs
+// of 256 threads per SM).  {Kn, KL, neq} steps, unsplit / split: FP32 256^2 (16 blocks)
+// 15.4 / 10.1 us, 512^2 (64) 17.5 / 12.0, 1021x517 (136) 17.1 / 18.9, 1024^2 (256)
+// 21.7 / 32.8; FP64 128^2 (8) 243 / 56, 512x256 (64) 227 / 150, 512^2 (128) 229 / 259; FP16
+// 512^2 (32 blocks of 256 columns) 21.0 / 12.9, 1021x517 (68) 20.3 / 15.3, 1024^2 (128)
+// 19.9 / 26.4.  All of Table 1, FP32: 256^2 44.7 / 18.0, 512^2 44.1 / 25.2.
+template <class T>
+int split_ranks(long long nblocks, int rows);
+
 // One step with adaptive algorithm refinement: the two-relaxation collision in the
 // region p.region (output steps rewrite it); mode as launch_step, always pull + store.
 template <class T>

@@ -2,6 +2,7 @@
 // storage precision by launch_f32.cu / launch_f64.cu with KSS_T defined.
 #pragma once
 
+#include <algorithm>
 #include <atomic>
 
 #include "launch.h"
@@ -43,6 +44,24 @@ cudaError_t allow_dynamic_smem() {
   }
 }
 
+// Let `kernel` run in clusters of more than eight CTAs on the current device, once per
+// device (as above).
+template <auto kernel>
+cudaError_t allow_large_clusters() {
+  constexpr int kMaxDev = 64;
+  static std::atomic<bool> done[kMaxDev] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxDev) return cudaErrorInvalidDevice;
+  if (!done[dev].load(std::memory_order_acquire)) {
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    done[dev].store(true, std::memory_order_release);
+  }
+  return cudaSuccess;
+}
+
 // CTAs of `kernel` (with DYN bytes of dynamic shared memory) resident on the current
 // device at once (its occupancy times the SM count), looked up once per device (racing
 // threads at most repeat the query).
@@ -79,9 +98,71 @@ int resident_ctas() {
 #define KSS_F16_CELLS8 1
 #endif
 
+// SMs of the current device, looked up once per device (0 on error).
+inline int sm_count() {
+  constexpr int kMaxDev = 64;
+  static std::atomic<int> cache[kMaxDev] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) return 0;
+  int n = cache[dev].load(std::memory_order_acquire);
+  if (!n) {
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    cache[dev].store(n, std::memory_order_release);
+  }
+  return n;
+}
+
+template <>
+int split_ranks<KSS_T>(long long nblocks, int rows) {
+  if (nblocks * (rows / kWarps) > 2LL * sm_count()) return 0;
+  const int ranks = std::min(rows / split_warps<KSS_T>(), 16);
+  return ranks >= 2 && ranks * split_warps<KSS_T>() * kSplitRows >= rows ? ranks : 0;
+}
+
+// One split step: a cluster of `ranks` CTAs per block of `grid` (the clusters of more than
+// eight CTAs of FP64 steps need an opt-in, once per device).
+template <int MODE, bool PULL, bool STORE, bool AAR, int VC>
+cudaError_t launch_split(const StepParams<KSS_T>& p, dim3 grid, int ranks, cudaStream_t stream) {
+  constexpr auto kern = step_kernel_split<KSS_T, MODE, PULL, STORE, AAR, VC>;
+  constexpr int dyn = VC == 8 ? split_warps<KSS_T>() * int(sizeof(PfWarpH8)) : 0;
+  cudaError_t e = allow_dynamic_smem<kern, dyn>();
+  if (e == cudaSuccess && ranks > 8) e = allow_large_clusters<kern>();
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid.x, grid.y, unsigned(ranks));
+  cfg.blockDim = dim3(32 * split_warps<KSS_T>());
+  cfg.dynamicSmemBytes = dyn;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 1;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = unsigned(ranks);
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, p);
+}
+
 template <int MODE>
 cudaError_t launch_step_mode(const StepParams<KSS_T>& p, dim3 grid, cudaStream_t stream) {
   const int nblocks = int(grid.x * grid.y);
+  if constexpr (MODE != MODE_PLAIN) {
+    const int rows = p.tile * p.bands;
+    if constexpr (std::is_same<KSS_T, __half>::value && MODE == MODE_STD && KSS_F16_CELLS8) {
+      // (the sums of an FP16 lattice's steps are those of its eight-cell blocks)
+      dim3 g8;
+      int bands8 = 0;
+      if (step_grid8(p.nx, p.ny, p.tile, p.bands, KSS_H8_WARPS, g8, bands8)) {
+        if (bands8 == p.bands)
+          if (const int ranks = split_ranks<KSS_T>((long long)g8.x * g8.y, rows))
+            return launch_split<MODE, true, true, false, 8>(p, g8, ranks, stream);
+      } else if (const int ranks = split_ranks<KSS_T>(nblocks, rows)) {
+        return launch_split<MODE, true, true, false, Vec<KSS_T>::N>(p, grid, ranks, stream);
+      }
+    } else if (const int ranks = split_ranks<KSS_T>(nblocks, rows)) {
+      return launch_split<MODE, true, true, false, Vec<KSS_T>::N>(p, grid, ranks, stream);
+    }
+  }
   constexpr bool kHalfPlain = std::is_same<KSS_T, __half>::value && MODE == MODE_PLAIN;
   if (KSS_PERSISTENT || kHalfPlain) {
     const int wave = resident_ctas<step_kernel_persistent<KSS_T, MODE, true, true>>();
@@ -144,6 +225,14 @@ cudaError_t launch_step<KSS_T>(const StepParams<KSS_T>& p, int mode, bool pull, 
       default: return cudaErrorInvalidValue;
     }
   } else if (!store) {
+    if (const int ranks = split_ranks<KSS_T>((long long)grid.x * grid.y, p.tile * p.bands)) {
+      constexpr int V = Vec<KSS_T>::N;
+      if (mode == MODE_STD)
+        return pull ? launch_split<MODE_STD, true, false, false, V>(p, grid, ranks, stream)
+                    : launch_split<MODE_STD, false, false, false, V>(p, grid, ranks, stream);
+      return pull ? launch_split<MODE_FULL, true, false, false, V>(p, grid, ranks, stream)
+                  : launch_split<MODE_FULL, false, false, false, V>(p, grid, ranks, stream);
+    }
     if (mode == MODE_STD && pull) step_kernel<KSS_T, MODE_STD, true, false><<<grid, block, 0, stream>>>(p);
     else if (mode == MODE_STD) step_kernel<KSS_T, MODE_STD, false, false><<<grid, block, 0, stream>>>(p);
     else if (mode == MODE_FULL && pull) step_kernel<KSS_T, MODE_FULL, true, false><<<grid, block, 0, stream>>>(p);
@@ -158,6 +247,13 @@ cudaError_t launch_step<KSS_T>(const StepParams<KSS_T>& p, int mode, bool pull, 
 template <>
 cudaError_t launch_step_aar<KSS_T>(const StepParams<KSS_T>& p, int mode, cudaStream_t stream) {
   const dim3 grid = step_grid<KSS_T>(p.nx, p.ny, p.tile, p.bands);
+  const int ranks =
+      mode == MODE_PLAIN ? 0 : split_ranks<KSS_T>((long long)grid.x * grid.y, p.tile * p.bands);
+  if (ranks) {
+    constexpr int V = Vec<KSS_T>::N;
+    return mode == MODE_STD ? launch_split<MODE_STD, true, true, true, V>(p, grid, ranks, stream)
+                            : launch_split<MODE_FULL, true, true, true, V>(p, grid, ranks, stream);
+  }
   switch (mode) {
     case MODE_PLAIN: step_kernel<KSS_T, MODE_PLAIN, true, true, true><<<grid, kThreads, 0, stream>>>(p); break;
     case MODE_STD: step_kernel<KSS_T, MODE_STD, true, true, true><<<grid, kThreads, 0, stream>>>(p); break;

@@ -760,37 +760,43 @@ template <> struct Red<double> {
 };
 
 // The last CTA's reduction of the per-CTA partials, in CTA order within each thread and
-// a fixed shuffle/shared-memory tree across threads (bitwise reproducible).
+// a fixed shuffle/shared-memory tree across threads (bitwise reproducible).  The tree of a
+// CTA of fewer than kThreads threads is that of kThreads: its warps take several shares.
 template <class S, int NTHREADS>
 __device__ __forceinline__ void finalize_sums(const double* part_sum, const uint32_t* part_cnt,
                                               int nblocks, double* out_sums,
                                               unsigned long long* out_counts) {
   using T = arith_t<S>;
-  __shared__ Red<T> f_sum[NTHREADS / 32][3];
-  __shared__ unsigned long long f_cnt[NTHREADS / 32][3];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  Red<T> t[3];
-  unsigned long long u[3] = {0, 0, 0};
-  for (int b = threadIdx.x; b < nblocks; b += NTHREADS) {
+  constexpr int kTree = NTHREADS > kThreads ? NTHREADS : kThreads, kShares = kTree / 32;
+  static_assert(kTree % NTHREADS == 0, "whole shares per warp");
+  __shared__ Red<T> f_sum[kShares][3];
+  __shared__ unsigned long long f_cnt[kShares][3];
+  const int lane = threadIdx.x & 31;
+#pragma unroll 1
+  for (int warp = threadIdx.x >> 5; warp < kShares; warp += NTHREADS / 32) {
+    Red<T> t[3];
+    unsigned long long u[3] = {0, 0, 0};
+    for (int b = 32 * warp + lane; b < nblocks; b += kTree) {
 #pragma unroll
-    for (int m = 0; m < 3; ++m) {
-      t[m].add(Red<T>::load(part_sum + 3 * b + m));
-      u[m] += __ldcg(part_cnt + 4 * b + m);
+      for (int m = 0; m < 3; ++m) {
+        t[m].add(Red<T>::load(part_sum + 3 * b + m));
+        u[m] += __ldcg(part_cnt + 4 * b + m);
+      }
     }
-  }
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
+    for (int off = 16; off > 0; off >>= 1) {
 #pragma unroll
-    for (int m = 0; m < 3; ++m) {
-      t[m].add(t[m].shfl_xor(off));
-      u[m] += __shfl_xor_sync(kFull, u[m], off);
+      for (int m = 0; m < 3; ++m) {
+        t[m].add(t[m].shfl_xor(off));
+        u[m] += __shfl_xor_sync(kFull, u[m], off);
+      }
     }
-  }
-  if (lane == 0) {
+    if (lane == 0) {
 #pragma unroll
-    for (int m = 0; m < 3; ++m) {
-      f_sum[warp][m] = t[m];
-      f_cnt[warp][m] = u[m];
+      for (int m = 0; m < 3; ++m) {
+        f_sum[warp][m] = t[m];
+        f_cnt[warp][m] = u[m];
+      }
     }
   }
   __syncthreads();
@@ -799,7 +805,7 @@ __device__ __forceinline__ void finalize_sums(const double* part_sum, const uint
     for (int m = 0; m < 3; ++m) {
       Red<T> r = f_sum[0][m];
       unsigned long long c = f_cnt[0][m];
-      for (int w = 1; w < NTHREADS / 32; ++w) {
+      for (int w = 1; w < kShares; ++w) {
         r.add(f_sum[w][m]);
         c += f_cnt[w][m];
       }
@@ -1664,8 +1670,7 @@ struct FullRow {
 
 template <class S, bool PULL, bool STORE, bool AAR, bool CG>
 __device__ __forceinline__ uint32_t full_row(const StepParams<S>& p, FullRow<S>& row, int c0,
-                                             int j, int lane, Acc<arith_t<S>>& a_rho,
-                                             Acc<arith_t<S>>& a_jx, Acc<arith_t<S>>& a_jy) {
+                                             int j, int lane) {
   using T = arith_t<S>;
   constexpr int V = Vec<S>::N;
   constexpr int cx[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
@@ -1719,9 +1724,23 @@ __device__ __forceinline__ uint32_t full_row(const StepParams<S>& p, FullRow<S>&
   __syncwarp();
   uint32_t fbits = 0;
 #pragma unroll
-  for (int k = 0; k < V; ++k) {
-    const int t = lane * V + k;
-    fbits |= uint32_t(row.flags[t]) << (8 * k);
+  for (int k = 0; k < V; ++k) fbits |= uint32_t(row.flags[lane * V + k]) << (8 * k);
+  if (c0 + lane * V < p.nx) {
+    const long long off = (long long)j * p.pitch + c0 + lane * V;
+    store_flags<V>(p.flags + off, fbits);
+    if (AAR && STORE && p.region) store_flags<V>(p.region + off, (fbits >> 1) & 0x01010101u);
+  }
+  return fbits;
+}
+
+// The lane's V cells of a row that full_row evaluated, added in order.
+template <class S>
+__device__ __forceinline__ void full_row_sums(const StepParams<S>& p, const FullRow<S>& row,
+                                              int c0, int lane, Acc<arith_t<S>>& a_rho,
+                                              Acc<arith_t<S>>& a_jx, Acc<arith_t<S>>& a_jy) {
+#pragma unroll
+  for (int k = 0; k < Vec<S>::N; ++k) {
+    const int t = lane * Vec<S>::N + k;
     if (c0 + t < p.nx) {
       a_rho.add(row.m[0][t]);
       a_jx.add(row.m[1][t]);
@@ -1729,12 +1748,6 @@ __device__ __forceinline__ uint32_t full_row(const StepParams<S>& p, FullRow<S>&
     }
   }
   __syncwarp();  // the row is rewritten by the warp's next row
-  if (c0 + lane * V < p.nx) {
-    const long long off = (long long)j * p.pitch + c0 + lane * V;
-    store_flags<V>(p.flags + off, fbits);
-    if (AAR && STORE && p.region) store_flags<V>(p.region + off, (fbits >> 1) & 0x01010101u);
-  }
-  return fbits;
 }
 
 // ---------------------------------------------------------------- the fused step ----
@@ -1892,8 +1905,8 @@ __device__ __forceinline__ void step_block(const StepParams<S>& p, const int bx,
       assemble_half_row(p, i0, lane, w, h, f);
       fbits = fused_row_paired<S, MODE, STORE>(p, f, i0, j, cv, a_rho, a_jx, a_jy);
     } else if constexpr (MODE == MODE_FULL) {
-      fbits = full_row<S, PULL, STORE, AAR, CG>(p, s_row[warp], bx * 32 * V, j, lane, a_rho,
-                                                a_jx, a_jy);
+      fbits = full_row<S, PULL, STORE, AAR, CG>(p, s_row[warp], bx * 32 * V, j, lane);
+      full_row_sums<S>(p, s_row[warp], bx * 32 * V, lane, a_rho, a_jx, a_jy);
     } else {
     T ft[9][V];
     const S* base = p.src + (long long)j * p.pitch;
@@ -2151,6 +2164,301 @@ step_kernel_persistent(const StepParams<S> p, int gx, int nblocks) {
     if (MODE != MODE_PLAIN) __syncthreads();  // shared memory is reused by the next block
   }
   if (MODE != MODE_PLAIN) ticket_and_finalize<S>(p, gridDim.x, nblocks);
+}
+
+// ---------------------------------------------------------------- split blocks ----
+// A block's rows shared out to the CTAs of a cluster, for lattices with too few blocks to
+// fill the GPU (split_ranks).  A warp of an unsplit block takes four or eight rows one after
+// the other; with 4 blocks (128^2) a step lasts as long as four rows, on 4 of 152 SMs.  Here
+// the cluster's CTAs (ranks) take NW rows each, one per warp, with the same row functions;
+// rank 0 then collects the block: tile counts and tags are added over the ranks, and the
+// moments, which every lane leaves in its CTA's shared memory as the values an unsplit block
+// would add to its accumulators, are added by rank 0 in that block's own order.  So the sums
+// are those of the unsplit block bit for bit.
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// *p of the CTA with this rank (p: an address in this CTA's shared memory).
+template <class T>
+__device__ __forceinline__ T ld_rank(const T* p, uint32_t rank) {
+  static_assert(sizeof(T) == 4 || sizeof(T) == 8, "one 4- or 8-byte load");
+  const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(p));
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  if constexpr (sizeof(T) == 4) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(r) : "memory");
+    return *reinterpret_cast<T*>(&v);
+  } else {
+    unsigned long long v;
+    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(r) : "memory");
+    return *reinterpret_cast<T*>(&v);
+  }
+}
+
+// Warps per rank: eight with FP32 arithmetic, where a row is bound by latency; two in FP64,
+// where a block is bound by the FP64 pipes of the SMs it runs on.
+template <class S>
+__host__ __device__ constexpr int split_warps() {
+  return std::is_same<S, double>::value ? 2 : kWarps;
+}
+constexpr int kSplitRows = 2;  // rows per warp of a rank, at most
+
+template <class T>
+__device__ __forceinline__ T acc_value(const Acc<T>& a) {
+  if constexpr (std::is_same<T, float>::value) {
+    return a.hi;
+  } else {
+    return a.v;
+  }
+}
+
+template <class S, int MODE, bool PULL, bool STORE, bool AAR, int VC>
+__global__ void __launch_bounds__(32 * split_warps<S>(), std::is_same<S, double>::value ? 4 : 2)
+step_kernel_split(const StepParams<S> p) {
+  using T = arith_t<S>;
+  constexpr int V = Vec<S>::N, NW = split_warps<S>(), NT = 32 * NW;
+  constexpr bool kH8 = VC == 8, FULL = MODE == MODE_FULL;
+  constexpr bool kHalfPaired = KSS_ROW_PAIRED && std::is_same<S, __half>::value && !FULL &&
+                               !AAR && PULL && V == 4;
+  static_assert(MODE != MODE_PLAIN && (VC == V || (kH8 && kHalfPaired && STORE)), "split steps");
+  constexpr int kVals = FULL ? 0 : (kH8 ? 2 : 1);  // accumulator additions per lane and row
+  constexpr int kSlots = kSplitRows * NW;          // rows of this rank
+  const int bx = blockIdx.x, by = blockIdx.y, gx = gridDim.x;
+  const uint32_t rank = cluster_rank(), ranks = cluster_size();
+  const int lane = threadIdx.x & 31, warp = __shfl_sync(kFull, int(threadIdx.x >> 5), 0);
+  const int rows = p.tile * p.bands, stride = int(ranks) * NW;
+  const int i0 = (bx * 32 + lane) * VC, c0 = bx * 32 * VC;
+  const bool cv = i0 < p.nx;
+  const int j0 = by * rows, j1 = min(j0 + rows, p.ny);
+  // (uniform over the cluster: every thread returns, before any barrier)
+  if (!bounds_ok(c0 < p.pitch && j0 < p.ny && p.bands >= 1 && p.bands <= kMaxBands &&
+                     rows <= 64 && rows <= stride * kSplitRows,
+                 p.err))
+    return;
+
+  __shared__ int s_tiles[2][kMaxBands][32];
+  __shared__ uint32_t s_cx[3];                        // tags (refine, switch, nonpos)
+  __shared__ uint16_t s_dl[NW][kSplitRows * 32 * VC];  // each warp's deferred cells
+  __shared__ uint32_t s_wn[NW];
+  __shared__ T s_val[FULL ? 1 : kSlots][3][kVals ? kVals : 1][32];
+  __shared__ FullRow<S> s_row[FULL ? kSlots : 1];
+  __shared__ Red<T> s_sum[kWarps][3];
+  extern __shared__ __align__(16) unsigned char kss_dyn_smem[];
+  for (int t = threadIdx.x; t < 2 * kMaxBands * 32; t += NT) (&s_tiles[0][0][0])[t] = 0;
+  if (threadIdx.x < 3) s_cx[threadIdx.x] = 0;
+  __syncthreads();
+
+  const int tshift = __ffs(p.tile) - 1;
+  const int lshift = tshift - (VC == 8 ? 3 : VC == 4 ? 2 : 1);
+  const int lpt = 1 << lshift;
+  uint32_t n_ref = 0, n_sw = 0, n_np = 0, wn = 0;
+#pragma unroll 1
+  for (int s = 0, rl = int(rank) * NW + warp; j0 + rl < j1; ++s, rl += stride) {
+    const int j = j0 + rl, slot = s * NW + warp;
+    uint32_t fbits, fbits2 = 0;
+    Acc<T> a[3], b[3];
+    if constexpr (FULL) {
+      fbits = full_row<S, PULL, STORE, AAR, false>(p, s_row[slot], c0, j, lane);
+    } else if constexpr (kH8) {
+      PfWarpH8* const pw = reinterpret_cast<PfWarpH8*>(kss_dyn_smem) + warp;
+      const bool tail = cv && i0 + 8 >= p.nx;
+      uint4 w[9];
+      F2 f[9][2];
+      __syncwarp();
+      pf_issue_h8(p, pw, j, i0, lane, cv, tail);
+      cp_async_wait_all();
+      __syncwarp();
+      pf_read_h8(pw, lane, (i0 == 0 && (p.nx & 1)) ? 0x5410u : 0x5432u,
+                 tail ? p.nx - 1 - i0 : 8, w);
+      decode_h8(p, w, false, f);
+      fbits = fused_row_paired<S, MODE, STORE>(p, f, i0, j, cv, a[0], a[1], a[2]);
+      decode_h8(p, w, true, f);
+      fbits2 = fused_row_paired<S, MODE, STORE>(p, f, i0 + 4, j, i0 + 4 < p.nx, b[0], b[1], b[2]);
+    } else if constexpr (kHalfPaired) {
+      F2 f[9][2];
+      uint2 w[9];
+      uint32_t h[9];
+      gather_half_row<false>(p, j, i0, lane, cv, w, h);
+      assemble_half_row(p, i0, lane, w, h, f);
+      fbits = fused_row_paired<S, MODE, STORE>(p, f, i0, j, cv, a[0], a[1], a[2]);
+    } else {
+      T ft[9][V];
+      uint32_t mbits = 0;
+      if constexpr (AAR && STORE) {
+        if (cv && p.region) mbits = load_bytes<V>(p.region + (long long)j * p.pitch + i0);
+      }
+      if constexpr (PULL) {
+        pull_row<S, false>(p, j, i0, lane, cv, ft);
+      } else {
+#pragma unroll
+        for (int q = 0; q < 9; ++q)
+          pop_vload<S, V, false>(p.src + (long long)j * p.pitch + q * p.plane + i0, cv, ft[q], q,
+                                 p.codec);
+      }
+      fbits = fused_row<S, MODE, PULL, STORE, AAR, false>(p, ft, i0, j, cv, a[0], a[1], a[2], mbits);
+    }
+    if constexpr (!FULL) {
+#pragma unroll
+      for (int m = 0; m < 3; ++m) {
+        s_val[slot][m][0][lane] = acc_value(a[m]);
+        if (kH8) s_val[slot][m][kVals - 1][lane] = acc_value(b[m]);
+      }
+    }
+    // tags of the lane's cells, which all lie in tile lane >> lshift of the row's band
+    int tr = __popc(fbits & 0x01010101u) + __popc(fbits2 & 0x01010101u);
+    int ts = __popc(fbits & 0x02020202u) + __popc(fbits2 & 0x02020202u);
+    n_ref += tr;
+    n_sw += ts;
+    n_np += __popc(fbits & 0x80808080u) + __popc(fbits2 & 0x80808080u);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      if (o < lpt) {
+        tr += __shfl_xor_sync(kFull, tr, o);
+        ts += __shfl_xor_sync(kFull, ts, o);
+      }
+    }
+    if ((lane & (lpt - 1)) == 0 && (tr | ts)) {
+      atomicAdd(&s_tiles[0][rl >> tshift][lane >> lshift], tr);
+      atomicAdd(&s_tiles[1][rl >> tshift][lane >> lshift], ts);
+    }
+    if constexpr (MODE == MODE_STD) {
+      // deferred cells (see step_block), as offsets in the block
+      const uint32_t dbits = fbits & 0x40404040u, dbits2 = fbits2 & 0x40404040u;
+      if (__any_sync(kFull, (dbits | dbits2) != 0)) {
+        const int nd = __popc(dbits) + __popc(dbits2);
+        int incl = nd;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int v = __shfl_up_sync(kFull, incl, o);
+          if (lane >= o) incl += v;
+        }
+        uint32_t at = wn + uint32_t(incl - nd);
+#pragma unroll
+        for (int k = 0; k < VC; ++k) {
+          if (((k < 4 ? dbits : dbits2) >> (8 * (k & 3))) & 0x40u) {
+            if (bounds_ok(at < uint32_t(kSplitRows * 32 * VC), p.err))
+              s_dl[warp][at] = uint16_t(rl * 32 * VC + lane * VC + k);
+            ++at;
+          }
+        }
+        wn += uint32_t(__shfl_sync(kFull, incl, 31));
+      }
+    }
+  }
+  n_ref = __reduce_add_sync(kFull, n_ref);
+  n_sw = __reduce_add_sync(kFull, n_sw);
+  n_np = __reduce_add_sync(kFull, n_np);
+  if (lane == 0) {
+    if (n_ref) atomicAdd(&s_cx[0], n_ref);
+    if (n_sw) atomicAdd(&s_cx[1], n_sw);
+    if (n_np) atomicAdd(&s_cx[2], n_np);
+    s_wn[warp] = wn;
+  }
+  if constexpr (MODE == MODE_STD) {
+    // this rank's deferred cells: exact recomputation (see step_block)
+    __syncthreads();
+    uint32_t total = 0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) total += s_wn[w];
+    if (total) {
+      const Pick3 pr(p.refine_s), ps(p.switch_s);
+      for (uint32_t e = threadIdx.x; e < total; e += NT) {
+        uint32_t w = 0, r = e;
+        while (r >= s_wn[w]) r -= s_wn[w++];
+        const int o = s_dl[w][r];
+        const int rl = o / (32 * VC), cl = o - rl * (32 * VC);
+        const int j = j0 + rl, i = c0 + cl;
+        if (!bounds_ok(j < j1 && i < p.nx && rl / p.tile < kMaxBands && cl / p.tile < 32, p.err))
+          continue;
+        const uint32_t tags = fix_cell<S, PULL, false>(p, pr, ps, i, j);
+        if (AAR && STORE && p.region) p.region[(long long)j * p.pitch + i] = uint8_t((tags >> 1) & 1u);
+        const int bd = rl / p.tile, tl = cl / p.tile;
+        if (tags & 1u) {
+          atomicAdd(&s_cx[0], 1u);
+          atomicAdd(&s_tiles[0][bd][tl], 1);
+        }
+        if (tags & 2u) {
+          atomicAdd(&s_cx[1], 1u);
+          atomicAdd(&s_tiles[1][bd][tl], 1);
+        }
+        if (tags & 4u) atomicAdd(&s_cx[2], 1u);
+      }
+    }
+  }
+  __syncwarp();
+  cluster_arrive();  // the ranks' rows, counts and moments are in shared memory
+  cluster_wait();
+  const int bid = by * gx + bx;
+  if (rank == 0) {
+    // the moments in the order of the unsplit block: its warp w adds rows w, w + 8, ...
+#pragma unroll 1
+    for (int w = warp; w < kWarps; w += NW) {
+      Acc<T> a[3];
+      for (int rl = w; rl < rows && j0 + rl < j1; rl += kWarps) {
+        const int at = rl % stride, slot = (rl / stride) * NW + at % NW;
+        const uint32_t from = uint32_t(at / NW);
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          if constexpr (FULL) {
+#pragma unroll
+            for (int k = 0; k < V; ++k) {
+              const int t = lane * V + k;
+              const T v = ld_rank(&s_row[slot].m[m][t], from);
+              if (c0 + t < p.nx) a[m].add(v);
+            }
+          } else {
+#pragma unroll
+            for (int c = 0; c < kVals; ++c) a[m].add(ld_rank(&s_val[slot][m][c][lane], from));
+          }
+        }
+      }
+#pragma unroll
+      for (int m = 0; m < 3; ++m) {
+        a[m].warp_reduce();
+        if (lane == 0) s_sum[w][m] = Red<T>::of(a[m]);
+      }
+    }
+    const int tpb = (32 * VC) / p.tile;
+    for (int t = threadIdx.x; t < 2 * tpb * p.bands; t += NT) {
+      const int set = t / (tpb * p.bands), u = t - set * (tpb * p.bands);
+      const int b = u / tpb, tl = u - b * tpb;
+      const int tx = bx * tpb + tl, ty = by * p.bands + b;
+      if (tx < p.ntx && ty < p.nty) {
+        int n = 0;
+        for (uint32_t r = 0; r < ranks; ++r) n += ld_rank(&s_tiles[set][b][tl], r);
+        p.tiles[(long long)set * p.ntx * p.nty + (long long)ty * p.ntx + tx] = n;
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x < 3) {
+      const int m = threadIdx.x;
+      Red<T> sum;
+      uint32_t c = 0;
+      for (int w = 0; w < kWarps; ++w) sum.add(s_sum[w][m]);
+      for (uint32_t r = 0; r < ranks; ++r) c += ld_rank(&s_cx[m], r);
+      sum.store(p.part_sum + 3 * bid + m);
+      p.part_cnt[4 * bid + m] = c;
+    }
+  }
+  __syncwarp();
+  cluster_arrive();  // rank 0 has read the other ranks' shared memory
+  cluster_wait();
+  // (threads 0-2 of rank 0 wrote the block's partials before the barrier above)
+  if (rank == 0) ticket_and_finalize<S, NT>(p, gx * int(gridDim.y), gx * int(gridDim.y));
 }
 
 // ---------------------------------------------------------------- multi-step ----
