@@ -10,6 +10,8 @@
 #include <cuda_runtime.h>
 #include <math_constants.h>
 
+#include "exact64.cuh"
+
 namespace kss {
 
 // Sensor ids (same numbering as kss_sensor in include/kss.h).
@@ -51,7 +53,7 @@ template <> struct Num<double> {
   // first dropped term x^16/240 is below 2^-53 of x^2/2 for |x| < 1/16
   static constexpr int kPhiOrder = 15;
   static constexpr int kPhiFastOrder = 15;
-  __device__ static __forceinline__ double rcp(double x) { return 1.0 / x; }
+  __device__ static __forceinline__ double rcp(double x) { return rcp64(x); }
   __device__ static __forceinline__ double log1p_(double x) { return log1p(x); }
   __device__ static __forceinline__ double sqrt_(double x) { return sqrt(x); }
   __device__ static __forceinline__ double inf() { return CUDART_INF; }

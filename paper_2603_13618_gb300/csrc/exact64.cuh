@@ -47,6 +47,32 @@ __device__ __forceinline__ double reciprocal46(uint64_t frac) {
   return __longlong_as_double((y & ((1ll << 52) - 1)) | (1022ll << 52));
 }
 
+// 1 / x rounded: reciprocal46 and one FP64 Newton step, which leaves 2^-86 before its
+// rounding (two operations of the FP64 pipe; the compiler's division takes about ten).
+// Exponents near the ends of the range, zero, infinities and NaN take the division.
+__device__ __forceinline__ double rcp64(double x) {
+  const uint32_t hi = uint32_t(__double2hiint(x)), e = (hi >> 20) & 0x7ffu;
+  if (e - 3u > 2040u) return 1.0 / x;
+  const uint64_t b = uint64_t(__double_as_longlong(x));
+  const double m = __longlong_as_double((long long)((b & ((1ull << 52) - 1)) | (1023ull << 52)));
+  const double y0 = reciprocal46(b & ((1ull << 52) - 1));
+  const double y = fma(fma(-m, y0, 1.0), y0, y0);
+  // times 2^(1023 - e), exact; the sign of x
+  return __hiloint2double(int((uint32_t(__double2hiint(y)) + ((1023u - e) << 20)) |
+                              (hi & 0x80000000u)),
+                          __double2loint(y));
+}
+
+// n / d rounded, for d positive and of ordinary size (2^-1000 < d < 2^1000; other d give
+// some number or NaN): three operations of the FP64 pipe.
+__device__ __forceinline__ double ratio64(double n, double d) {
+  const uint64_t b = uint64_t(__double_as_longlong(d));
+  const double y = reciprocal46(b & ((1ull << 52) - 1));
+  const uint32_t e = uint32_t(b >> 52) & 0x7ffu;
+  return quotient(n, d, __hiloint2double(int(uint32_t(__double2hiint(y)) + ((1023u - e) << 20)),
+                                         __double2loint(y)));
+}
+
 // rho = sum v, ux = jx / rho and uy = jy / rho of nine FP32 populations as FP64 arithmetic
 // gives them.  Where the populations are positive and their exponents span at most 25, the
 // moments are integers below 2^53 in units of the smallest population's last place: every

@@ -115,8 +115,8 @@ inline int sm_count() {
 template <>
 int split_ranks<KSS_T>(long long nblocks, int rows) {
   if (nblocks * (rows / kWarps) > 2LL * sm_count()) return 0;
-  const int ranks = std::min(rows / split_warps<KSS_T>(), 16);
-  return ranks >= 2 && ranks * split_warps<KSS_T>() * kSplitRows >= rows ? ranks : 0;
+  const int ranks = std::min(rows / split_rows<KSS_T>(), 16);
+  return ranks >= 2 && ranks * split_rows<KSS_T>() * kSplitTurns >= rows ? ranks : 0;
 }
 
 // One split step: a cluster of `ranks` CTAs per block of `grid` (the clusters of more than
@@ -124,8 +124,8 @@ int split_ranks<KSS_T>(long long nblocks, int rows) {
 template <int MODE, bool PULL, bool STORE, bool AAR, int VC>
 cudaError_t launch_split(const StepParams<KSS_T>& p, dim3 grid, int ranks, cudaStream_t stream) {
   constexpr auto kern = step_kernel_split<KSS_T, MODE, PULL, STORE, AAR, VC>;
-  constexpr int dyn = VC == 8 ? split_warps<KSS_T>() * int(sizeof(PfWarpH8)) : 0;
-  cudaError_t e = allow_dynamic_smem<kern, dyn>();
+  const int dyn = split_smem<KSS_T, MODE, VC>(p.tile * p.bands);
+  cudaError_t e = allow_dynamic_smem<kern, split_smem<KSS_T, MODE, VC>(64)>();  // any height
   if (e == cudaSuccess && ranks > 8) e = allow_large_clusters<kern>();
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
@@ -143,9 +143,26 @@ cudaError_t launch_split(const StepParams<KSS_T>& p, dim3 grid, int ranks, cudaS
   return cudaLaunchKernelEx(&cfg, kern, p);
 }
 
+// A plain FP64 step of a lattice whose 8-row CTAs leave SMs idle (step_plain_f64_kernel:
+// 128^2 13.0 -> 5.1 us); true if launched.
+template <bool AAR>
+bool launch_plain_f64(const StepParams<KSS_T>& p, dim3 grid, cudaStream_t stream) {
+  if constexpr (std::is_same<KSS_T, double>::value) {
+    if (p.tile * p.bands != 8 || (long long)grid.x * grid.y >= sm_count()) return false;
+    const dim3 g((p.nx + 63) / 64, (p.ny + 1) / 2);
+    if (g.y > 65535) return false;
+    step_plain_f64_kernel<AAR><<<g, 128, 0, stream>>>(p);
+    return true;
+  }
+  return false;
+}
+
 template <int MODE>
 cudaError_t launch_step_mode(const StepParams<KSS_T>& p, dim3 grid, cudaStream_t stream) {
   const int nblocks = int(grid.x * grid.y);
+  if constexpr (MODE == MODE_PLAIN) {
+    if (launch_plain_f64<false>(p, grid, stream)) return cudaGetLastError();
+  }
   if constexpr (MODE != MODE_PLAIN) {
     const int rows = p.tile * p.bands;
     if constexpr (std::is_same<KSS_T, __half>::value && MODE == MODE_STD && KSS_F16_CELLS8) {
@@ -254,6 +271,7 @@ cudaError_t launch_step_aar<KSS_T>(const StepParams<KSS_T>& p, int mode, cudaStr
     return mode == MODE_STD ? launch_split<MODE_STD, true, true, true, V>(p, grid, ranks, stream)
                             : launch_split<MODE_FULL, true, true, true, V>(p, grid, ranks, stream);
   }
+  if (mode == MODE_PLAIN && launch_plain_f64<true>(p, grid, stream)) return cudaGetLastError();
   switch (mode) {
     case MODE_PLAIN: step_kernel<KSS_T, MODE_PLAIN, true, true, true><<<grid, kThreads, 0, stream>>>(p); break;
     case MODE_STD: step_kernel<KSS_T, MODE_STD, true, true, true><<<grid, kThreads, 0, stream>>>(p); break;

@@ -50,8 +50,9 @@ namespace kss {
 //                        launches take 0.2029 ms per step against 0.2241 ms at three CTAs
 //                        (80 registers, spilling), one-step launches 0.838 against 0.725 of
 //                        the measured bandwidth.
-//   KSS_STEP_MIN_BLOCKS  FP64 and FP16-deviation plain steps, FP64 {Kn, KL, neq} steps: three
-//                        CTAs (80 registers).
+//   KSS_STEP_MIN_BLOCKS  FP64 and FP16-deviation plain steps: three CTAs (80 registers).
+//   KSS_F64_MIN_BLOCKS   FP64 {Kn, KL, neq} steps, which keep all nine ratios of a row: two
+//                        (2048^2: 1.88 / 1.75 / 1.81 ms at one / two / three).
 //   KSS_F16_MIN_BLOCKS   FP16-deviation {Kn, KL, neq} steps: three (0.659 ms per 8192^2 step
 //                        against 0.706 ms at two: its 8-byte rows need more warps in flight).
 //   KSS_FULL_MIN_BLOCKS  the all-sensor steps with FP32 arithmetic: four CTAs at 64 registers
@@ -68,6 +69,9 @@ namespace kss {
 #endif
 #ifndef KSS_FULL_MIN_BLOCKS
 #define KSS_FULL_MIN_BLOCKS 4
+#endif
+#ifndef KSS_F64_MIN_BLOCKS
+#define KSS_F64_MIN_BLOCKS 2
 #endif
 #ifndef KSS_F16_MIN_BLOCKS
 #define KSS_F16_MIN_BLOCKS KSS_STEP_MIN_BLOCKS
@@ -87,6 +91,7 @@ template <class S, int MODE>
 __host__ __device__ constexpr int step_min_blocks() {
   return MODE == MODE_FULL ? (std::is_same<S, double>::value ? 2 : KSS_FULL_MIN_BLOCKS)
          : std::is_same<S, float>::value ? KSS_F32_MIN_BLOCKS
+         : (std::is_same<S, double>::value && MODE == MODE_STD) ? KSS_F64_MIN_BLOCKS
          : (std::is_same<S, __half>::value && MODE == MODE_STD) ? KSS_F16_MIN_BLOCKS
                                                                 : KSS_STEP_MIN_BLOCKS;
 }
@@ -149,13 +154,16 @@ template <class T, int V> struct VecT;
 template <> struct VecT<float, 4> { using type = float4; };
 template <> struct VecT<float, 2> { using type = float2; };
 template <> struct VecT<double, 2> { using type = double2; };
+template <> struct VecT<double, 1> { using type = double; };
 
 template <class VT, class T, int N>
 __device__ __forceinline__ VT make_vec(const T (&v)[N]) {
   if constexpr (N == 4) {
     return VT{v[0], v[1], v[2], v[3]};
-  } else {
+  } else if constexpr (N == 2) {
     return VT{v[0], v[1]};
+  } else {
+    return v[0];
   }
 }
 
@@ -494,8 +502,10 @@ template <int V>
 __device__ __forceinline__ void store_flags(uint8_t* p, uint32_t bits) {
   if constexpr (V == 4) {
     *reinterpret_cast<uint32_t*>(p) = bits;
-  } else {
+  } else if constexpr (V == 2) {
     *reinterpret_cast<uint16_t*>(p) = uint16_t(bits);
+  } else {
+    *p = uint8_t(bits);
   }
 }
 
@@ -505,20 +515,76 @@ template <int V>
 __device__ __forceinline__ uint32_t load_bytes(const uint8_t* p) {
   if constexpr (V == 4) {
     return *reinterpret_cast<const uint32_t*>(p);
-  } else {
+  } else if constexpr (V == 2) {
     return *reinterpret_cast<const uint16_t*>(p);
+  } else {
+    return *p;
   }
 }
 
 // ---------------------------------------------------------------- fused Kn/KL/neq ----
-// Per-cell accumulators of the {Kn, KL, neq} set.
-template <class T>
+// Per-cell accumulators of the {Kn, KL, neq} set for V cells.
+template <class T, int V = Vec<T>::N>
 struct StdAcc {
-  T kn[Vec<T>::N], neq[Vec<T>::N], kl[Vec<T>::N];
-  T qe[Vec<T>::N];  // AAR steps only: the quasi-equilibrium sensor
+  T kn[V], neq[V], kl[V];
+  T qe[V];  // AAR steps only: the quasi-equilibrium sensor
+  // FP64: x_q and f^neq_q x_q, kept for kl_f64
+  T x[std::is_same<T, double>::value ? 9 : 1][V];
+  T w[std::is_same<T, double>::value ? 9 : 1][V];
 };
 
-// Relax one population of V cells in place (BGK: f <- f - (f - f^eq)/tau) and, on
+// The Kullback-Leibler sums of an FP64 row from x_q and f^neq_q x_q, by the series of phi.
+// The FP64 pipe bounds these rows, so the series is cut where its first dropped term,
+// 2 |x|^(N-1) / (N (N+1)) of its first one, is below 2^-54 for every cell of the warp:
+// N = 6 for |x| < 2^-10, 8 for 2^-7, 15 for 2^-4, 24 for 2^-2.  keep[k] returns whether cell
+// k has |x| < 1/4 throughout; the others are deferred (with cells up to Kn = 1/16 only, the
+// exact recomputation of the cells around a density step took 20 to 30 us per 64^2 step).
+constexpr int kPhiF64Orders[4] = {6, 8, 15, 24};
+template <int N, int V>
+__device__ __forceinline__ void kl_sum_f64(StdAcc<double, V>& a) {
+  constexpr int order[9] = {0, 1, 3, 2, 4, 5, 7, 6, 8};  // as the pairs are relaxed
+#pragma unroll
+  for (int n = 0; n < 9; ++n)
+#pragma unroll
+    for (int k = 0; k < V; ++k)
+      a.kl[k] = fma(a.w[order[n]][k], phi_over_x2<double, N>(a.x[order[n]][k]), a.kl[k]);
+}
+// pair (rows of two warps only, see step_kernel_split): two words of shared memory of the
+// row's warps, which then take the order that a warp of all 64 columns would take.
+template <int V>
+__device__ __forceinline__ void kl_f64(StdAcc<double, V>& a, bool (&keep)[V],
+                                       uint32_t* pair) {
+  // |x| is compared by its high word (sign cleared): NaN and infinity are above every bound
+  constexpr uint32_t kOne = 1023u << 20;
+  uint32_t top = 0;
+#pragma unroll
+  for (int k = 0; k < V; ++k) {
+    uint32_t m = 0;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) m = max(m, uint32_t(__double2hiint(a.x[q][k])) & 0x7fffffffu);
+    keep[k] = m < kOne - (2u << 20);
+    if (keep[k]) top = max(top, m);
+  }
+  top = __reduce_max_sync(kFull, top);
+  if constexpr (V == 1) {
+    const int warp = threadIdx.x >> 5, bar = 1 + (warp >> 1);  // (0 is __syncthreads')
+    if ((threadIdx.x & 31) == 0) pair[warp & 1] = top;
+    asm volatile("bar.sync %0, 64;" ::"r"(bar) : "memory");
+    top = max(pair[0], pair[1]);
+    asm volatile("bar.sync %0, 64;" ::"r"(bar) : "memory");  // read before the next row's
+  }
+  if (top < kOne - (10u << 20)) {
+    kl_sum_f64<kPhiF64Orders[0]>(a);
+  } else if (top < kOne - (7u << 20)) {
+    kl_sum_f64<kPhiF64Orders[1]>(a);
+  } else if (top < kOne - (4u << 20)) {
+    kl_sum_f64<kPhiF64Orders[2]>(a);
+  } else {
+    kl_sum_f64<kPhiF64Orders[3]>(a);
+  }
+}
+
+// Relax one population (q) of V cells in place (BGK: f <- f - (f - f^eq)/tau) and, on
 // output steps, accumulate Kn += |x|, neq += |f^neq| and the Kullback-Leibler term
 // f^eq phi(x) = f^neq x (phi(x)/x^2), x = f^neq / f^eq, by the series of phi.  The
 // series is exact to FP32 for |x| < 1/16; a cell where that, or positivity, cannot be
@@ -534,15 +600,15 @@ struct StdAcc {
 #ifndef KSS_AAR_PAIRED
 #define KSS_AAR_PAIRED 1
 #endif
-template <class T, bool OUT, bool COLLIDE>
-__device__ __forceinline__ void relax_pop(T (&f)[Vec<T>::N], const T (&feq)[Vec<T>::N], T omega,
-                                          StdAcc<T>& a) {
+template <class T, bool OUT, bool COLLIDE, int V>
+__device__ __forceinline__ void relax_pop(T (&f)[V], const T (&feq)[V], T omega,
+                                          StdAcc<T, V>& a, int q) {
 #if KSS_PAIRED_F32
   if constexpr (std::is_same<T, float>::value) {
     constexpr int N = Num<float>::kPhiFastOrder;
     const F2 nom = pack2(-omega, -omega);
 #pragma unroll
-    for (int k = 0; k < Vec<T>::N; k += 2) {
+    for (int k = 0; k < V; k += 2) {
       const F2 F = pack2(f[k], f[k + 1]);
       const F2 fneq = sub2(F, pack2(feq[k], feq[k + 1]));
       if (OUT) {
@@ -574,9 +640,15 @@ __device__ __forceinline__ void relax_pop(T (&f)[Vec<T>::N], const T (&feq)[Vec<
   }
 #endif
 #pragma unroll
-  for (int k = 0; k < Vec<T>::N; ++k) {
+  for (int k = 0; k < V; ++k) {
     const T fneq = f[k] - feq[k];
-    if (OUT) {
+    if constexpr (OUT && std::is_same<T, double>::value) {
+      const T x = ratio64(fneq, feq[k]);  // (used where every feq is positive: fused_row)
+      a.kn[k] += fabs(x);
+      a.neq[k] += fabs(fneq);
+      a.x[q][k] = x;
+      a.w[q][k] = fneq * x;
+    } else if constexpr (OUT) {
       const T x = fneq * Num<T>::rcp(feq[k]);
       a.kn[k] += fabs(x);
       a.neq[k] += fabs(fneq);
@@ -590,16 +662,14 @@ __device__ __forceinline__ void relax_pop(T (&f)[Vec<T>::N], const T (&feq)[Vec<
 // +- 3 cu); both relaxed and (STORE) written out.  AAR: the cells whose region byte (in
 // mbits, one per cell) is set take the two-relaxation update of cell_update, which
 // couples the pair; the others the BGK update, bit for bit.
-template <class S, bool OUT, bool STORE, int QP, int QM, bool AAR = false>
-__device__ __forceinline__ void pair_pops(arith_t<S> (&fp)[Vec<S>::N], arith_t<S> (&fm)[Vec<S>::N],
-                                          const arith_t<S> (&cu)[Vec<S>::N],
-                                          const arith_t<S> (&base)[Vec<S>::N],
-                                          const arith_t<S> (&rw)[Vec<S>::N], arith_t<S> omega,
-                                          StdAcc<arith_t<S>>& a, S* dst_p, S* dst_m,
+template <class S, bool OUT, bool STORE, int QP, int QM, bool AAR, int V>
+__device__ __forceinline__ void pair_pops(arith_t<S> (&fp)[V], arith_t<S> (&fm)[V],
+                                          const arith_t<S> (&cu)[V], const arith_t<S> (&base)[V],
+                                          const arith_t<S> (&rw)[V], arith_t<S> omega,
+                                          StdAcc<arith_t<S>, V>& a, S* dst_p, S* dst_m,
                                           const codec_t<S>& codec, bool cv, uint32_t mbits = 0,
                                           const Trt<arith_t<S>>& trt = Trt<arith_t<S>>{}) {
   using T = arith_t<S>;
-  constexpr int V = Vec<S>::N;
   T ep[V], em[V];
 #pragma unroll
   for (int k = 0; k < V; ++k) {
@@ -608,8 +678,8 @@ __device__ __forceinline__ void pair_pops(arith_t<S> (&fp)[Vec<S>::N], arith_t<S
     em[k] = Num<T>::mul(rw[k], fma(T(-3), cu[k], t));
   }
   if constexpr (AAR) {
-    relax_pop<T, OUT, false>(fp, ep, omega, a);  // the sensors only
-    relax_pop<T, OUT, false>(fm, em, omega, a);
+    relax_pop<T, OUT, false>(fp, ep, omega, a, QP);  // the sensors only
+    relax_pop<T, OUT, false>(fm, em, omega, a, QM);
     if (STORE) {
 #if KSS_PAIRED_F32 && KSS_AAR_PAIRED
       if constexpr (std::is_same<T, float>::value) {
@@ -652,9 +722,9 @@ __device__ __forceinline__ void pair_pops(arith_t<S> (&fp)[Vec<S>::N], arith_t<S
     }
     return;
   }
-  relax_pop<T, OUT, STORE>(fp, ep, omega, a);
+  relax_pop<T, OUT, STORE>(fp, ep, omega, a, QP);
   if (STORE && cv) pop_vstore<S>(dst_p, fp, QP, codec);
-  relax_pop<T, OUT, STORE>(fm, em, omega, a);
+  relax_pop<T, OUT, STORE>(fm, em, omega, a, QM);
   if (STORE && cv) pop_vstore<S>(dst_m, fm, QM, codec);
 }
 
@@ -783,12 +853,14 @@ __device__ __forceinline__ void finalize_sums(const double* part_sum, const uint
         u[m] += __ldcg(part_cnt + 4 * b + m);
       }
     }
+    if (32 * warp < nblocks) {  // (a share without blocks is zero)
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
+      for (int off = 16; off > 0; off >>= 1) {
 #pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        t[m].add(t[m].shfl_xor(off));
-        u[m] += __shfl_xor_sync(kFull, u[m], off);
+        for (int m = 0; m < 3; ++m) {
+          t[m].add(t[m].shfl_xor(off));
+          u[m] += __shfl_xor_sync(kFull, u[m], off);
+        }
       }
     }
     if (lane == 0) {
@@ -1214,15 +1286,14 @@ __device__ __forceinline__ uint32_t fused_row_paired(const StepParams<S>& p,
 // one spills there and measured slower, 0.2257 vs 0.2133 ms per 4096^2 step, while it is
 // faster in one-step launches, 0.2375 vs 0.2769 ms; both give the same results bit for
 // bit).
-template <class S, int MODE, bool PULL, bool STORE, bool AAR = false, bool MULTI = false>
+template <class S, int MODE, bool PULL, bool STORE, bool AAR = false, bool MULTI = false,
+          int V = Vec<S>::N>
 __device__ __forceinline__ uint32_t fused_row(const StepParams<S>& p,
-                                              arith_t<S> (&ft)[9][Vec<S>::N], int i0, int j,
-                                              bool cv, Acc<arith_t<S>>& a_rho,
+                                              arith_t<S> (&ft)[9][V], int i0, int j, bool cv, Acc<arith_t<S>>& a_rho,
                                               Acc<arith_t<S>>& a_jx, Acc<arith_t<S>>& a_jy,
-                                              uint32_t mbits = 0) {
+                                              uint32_t mbits = 0, uint32_t* pair = nullptr) {
   // (AAR: mbits holds the row's region bytes, loaded by the caller with the populations)
   using T = arith_t<S>;
-  constexpr int V = Vec<S>::N;
   constexpr bool OUT = MODE != MODE_PLAIN;
   const long long off = (long long)j * p.pitch + i0;
   uint32_t fbits = 0;
@@ -1254,7 +1325,7 @@ __device__ __forceinline__ uint32_t fused_row(const StepParams<S>& p,
     // per cell: rho/9 (the rest and diagonal weights are exact power-of-two multiples:
     // 4/9 = 4 (1/9), 1/36 = (1/9)/4), u and 1 - 3/2 u^2; kept small for registers
     T rw1[V], ux[V], uy[V], base[V];
-    StdAcc<T> a;
+    StdAcc<T, V> a;
     T rs = T(0), xs = T(0), ys = T(0);
 #pragma unroll
     for (int k = 0; k < V; ++k) {
@@ -1284,7 +1355,7 @@ __device__ __forceinline__ uint32_t fused_row(const StepParams<S>& p,
     // q = 0 (rest)
 #pragma unroll
     for (int k = 0; k < V; ++k) feq[k] = Num<T>::mul(T(4) * rw1[k], base[k]);
-    relax_pop<T, OUT, STORE>(ft[0], feq, p.omega, a);
+    relax_pop<T, OUT, STORE>(ft[0], feq, p.omega, a, 0);
     if (STORE && cv) pop_vstore<S>(p.dst + 0 * p.plane + off, ft[0], 0, p.codec);
     // axis pairs (1, 3): c.u = +-ux ; (2, 4): +-uy ; diagonal pairs (5, 7): +-(ux + uy),
     // (6, 8): +-(uy - ux)
@@ -1312,6 +1383,9 @@ __device__ __forceinline__ uint32_t fused_row(const StepParams<S>& p,
     }
     if (OUT) {
       const Pick3 pr(p.refine_s), ps(p.switch_s);
+      constexpr bool kF64 = std::is_same<T, double>::value;
+      bool keep[V];
+      if constexpr (kF64) kl_f64(a, keep, pair);
 #pragma unroll
       for (int k = 0; k < V; ++k) {
         // rho > 0 and |u|^2 < 0.3 make every f^eq_q >= 0.05 w_q rho > 0, and Kn < 1/16
@@ -1320,7 +1394,13 @@ __device__ __forceinline__ uint32_t fused_row(const StepParams<S>& p,
         // flag byte is KSS_FLAG_DEFERRED only, it is not counted here, and it is
         // recomputed exactly from the unchanged source populations (CTA epilogue or
         // fixup_kernel).
-        const bool fast = (rw1[k] > T(0)) & (base[k] > T(0.55)) & (a.kn[k] < T(0.0625));
+        // (FP64: |x_q| < 1/4, see kl_f64, and rho within the range of ratio64)
+        bool fast = (rw1[k] > T(0)) & (base[k] > T(0.55));
+        if constexpr (kF64) {
+          fast &= keep[k] & (rw1[k] > 0x1p-900) & (rw1[k] < 0x1p900);
+        } else {
+          fast &= a.kn[k] < T(0.0625);
+        }
         a.kl[k] = fabs(a.kl[k]);
         const T er = AAR ? pr(a.kn[k], a.kl[k], a.neq[k], a.qe[k]) : pr(a.kn[k], a.kl[k], a.neq[k]);
         const T es = AAR ? ps(a.kn[k], a.kl[k], a.neq[k], a.qe[k]) : ps(a.kn[k], a.kl[k], a.neq[k]);
@@ -1668,58 +1748,74 @@ struct FullRow {
   uint8_t flags[kCells];
 };
 
-template <class S, bool PULL, bool STORE, bool AAR, bool CG>
-__device__ __forceinline__ uint32_t full_row(const StepParams<S>& p, FullRow<S>& row, int c0,
-                                             int j, int lane) {
-  using T = arith_t<S>;
-  constexpr int V = Vec<S>::N;
+// The nine populations of cell (i, j), one cell per lane (pulled when PULL); ones where !ok
+// (finite: nothing of such a cell is stored or added).
+template <class S, bool PULL, bool CG>
+__device__ __forceinline__ void pull_cell(const StepParams<S>& p, int i, int j, bool ok,
+                                          arith_t<S> (&f)[9]) {
   constexpr int cx[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
   constexpr int cy[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
   long long up, dn;  // rows j - 1 and j + 1
   row_neighbours(p, j, up, dn);
   const S* const src = p.src + (long long)j * p.pitch;
+  const int l = i == 0 ? p.nx - 1 : i - 1, r = i + 1 == p.nx ? 0 : i + 1;
+#pragma unroll
+  for (int q = 0; q < 9; ++q) {
+    f[q] = arith_t<S>(1);
+    if (ok) {
+      const int col = !PULL || cx[q] == 0 ? i : (cx[q] > 0 ? l : r);
+      const long long off = !PULL || cy[q] == 0 ? 0 : (cy[q] > 0 ? up : dn);
+      f[q] = decode<S>(ld_pop<CG>(src + q * p.plane + off + col), q, p.codec);
+    }
+  }
+}
+
+// One cell per lane of an all-sensor step: stores the new populations and the recorded
+// sensors, returns the flag byte and the moments.
+template <class S, bool PULL, bool STORE, bool AAR, bool CG>
+__device__ __forceinline__ uint32_t full_cell(const StepParams<S>& p, int i, int j, bool ok,
+                                              arith_t<S> (&m)[3]) {
+  using T = arith_t<S>;
+  const long long off = (long long)j * p.pitch + i;
+  T f[9], fo[9];
+  pull_cell<S, PULL, CG>(p, i, j, ok, f);
+  // (in a batch, a member without the model has no region: it steps as BGK)
+  const bool switched = AAR && STORE && ok && p.region && p.region[off];
+  CellOut<T> co;
+  cell_update<T, MODE_FULL, STORE, AAR>(f, p.omega, p.tau, fo, co, p.trt, switched, p.need);
+  if (ok) {
+    if (STORE) {
+#pragma unroll
+      for (int q = 0; q < 9; ++q) __stcs(p.dst + q * p.plane + off, encode<S>(fo[q], q, p.codec));
+    }
+#pragma unroll
+    for (int sid = 0; sid < S_COUNT; ++sid) {
+      const int slot = p.rec_slot[sid];
+      if (slot >= 0) p.rec[slot * p.plane + off] = co.sv[sid];
+    }
+  }
+  const bool rf = ok && (pick<T>(co.sv, p.refine_s) > p.thr_r);
+  const bool sw = ok && p.switch_on && (pick<T>(co.sv, p.switch_s) > p.thr_s);
+  m[0] = co.rho;
+  m[1] = co.jx;
+  m[2] = co.jy;
+  return uint32_t(rf) | (uint32_t(sw) << 1) | (uint32_t(ok && co.nonpos) << 7);
+}
+
+template <class S, bool PULL, bool STORE, bool AAR, bool CG>
+__device__ __forceinline__ uint32_t full_row(const StepParams<S>& p, FullRow<S>& row, int c0,
+                                             int j, int lane) {
+  using T = arith_t<S>;
+  constexpr int V = Vec<S>::N;
 #pragma unroll 1
   for (int c = 0; c < V; ++c) {
-    const int t = 32 * c + lane, i = c0 + t;
-    const bool ok = i < p.nx;
-    T f[9], fo[9];
-    uint32_t switched = 0;
-    if (ok) {
-      const int l = i == 0 ? p.nx - 1 : i - 1, r = i + 1 == p.nx ? 0 : i + 1;
-#pragma unroll
-      for (int q = 0; q < 9; ++q) {
-        const int col = !PULL || cx[q] == 0 ? i : (cx[q] > 0 ? l : r);
-        const long long off = !PULL || cy[q] == 0 ? 0 : (cy[q] > 0 ? up : dn);
-        f[q] = decode<S>(ld_pop<CG>(src + q * p.plane + off + col), q, p.codec);
-      }
-      // (in a batch, a member without the model has no region: it steps as BGK)
-      if (AAR && STORE && p.region) switched = p.region[(long long)j * p.pitch + i];
-    } else {
-#pragma unroll
-      for (int q = 0; q < 9; ++q) f[q] = T(1);  // finite; nothing of it is stored or added
-    }
-    CellOut<T> co;
-    cell_update<T, MODE_FULL, STORE, AAR>(f, p.omega, p.tau, fo, co, p.trt, switched != 0u,
-                                          p.need);
-    const long long off = (long long)j * p.pitch + i;
-    if (ok) {
-      if (STORE) {
-#pragma unroll
-        for (int q = 0; q < 9; ++q)
-          __stcs(p.dst + q * p.plane + off, encode<S>(fo[q], q, p.codec));
-      }
-#pragma unroll
-      for (int sid = 0; sid < S_COUNT; ++sid) {
-        const int slot = p.rec_slot[sid];
-        if (slot >= 0) p.rec[slot * p.plane + off] = co.sv[sid];
-      }
-    }
-    const bool rf = ok && (pick<T>(co.sv, p.refine_s) > p.thr_r);
-    const bool sw = ok && p.switch_on && (pick<T>(co.sv, p.switch_s) > p.thr_s);
-    row.flags[t] = uint8_t(uint32_t(rf) | (uint32_t(sw) << 1) | (uint32_t(ok && co.nonpos) << 7));
-    row.m[0][t] = co.rho;
-    row.m[1][t] = co.jx;
-    row.m[2][t] = co.jy;
+    const int t = 32 * c + lane;
+    T m[3];
+    row.flags[t] =
+        uint8_t(full_cell<S, PULL, STORE, AAR, CG>(p, c0 + t, j, c0 + t < p.nx, m));
+    row.m[0][t] = m[0];
+    row.m[1][t] = m[1];
+    row.m[2][t] = m[2];
   }
   __syncwarp();
   uint32_t fbits = 0;
@@ -2170,11 +2266,13 @@ step_kernel_persistent(const StepParams<S> p, int gx, int nblocks) {
 // A block's rows shared out to the CTAs of a cluster, for lattices with too few blocks to
 // fill the GPU (split_ranks).  A warp of an unsplit block takes four or eight rows one after
 // the other; with 4 blocks (128^2) a step lasts as long as four rows, on 4 of 152 SMs.  Here
-// the cluster's CTAs (ranks) take NW rows each, one per warp, with the same row functions;
-// rank 0 then collects the block: tile counts and tags are added over the ranks, and the
-// moments, which every lane leaves in its CTA's shared memory as the values an unsplit block
-// would add to its accumulators, are added by rank 0 in that block's own order.  So the sums
-// are those of the unsplit block bit for bit.
+// the cluster's CTAs (ranks) take NW rows each, one per warp, with the same row functions,
+// and push what the block needs into rank 0's shared memory: tile counts and tags by remote
+// adds, and the moments as the values that the unsplit block's lanes would add to their
+// accumulators.  Rank 0 adds those in the unsplit block's own order, so the sums are the
+// same bit for bit.  Nothing reads another CTA's memory, so no rank waits on a remote load
+// (with rank 0 pulling from 16 ranks, the FP64 epilogue took half of a 37 us step), and the
+// other ranks are done when they have pushed.
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -2191,31 +2289,48 @@ __device__ __forceinline__ void cluster_arrive() {
 __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// *p of the CTA with this rank (p: an address in this CTA's shared memory).
-template <class T>
-__device__ __forceinline__ T ld_rank(const T* p, uint32_t rank) {
-  static_assert(sizeof(T) == 4 || sizeof(T) == 8, "one 4- or 8-byte load");
-  const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(p));
+// The address, in rank 0's shared memory, of p in this CTA's.
+__device__ __forceinline__ uint32_t in_rank0(const void* p) {
   uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-  if constexpr (sizeof(T) == 4) {
-    uint32_t v;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(r) : "memory");
-    return *reinterpret_cast<T*>(&v);
-  } else {
-    unsigned long long v;
-    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(r) : "memory");
-    return *reinterpret_cast<T*>(&v);
-  }
+  asm("mapa.shared::cluster.u32 %0, %1, 0;"
+      : "=r"(r) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(p))));
+  return r;
+}
+__device__ __forceinline__ void st_cluster(uint32_t a, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster(uint32_t a, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void add_cluster(uint32_t a, uint32_t v) {
+  asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 
-// Warps per rank: eight with FP32 arithmetic, where a row is bound by latency; two in FP64,
-// where a block is bound by the FP64 pipes of the SMs it runs on.
+// Warps of a rank and its rows: eight rows of one warp each with FP32 arithmetic, where a
+// row is bound by latency.  FP64 rows are bound by the FP64 pipes, of which each quarter of
+// an SM has its own (64 cycles per warp instruction): a rank takes two rows with two warps
+// each, 32 columns and one cell per lane.
 template <class S>
 __host__ __device__ constexpr int split_warps() {
+  return std::is_same<S, double>::value ? 4 : kWarps;
+}
+template <class S>
+__host__ __device__ constexpr int split_rows() {
   return std::is_same<S, double>::value ? 2 : kWarps;
 }
-constexpr int kSplitRows = 2;  // rows per warp of a rank, at most
+constexpr int kSplitTurns = 2;  // rows per warp of a rank, at most
+
+// Moments per lane and row that rank 0 adds, and the dynamic shared memory of a split block
+// of `rows` rows: the staging slots of the eight-cell rows, then the rows' moments.
+template <class S, int MODE, int VC>
+__host__ __device__ constexpr int split_vals() {
+  return MODE == MODE_FULL || std::is_same<S, double>::value ? Vec<S>::N : (VC == 8 ? 2 : 1);
+}
+template <class S, int MODE, int VC>
+__host__ __device__ constexpr int split_smem(int rows) {
+  return (VC == 8 ? split_warps<S>() * int(sizeof(PfWarpH8)) : 0) +
+         rows * 3 * 32 * split_vals<S, MODE, VC>() * int(sizeof(arith_t<S>));
+}
 
 template <class T>
 __device__ __forceinline__ T acc_value(const Acc<T>& a) {
@@ -2226,53 +2341,148 @@ __device__ __forceinline__ T acc_value(const Acc<T>& a) {
   }
 }
 
+// fix_cell by 16 lanes, lane q < 9 of which takes population q: the nine ratios and their
+// logarithms, which one lane would evaluate one after the other, at once.  Every lane of the
+// warp calls it; `has`: this group of 16 has a cell.  The arithmetic and its order are those
+// of cell_update.  Returns the tags (in every lane of the group).
+template <class S, bool PULL>
+__device__ __forceinline__ uint32_t fix_cell_16(const StepParams<S>& p, const Pick3& pr,
+                                                const Pick3& ps, int i, int j, bool has) {
+  using T = arith_t<S>;
+  const int q = min(int(threadIdx.x & 15), 8);
+  const int cx = q == 0 || q == 2 || q == 4 ? 0 : (q == 1 || q == 5 || q == 8 ? 1 : -1);
+  const int cy = q == 0 || q == 1 || q == 3 ? 0 : (q == 2 || q == 5 || q == 6 ? 1 : -1);
+  T own = T(1);
+  if (has) {
+    int si = i, sj = j;
+    if (PULL) {
+      si = i - cx;
+      sj = j - cy;
+      si = si < 0 ? si + p.nx : (si >= p.nx ? si - p.nx : si);
+      if (!p.slab) sj = sj < 0 ? sj + p.ny : (sj >= p.ny ? sj - p.ny : sj);
+    }
+    own = decode<S>(ld_pop<false>(p.src + q * p.plane + (long long)sj * p.pitch + si), q, p.codec);
+  }
+  T c[9];
+#pragma unroll
+  for (int r = 0; r < 9; ++r) c[r] = __shfl_sync(kFull, own, r, 16);
+  const T rho = ((c[0] + c[1]) + (c[2] + c[3])) + ((c[4] + c[5]) + (c[6] + c[7])) + c[8];
+  const T jx = (c[1] + c[5] + c[8]) - (c[3] + c[6] + c[7]);
+  const T jy = (c[2] + c[5] + c[6]) - (c[4] + c[7] + c[8]);
+  const T inv_rho = Num<T>::rcp(rho);
+  const T ux = Num<T>::mul(jx, inv_rho), uy = Num<T>::mul(jy, inv_rho);
+  // f^eq_q (equilibrium)
+  const T base = fma(T(-1.5), fma(ux, ux, uy * uy), T(1));
+  const T r1 = rho * T(1.0 / 9.0);
+  const T cu = q == 1 || q == 3 ? ux
+               : q == 2 || q == 4 ? uy
+               : q == 5 || q == 7 ? Num<T>::add(ux, uy)
+                                  : Num<T>::sub(uy, ux);
+  const bool minus = q == 3 || q == 4 || q == 7 || q == 8;
+  const T t = fma(T(4.5) * cu, cu, base);
+  const T feq = q == 0 ? Num<T>::mul(T(4) * r1, base)
+                       : Num<T>::mul(q < 5 ? r1 : T(0.25) * r1, fma(minus ? T(-3) : T(3), cu, t));
+  const T fneq = own - feq;
+  const bool bad = (own <= T(0)) | (feq <= T(0));
+  const T x = fneq * Num<T>::rcp(feq);
+  const T ph = phi<T>(x);
+  const unsigned group = 0xffffu << (threadIdx.x & 16);
+  const bool nonpos = (__ballot_sync(kFull, bad) & group) != 0u;
+  T kn = T(0), neq = T(0), kl = T(0), d[9];
+#pragma unroll
+  for (int r = 0; r < 9; ++r) {
+    kn += fabs(__shfl_sync(kFull, x, r, 16));
+    d[r] = __shfl_sync(kFull, fneq, r, 16);
+    neq += fabs(d[r]);
+    kl = fma(__shfl_sync(kFull, feq, r, 16), __shfl_sync(kFull, ph, r, 16), kl);
+  }
+  const T kInf = Num<T>::inf();
+  kn = nonpos ? kInf : kn;
+  kl = nonpos ? kInf : fabs(kl);
+  const T qe = p.trt.qe ? ((fabs(d[1] - d[3]) + fabs(d[2] - d[4])) + fabs(d[5] - d[7])) +
+                              fabs(d[6] - d[8])
+                        : T(0);
+  const bool rr = pr(kn, kl, neq, qe) > p.thr_r;
+  const bool ss = p.switch_on && (ps(kn, kl, neq, qe) > p.thr_s);
+  if (has && (threadIdx.x & 15) == 0) {
+    const long long off = (long long)j * p.pitch + i;
+    p.flags[off] = uint8_t(uint32_t(rr) | (uint32_t(ss) << 1) | (uint32_t(nonpos) << 7));
+    if (p.rec_slot[S_KN] >= 0) p.rec[p.rec_slot[S_KN] * p.plane + off] = kn;
+    if (p.rec_slot[S_KL] >= 0) p.rec[p.rec_slot[S_KL] * p.plane + off] = kl;
+    if (p.rec_slot[S_NEQ] >= 0) p.rec[p.rec_slot[S_NEQ] * p.plane + off] = neq;
+    if (p.trt.qe && p.rec_slot[S_QE] >= 0) p.rec[p.rec_slot[S_QE] * p.plane + off] = qe;
+  }
+  return uint32_t(rr) | (uint32_t(ss) << 1) | (uint32_t(nonpos) << 2);
+}
+
 template <class S, int MODE, bool PULL, bool STORE, bool AAR, int VC>
 __global__ void __launch_bounds__(32 * split_warps<S>(), std::is_same<S, double>::value ? 4 : 2)
 step_kernel_split(const StepParams<S> p) {
   using T = arith_t<S>;
   constexpr int V = Vec<S>::N, NW = split_warps<S>(), NT = 32 * NW;
-  constexpr bool kH8 = VC == 8, FULL = MODE == MODE_FULL;
+  constexpr bool kH8 = VC == 8, FULL = MODE == MODE_FULL, kF64 = std::is_same<S, double>::value;
   constexpr bool kHalfPaired = KSS_ROW_PAIRED && std::is_same<S, __half>::value && !FULL &&
                                !AAR && PULL && V == 4;
   static_assert(MODE != MODE_PLAIN && (VC == V || (kH8 && kHalfPaired && STORE)), "split steps");
-  constexpr int kVals = FULL ? 0 : (kH8 ? 2 : 1);  // accumulator additions per lane and row
-  constexpr int kSlots = kSplitRows * NW;          // rows of this rank
+  constexpr int kVals = split_vals<S, MODE, VC>();
+  constexpr int kCells = kF64 ? 1 : VC;   // cells per lane of a row
+  constexpr int kShare = VC / kCells;     // warps per row
+  static_assert(NW == split_rows<S>() * kShare, "warps of a rank");
   const int bx = blockIdx.x, by = blockIdx.y, gx = gridDim.x;
-  const uint32_t rank = cluster_rank(), ranks = cluster_size();
+  const uint32_t rank = cluster_rank();
   const int lane = threadIdx.x & 31, warp = __shfl_sync(kFull, int(threadIdx.x >> 5), 0);
-  const int rows = p.tile * p.bands, stride = int(ranks) * NW;
-  const int i0 = (bx * 32 + lane) * VC, c0 = bx * 32 * VC;
+  const int rows = p.tile * p.bands, stride = int(cluster_size()) * split_rows<S>();
+  const int c0 = bx * 32 * VC;                             // first column of the block
+  const int t0 = ((warp % kShare) * 32 + lane) * kCells;   // the lane's first cell in its row
+  const int i0 = c0 + t0;
   const bool cv = i0 < p.nx;
   const int j0 = by * rows, j1 = min(j0 + rows, p.ny);
   // (uniform over the cluster: every thread returns, before any barrier)
   if (!bounds_ok(c0 < p.pitch && j0 < p.ny && p.bands >= 1 && p.bands <= kMaxBands &&
-                     rows <= 64 && rows <= stride * kSplitRows,
+                     rows <= 64 && rows <= stride * kSplitTurns,
                  p.err))
     return;
 
-  __shared__ int s_tiles[2][kMaxBands][32];
-  __shared__ uint32_t s_cx[3];                        // tags (refine, switch, nonpos)
-  __shared__ uint16_t s_dl[NW][kSplitRows * 32 * VC];  // each warp's deferred cells
+  __shared__ uint32_t s_tiles[2][kMaxBands][32];           // (rank 0's) tag counts per tile
+  __shared__ uint32_t s_cx[3];                             // (rank 0's) refine, switch, nonpos
+  __shared__ uint16_t s_dl[NW][kSplitTurns * 32 * kCells];  // each warp's deferred cells
   __shared__ uint32_t s_wn[NW];
-  __shared__ T s_val[FULL ? 1 : kSlots][3][kVals ? kVals : 1][32];
-  __shared__ FullRow<S> s_row[FULL ? kSlots : 1];
+  __shared__ FullRow<S> s_row[FULL && !kF64 ? NW : 1];
   __shared__ Red<T> s_sum[kWarps][3];
+  __shared__ uint32_t s_pair[split_rows<S>()][2];  // (FP64: kl_f64)
   extern __shared__ __align__(16) unsigned char kss_dyn_smem[];
+  // (rank 0's) moments: [row of the block][rho, jx, jy][value][lane of the unsplit block]
+  T* const s_val =
+      reinterpret_cast<T*>(kss_dyn_smem + (kH8 ? NW * int(sizeof(PfWarpH8)) : 0));
   for (int t = threadIdx.x; t < 2 * kMaxBands * 32; t += NT) (&s_tiles[0][0][0])[t] = 0;
   if (threadIdx.x < 3) s_cx[threadIdx.x] = 0;
-  __syncthreads();
+  __syncwarp();
+  cluster_arrive();  // rank 0's counters are zero (waited for before the first push)
+  const uint32_t tiles0 = in_rank0(&s_tiles[0][0][0]), cx0 = in_rank0(s_cx);
+  const uint32_t val0 = in_rank0(s_val);
+  auto add_tile = [&](int set, int band, int tl, uint32_t n) {
+    add_cluster(tiles0 + 4u * uint32_t((set * kMaxBands + band) * 32 + tl), n);
+  };
 
   const int tshift = __ffs(p.tile) - 1;
-  const int lshift = tshift - (VC == 8 ? 3 : VC == 4 ? 2 : 1);
-  const int lpt = 1 << lshift;
+  const int lpt = min(p.tile / kCells, 32);  // lanes of a warp in one tile
   uint32_t n_ref = 0, n_sw = 0, n_np = 0, wn = 0;
+  bool waited = false;
 #pragma unroll 1
-  for (int s = 0, rl = int(rank) * NW + warp; j0 + rl < j1; ++s, rl += stride) {
-    const int j = j0 + rl, slot = s * NW + warp;
+  for (int rl = int(rank) * split_rows<S>() + warp / kShare; j0 + rl < j1; rl += stride) {
+    const int j = j0 + rl;
     uint32_t fbits, fbits2 = 0;
+    T mom[3];  // (one value per lane and row)
     Acc<T> a[3], b[3];
-    if constexpr (FULL) {
-      fbits = full_row<S, PULL, STORE, AAR, false>(p, s_row[slot], c0, j, lane);
+    if constexpr (FULL && kF64) {
+      fbits = full_cell<S, PULL, STORE, AAR, false>(p, i0, j, cv, mom);
+      if (cv) {
+        const long long off = (long long)j * p.pitch + i0;
+        store_flags<1>(p.flags + off, fbits);
+        if (AAR && STORE && p.region) store_flags<1>(p.region + off, (fbits >> 1) & 1u);
+      }
+    } else if constexpr (FULL) {
+      fbits = full_row<S, PULL, STORE, AAR, false>(p, s_row[warp], c0, j, lane);
     } else if constexpr (kH8) {
       PfWarpH8* const pw = reinterpret_cast<PfWarpH8*>(kss_dyn_smem) + warp;
       const bool tail = cv && i0 + 8 >= p.nx;
@@ -2296,12 +2506,17 @@ step_kernel_split(const StepParams<S> p) {
       assemble_half_row(p, i0, lane, w, h, f);
       fbits = fused_row_paired<S, MODE, STORE>(p, f, i0, j, cv, a[0], a[1], a[2]);
     } else {
-      T ft[9][V];
+      T ft[9][kCells];
       uint32_t mbits = 0;
       if constexpr (AAR && STORE) {
-        if (cv && p.region) mbits = load_bytes<V>(p.region + (long long)j * p.pitch + i0);
+        if (cv && p.region) mbits = load_bytes<kCells>(p.region + (long long)j * p.pitch + i0);
       }
-      if constexpr (PULL) {
+      if constexpr (kF64) {
+        T f[9];
+        pull_cell<S, PULL, false>(p, i0, j, cv, f);
+#pragma unroll
+        for (int q = 0; q < 9; ++q) ft[q][0] = f[q];
+      } else if constexpr (PULL) {
         pull_row<S, false>(p, j, i0, lane, cv, ft);
       } else {
 #pragma unroll
@@ -2309,16 +2524,30 @@ step_kernel_split(const StepParams<S> p) {
           pop_vload<S, V, false>(p.src + (long long)j * p.pitch + q * p.plane + i0, cv, ft[q], q,
                                  p.codec);
       }
-      fbits = fused_row<S, MODE, PULL, STORE, AAR, false>(p, ft, i0, j, cv, a[0], a[1], a[2], mbits);
+      fbits = fused_row<S, MODE, PULL, STORE, AAR, false, kCells>(p, ft, i0, j, cv, a[0], a[1],
+                                                                  a[2], mbits,
+                                                                  s_pair[warp / kShare]);
     }
-    if constexpr (!FULL) {
+    __syncwarp();
+    if (!waited) cluster_wait();
+    waited = true;
 #pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        s_val[slot][m][0][lane] = acc_value(a[m]);
-        if (kH8) s_val[slot][m][kVals - 1][lane] = acc_value(b[m]);
+    for (int m = 0; m < 3; ++m) {
+      // value k of lane l of the unsplit block: cell V l + k (FP64, all sensors), or its sums
+      const uint32_t at = val0 + uint32_t(sizeof(T)) * uint32_t((rl * 3 + m) * kVals * 32);
+      auto slot = [&](int k, int l) { return at + uint32_t(sizeof(T)) * uint32_t(32 * k + l); };
+      if constexpr (kF64) {
+        st_cluster(slot(t0 % V, t0 / V), FULL ? mom[m] : acc_value(a[m]));
+      } else if constexpr (FULL) {
+#pragma unroll
+        for (int k = 0; k < V; ++k) st_cluster(slot(k, lane), s_row[warp].m[m][lane * V + k]);
+      } else {
+        st_cluster(slot(0, lane), acc_value(a[m]));
+        if constexpr (kH8) st_cluster(slot(1, lane), acc_value(b[m]));
       }
     }
-    // tags of the lane's cells, which all lie in tile lane >> lshift of the row's band
+    if constexpr (FULL) __syncwarp();  // the row is rewritten by the warp's next row
+    // tags of the lane's cells, which all lie in tile t0 >> tshift of the row's band
     int tr = __popc(fbits & 0x01010101u) + __popc(fbits2 & 0x01010101u);
     int ts = __popc(fbits & 0x02020202u) + __popc(fbits2 & 0x02020202u);
     n_ref += tr;
@@ -2331,9 +2560,9 @@ step_kernel_split(const StepParams<S> p) {
         ts += __shfl_xor_sync(kFull, ts, o);
       }
     }
-    if ((lane & (lpt - 1)) == 0 && (tr | ts)) {
-      atomicAdd(&s_tiles[0][rl >> tshift][lane >> lshift], tr);
-      atomicAdd(&s_tiles[1][rl >> tshift][lane >> lshift], ts);
+    if ((lane & (lpt - 1)) == 0) {
+      if (tr) add_tile(0, rl >> tshift, t0 >> tshift, uint32_t(tr));
+      if (ts) add_tile(1, rl >> tshift, t0 >> tshift, uint32_t(ts));
     }
     if constexpr (MODE == MODE_STD) {
       // deferred cells (see step_block), as offsets in the block
@@ -2348,10 +2577,10 @@ step_kernel_split(const StepParams<S> p) {
         }
         uint32_t at = wn + uint32_t(incl - nd);
 #pragma unroll
-        for (int k = 0; k < VC; ++k) {
+        for (int k = 0; k < kCells; ++k) {
           if (((k < 4 ? dbits : dbits2) >> (8 * (k & 3))) & 0x40u) {
-            if (bounds_ok(at < uint32_t(kSplitRows * 32 * VC), p.err))
-              s_dl[warp][at] = uint16_t(rl * 32 * VC + lane * VC + k);
+            if (bounds_ok(at < uint32_t(kSplitTurns * 32 * kCells), p.err))
+              s_dl[warp][at] = uint16_t(rl * 32 * VC + t0 + k);
             ++at;
           }
         }
@@ -2359,106 +2588,136 @@ step_kernel_split(const StepParams<S> p) {
       }
     }
   }
+  __syncwarp();
+  if (!waited) cluster_wait();
   n_ref = __reduce_add_sync(kFull, n_ref);
   n_sw = __reduce_add_sync(kFull, n_sw);
   n_np = __reduce_add_sync(kFull, n_np);
   if (lane == 0) {
-    if (n_ref) atomicAdd(&s_cx[0], n_ref);
-    if (n_sw) atomicAdd(&s_cx[1], n_sw);
-    if (n_np) atomicAdd(&s_cx[2], n_np);
+    if (n_ref) add_cluster(cx0, n_ref);
+    if (n_sw) add_cluster(cx0 + 4, n_sw);
+    if (n_np) add_cluster(cx0 + 8, n_np);
     s_wn[warp] = wn;
   }
   if constexpr (MODE == MODE_STD) {
-    // this rank's deferred cells: exact recomputation (see step_block)
+    // this rank's deferred cells: exact recomputation (see step_block), 16 lanes per cell
+    // while that takes each group two cells at most (one in FP64, where every warp
+    // instruction costs the same however few of its lanes work), else one lane per cell
     __syncthreads();
     uint32_t total = 0;
 #pragma unroll
     for (int w = 0; w < NW; ++w) total += s_wn[w];
     if (total) {
       const Pick3 pr(p.refine_s), ps(p.switch_s);
-      for (uint32_t e = threadIdx.x; e < total; e += NT) {
-        uint32_t w = 0, r = e;
-        while (r >= s_wn[w]) r -= s_wn[w++];
-        const int o = s_dl[w][r];
+      const bool few = total <= (kF64 ? 1u : 2u) * (NT / 16);
+      const uint32_t step = few ? NT / 16 : NT;
+      const uint32_t first = few ? threadIdx.x >> 4 : threadIdx.x;
+      for (uint32_t e0 = 0; e0 < total; e0 += step) {  // (uniform trips)
+        const uint32_t e = e0 + first;
+        const bool has = e < total;
+        uint32_t w = 0, r = has ? e : 0;
+        while (has && r >= s_wn[w]) r -= s_wn[w++];
+        const int o = has ? s_dl[w][r] : 0;
         const int rl = o / (32 * VC), cl = o - rl * (32 * VC);
         const int j = j0 + rl, i = c0 + cl;
-        if (!bounds_ok(j < j1 && i < p.nx && rl / p.tile < kMaxBands && cl / p.tile < 32, p.err))
-          continue;
-        const uint32_t tags = fix_cell<S, PULL, false>(p, pr, ps, i, j);
+        const bool ok = has && bounds_ok(j < j1 && i < p.nx && rl / p.tile < kMaxBands &&
+                                             cl / p.tile < 32, p.err);
+        uint32_t tags = 0;
+        if (few) {
+          tags = fix_cell_16<S, PULL>(p, pr, ps, i, j, ok);
+          if (threadIdx.x & 15) continue;
+        } else if (ok) {
+          tags = fix_cell<S, PULL, false>(p, pr, ps, i, j);
+        }
+        if (!ok) continue;
         if (AAR && STORE && p.region) p.region[(long long)j * p.pitch + i] = uint8_t((tags >> 1) & 1u);
         const int bd = rl / p.tile, tl = cl / p.tile;
         if (tags & 1u) {
-          atomicAdd(&s_cx[0], 1u);
-          atomicAdd(&s_tiles[0][bd][tl], 1);
+          add_cluster(cx0, 1u);
+          add_tile(0, bd, tl, 1u);
         }
         if (tags & 2u) {
-          atomicAdd(&s_cx[1], 1u);
-          atomicAdd(&s_tiles[1][bd][tl], 1);
+          add_cluster(cx0 + 4, 1u);
+          add_tile(1, bd, tl, 1u);
         }
-        if (tags & 4u) atomicAdd(&s_cx[2], 1u);
+        if (tags & 4u) add_cluster(cx0 + 8, 1u);
       }
     }
   }
   __syncwarp();
-  cluster_arrive();  // the ranks' rows, counts and moments are in shared memory
+  cluster_arrive();  // everything this rank pushes has been pushed
+  if (rank != 0) return;
   cluster_wait();
   const int bid = by * gx + bx;
-  if (rank == 0) {
-    // the moments in the order of the unsplit block: its warp w adds rows w, w + 8, ...
-#pragma unroll 1
-    for (int w = warp; w < kWarps; w += NW) {
-      Acc<T> a[3];
-      for (int rl = w; rl < rows && j0 + rl < j1; rl += kWarps) {
-        const int at = rl % stride, slot = (rl / stride) * NW + at % NW;
-        const uint32_t from = uint32_t(at / NW);
+  // the moments in the order of the unsplit block: its warp w adds rows w, w + 8, ...
+  Acc<T> a[kWarps / NW][3];
+  for (int r8 = 0; r8 < rows; r8 += kWarps) {
+#pragma unroll
+    for (int n = 0; n < kWarps / NW; ++n) {
+      const int rl = r8 + n * NW + warp;
+      if (j0 + rl < j1) {
 #pragma unroll
         for (int m = 0; m < 3; ++m) {
-          if constexpr (FULL) {
+          const T* const v = s_val + (rl * 3 + m) * kVals * 32 + lane;
+          if constexpr (kF64 && !FULL) {  // the lane's cells, then the row
+            T sum = T(0);
 #pragma unroll
-            for (int k = 0; k < V; ++k) {
-              const int t = lane * V + k;
-              const T v = ld_rank(&s_row[slot].m[m][t], from);
-              if (c0 + t < p.nx) a[m].add(v);
-            }
+            for (int k = 0; k < kVals; ++k) sum += v[32 * k];
+            a[n][m].add(sum);
           } else {
+            // (an all-sensor row adds its lane's cells one by one, those of the lattice)
 #pragma unroll
-            for (int c = 0; c < kVals; ++c) a[m].add(ld_rank(&s_val[slot][m][c][lane], from));
+            for (int k = 0; k < kVals; ++k)
+              if (!FULL || c0 + lane * V + k < p.nx) a[n][m].add(v[32 * k]);
           }
         }
       }
-#pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        a[m].warp_reduce();
-        if (lane == 0) s_sum[w][m] = Red<T>::of(a[m]);
-      }
-    }
-    const int tpb = (32 * VC) / p.tile;
-    for (int t = threadIdx.x; t < 2 * tpb * p.bands; t += NT) {
-      const int set = t / (tpb * p.bands), u = t - set * (tpb * p.bands);
-      const int b = u / tpb, tl = u - b * tpb;
-      const int tx = bx * tpb + tl, ty = by * p.bands + b;
-      if (tx < p.ntx && ty < p.nty) {
-        int n = 0;
-        for (uint32_t r = 0; r < ranks; ++r) n += ld_rank(&s_tiles[set][b][tl], r);
-        p.tiles[(long long)set * p.ntx * p.nty + (long long)ty * p.ntx + tx] = n;
-      }
-    }
-    __syncthreads();
-    if (threadIdx.x < 3) {
-      const int m = threadIdx.x;
-      Red<T> sum;
-      uint32_t c = 0;
-      for (int w = 0; w < kWarps; ++w) sum.add(s_sum[w][m]);
-      for (uint32_t r = 0; r < ranks; ++r) c += ld_rank(&s_cx[m], r);
-      sum.store(p.part_sum + 3 * bid + m);
-      p.part_cnt[4 * bid + m] = c;
     }
   }
-  __syncwarp();
-  cluster_arrive();  // rank 0 has read the other ranks' shared memory
-  cluster_wait();
-  // (threads 0-2 of rank 0 wrote the block's partials before the barrier above)
-  if (rank == 0) ticket_and_finalize<S, NT>(p, gx * int(gridDim.y), gx * int(gridDim.y));
+#pragma unroll
+  for (int n = 0; n < kWarps / NW; ++n)
+#pragma unroll
+    for (int m = 0; m < 3; ++m) {
+      a[n][m].warp_reduce();
+      if (lane == 0) s_sum[n * NW + warp][m] = Red<T>::of(a[n][m]);
+    }
+  const int tpb = (32 * VC) / p.tile;
+  for (int t = threadIdx.x; t < 2 * tpb * p.bands; t += NT) {
+    const int set = t / (tpb * p.bands), u = t - set * (tpb * p.bands);
+    const int b = u / tpb, tl = u - b * tpb;
+    const int tx = bx * tpb + tl, ty = by * p.bands + b;
+    if (tx < p.ntx && ty < p.nty)
+      p.tiles[(long long)set * p.ntx * p.nty + (long long)ty * p.ntx + tx] =
+          int(s_tiles[set][b][tl]);
+  }
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    const int m = threadIdx.x;
+    Red<T> sum;
+    for (int w = 0; w < kWarps; ++w) sum.add(s_sum[w][m]);
+    sum.store(p.part_sum + 3 * bid + m);
+    p.part_cnt[4 * bid + m] = s_cx[m];
+  }
+  __syncwarp();  // thread 0's fence covers the partials that threads 1 and 2 wrote
+  ticket_and_finalize<S, NT>(p, gx * int(gridDim.y), gx * int(gridDim.y));
+}
+
+// A plain FP64 step of a small lattice: CTAs of two rows of 64 columns, one cell per lane
+// (four warps: one on each of the SM's FP64 pipes; see split_warps).
+template <bool AAR>
+__global__ void __launch_bounds__(128) step_plain_f64_kernel(const StepParams<double> p) {
+  const int lane = threadIdx.x & 31, warp = __shfl_sync(kFull, int(threadIdx.x >> 5), 0);
+  const int i = blockIdx.x * 64 + (warp & 1) * 32 + lane, j = blockIdx.y * 2 + (warp >> 1);
+  if (j >= p.ny) return;
+  const bool ok = i < p.nx;
+  double f[9], ft[9][1];
+  pull_cell<double, true, false>(p, i, j, ok, f);
+#pragma unroll
+  for (int q = 0; q < 9; ++q) ft[q][0] = f[q];
+  const uint32_t mbits = AAR && ok && p.region ? p.region[(long long)j * p.pitch + i] : 0u;
+  Acc<double> unused[3];
+  fused_row<double, MODE_PLAIN, true, true, AAR, false, 1>(p, ft, i, j, ok, unused[0], unused[1],
+                                                           unused[2], mbits);
 }
 
 // ---------------------------------------------------------------- multi-step ----
