@@ -457,7 +457,7 @@ int kss_regrid(kss_lattice* L, int32_t buffer, double efficiency, uint8_t* tile_
     return fail(L, KSS_ERR_ARG, "invalid regrid argument");
   DeviceGuard g(L->device);
   // the flags of the current step (evaluated if this step had no outputs)
-  if ((rc = kss_read_flags(L, nullptr, nullptr, nullptr, 1)) < 0) return rc;
+  if ((rc = ensure_flags(L)) || (rc = device_error(L))) return rc;
   if (!L->regrid) {
     L->regrid = new (std::nothrow) RegridWS();
     if (!L->regrid) return fail(L, KSS_ERR_OOM, "regrid workspace");

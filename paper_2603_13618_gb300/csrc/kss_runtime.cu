@@ -382,36 +382,133 @@ int ensure_outputs(kss_lattice* L, int sensor, const void** field) {
   return KSS_OK;
 }
 
-int nonpos_status(kss_lattice* L) {
-  unsigned long long c[3];
-  KSS_CUDA(L, cudaMemcpyAsync(c, L->stat_counts, sizeof(c), cudaMemcpyDeviceToHost, L->stream));
-  KSS_CUDA(L, cudaStreamSynchronize(L->stream));
-  const int rc = device_error(L);
-  if (rc) return rc;
-  return c[2] > 0 ? KSS_WARN_NONPOSITIVE : KSS_OK;
+// The status block into page-locked host memory (one CTA of 64 threads, one word each).
+__global__ void status_kernel(const uint32_t* __restrict__ block, uint32_t* __restrict__ mail) {
+  mail[threadIdx.x] = block[threadIdx.x];
+}
+
+// Flag bytes (pitched) and tile counts to dense arrays (nullptr: not wanted), V flags per
+// thread: one launch instead of a 2-D copy and a copy.
+template <int V>
+struct alignas(V) Bytes {
+  uint8_t b[V];
+};
+template <int V>
+__global__ void flags_out_kernel(const uint8_t* __restrict__ flags, int pitch, int nx, int ny,
+                                 uint8_t* __restrict__ out, const int32_t* __restrict__ tiles,
+                                 int ntiles, int32_t* __restrict__ tiles_out) {
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) * V;
+  if (out && i < nx)
+    for (int j = blockIdx.y; j < ny; j += gridDim.y)
+      *reinterpret_cast<Bytes<V>*>(out + (long long)j * nx + i) =
+          *reinterpret_cast<const Bytes<V>*>(flags + (long long)j * pitch + i);
+  if (tiles_out) {
+    const int per = gridDim.x * blockDim.x;
+    for (long long t = (long long)blockIdx.y * per + blockIdx.x * blockDim.x + threadIdx.x;
+         t < ntiles; t += (long long)gridDim.y * per)
+      tiles_out[t] = tiles[t];
+  }
+}
+
+cudaError_t launch_flags_out(kss_lattice* L, uint8_t* out, int32_t* tiles_out) {
+  const int nx = L->cfg.nx, ny = L->cfg.ny, n = 2 * L->ntx * L->nty;
+  const uintptr_t at = reinterpret_cast<uintptr_t>(out);
+  auto go = [&](auto width) {
+    constexpr int V = decltype(width)::value;
+    const dim3 g((nx + 256 * V - 1) / (256 * V), ny < 65535 ? ny : 65535);
+    flags_out_kernel<V><<<g, 256, 0, L->stream>>>(L->flags, L->pitch, nx, ny, out, L->tiles, n,
+                                                  tiles_out);
+    return cudaGetLastError();
+  };
+  // (rows of the pitched plane are 16-byte aligned: its pitch is a multiple of 16 elements)
+  if (nx % 16 == 0 && at % 16 == 0) return go(std::integral_constant<int, 16>{});
+  if (nx % 4 == 0 && at % 4 == 0) return go(std::integral_constant<int, 4>{});
+  return go(std::integral_constant<int, 1>{});
 }
 
 }  // namespace
 
 namespace kss_rt {
 
-// After a stream synchronisation: did a bounded device wait run out?  (sticky)
-int device_error(kss_lattice* L) {
-  uint32_t w = 0;
-  KSS_CUDA(L, cudaMemcpyAsync(&w, L->err_word, sizeof(w), cudaMemcpyDeviceToHost, L->stream));
+// ---- borrowed page-locked memory ----
+namespace lease_pool {
+std::mutex g_mutex;
+unsigned char* g_kept[HostLease::kKeptLeases];
+int g_n = 0;
+}  // namespace lease_pool
+
+HostLease::HostLease(bool wanted) : p(nullptr) {
+  if (!wanted) return;
+  {
+    std::lock_guard<std::mutex> lock(lease_pool::g_mutex);
+    if (lease_pool::g_n > 0) {
+      p = lease_pool::g_kept[--lease_pool::g_n];
+      return;
+    }
+  }
+  // (another thread's stream capture is not disturbed by the allocation)
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  void* q = nullptr;
+  if (cudaHostAlloc(&q, kBytes, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+    cudaGetLastError();
+    q = nullptr;
+  }
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  p = static_cast<unsigned char*>(q);
+}
+
+HostLease::~HostLease() {
+  if (!p) return;
+  {
+    std::lock_guard<std::mutex> lock(lease_pool::g_mutex);
+    if (lease_pool::g_n < kKeptLeases) {
+      lease_pool::g_kept[lease_pool::g_n++] = p;
+      return;
+    }
+  }
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (cudaFreeHost(p) != cudaSuccess) cudaGetLastError();
+  cudaThreadExchangeStreamCaptureMode(&mode);
+}
+
+int finish(kss_lattice* L, const HostLease& lease, Status* st) {
+  unsigned char block[HostLease::kMailBytes];
+  const unsigned char* b = lease.p;
+  if (b) {
+    status_kernel<<<1, 64, 0, L->stream>>>(reinterpret_cast<const uint32_t*>(L->small),
+                                           reinterpret_cast<uint32_t*>(lease.p));
+    KSS_CUDA(L, cudaGetLastError());
+  } else {
+    KSS_CUDA(L, cudaMemcpyAsync(block, L->small, sizeof(block), cudaMemcpyDeviceToHost, L->stream));
+    b = block;
+  }
   KSS_CUDA(L, cudaStreamSynchronize(L->stream));
-  if (w & kss::kErrBounds) {
+  Status s;
+  std::memcpy(s.sums, b + 64, sizeof(s.sums));
+  std::memcpy(s.counts, b + 128, sizeof(s.counts));
+  std::memcpy(&s.err, b + 192, sizeof(s.err));
+  if (st) *st = s;
+  if (s.err & kss::kErrBounds) {
     L->err = KSS_ERR_BOUNDS;
     L->msg = "a device bounds check failed (debug build)";
     return KSS_ERR_BOUNDS;
   }
-  if (w) {
+  if (s.err) {
     L->err = KSS_ERR_TIMEOUT;
     L->msg = "a bounded device wait ran out (bulk copy did not complete)";
     return KSS_ERR_TIMEOUT;
   }
   return KSS_OK;
 }
+
+int device_error(kss_lattice* L) {
+  const HostLease lease;
+  return finish(L, lease);
+}
+
+int ensure_flags(kss_lattice* L) { return ensure_outputs(L, -1, nullptr); }
 
 // ---- counted device allocations and host-side fault injection (test support) ----
 namespace inject {
@@ -704,7 +801,16 @@ int set_fields_of(kss_lattice* L, const E* rho, const E* ux, const E* uy, int on
     u = pinned_device_view(ux);
     v = pinned_device_view(uy);
   }
-  if (!on_device && !(r && u && v)) {
+  const HostLease lease(!on_device && !(r && u && v));
+  E* const mail = static_cast<E*>(lease.room(3 * n * sizeof(E)));
+  if (!on_device && !(r && u && v) && mail) {  // small arrays: through page-locked memory
+    std::memcpy(mail, rho, n * sizeof(E));
+    std::memcpy(mail + n, ux, n * sizeof(E));
+    std::memcpy(mail + 2 * n, uy, n * sizeof(E));
+    r = mail;
+    u = mail + n;
+    v = mail + 2 * n;
+  } else if (!on_device && !(r && u && v)) {
     // (the staging buffer holds 3 n doubles: enough for 3 n elements of either type)
     if ((rc = ensure_staging(L, 3 * n))) return rc;
     E* st = reinterpret_cast<E*>(L->staging);
@@ -750,6 +856,11 @@ int kss_set_populations(kss_lattice* L, const double* f, int on_device) {
   DeviceGuard g(L->device);
   const size_t n = 9 * size_t(L->cfg.nx) * L->cfg.ny;
   const double* src = on_device ? f : pinned_device_view(f);
+  const HostLease lease(!src);
+  if (double* const mail = src ? nullptr : static_cast<double*>(lease.room(n * 8))) {
+    std::memcpy(mail, f, n * 8);
+    src = mail;
+  }
   if (!src) {
     if ((rc = ensure_staging(L, n))) return rc;
     KSS_CUDA(L, cudaMemcpyAsync(L->staging, f, n * 8, cudaMemcpyHostToDevice, L->stream));
@@ -772,8 +883,10 @@ int kss_get_populations(kss_lattice* L, double* f, int on_device) {
   if (!f) return fail(L, KSS_ERR_ARG, "null population pointer");
   DeviceGuard g(L->device);
   const size_t n = 9 * size_t(L->cfg.nx) * L->cfg.ny;
-  double* dst = f;
-  if (!on_device) {
+  const HostLease lease;
+  double* const mail = on_device ? nullptr : static_cast<double*>(lease.room(n * 8));
+  double* dst = mail ? mail : f;
+  if (!on_device && !mail) {
     if ((rc = ensure_staging(L, n))) return rc;
     dst = L->staging;
   }
@@ -783,10 +896,11 @@ int kss_get_populations(kss_lattice* L, double* f, int on_device) {
              return kss::launch_pops_to_dense<S>(static_cast<const S*>(L->f[L->cur]), L->plane,
                                                  L->pitch, nx, ny, dst, codec_of<S>(L), L->stream);
            }));
-  if (!on_device)
+  if (!on_device && !mail)
     KSS_CUDA(L, cudaMemcpyAsync(f, L->staging, n * 8, cudaMemcpyDeviceToHost, L->stream));
-  KSS_CUDA(L, cudaStreamSynchronize(L->stream));
-  return device_error(L);
+  if ((rc = finish(L, lease))) return rc;
+  if (mail) std::memcpy(f, mail, n * 8);
+  return KSS_OK;
 }
 
 int kss_step(kss_lattice* L, int32_t nsteps) {
@@ -851,12 +965,14 @@ int kss_read_moments(kss_lattice* L, double* rho, double* ux, double* uy, int on
   if (!rho || !ux || !uy) return fail(L, KSS_ERR_ARG, "null field pointer");
   DeviceGuard g(L->device);
   const size_t n = size_t(L->cfg.nx) * L->cfg.ny;
+  const HostLease lease;
+  double* const mail = on_device ? nullptr : static_cast<double*>(lease.room(3 * n * 8));
   double *r = rho, *u = ux, *v = uy;
   if (!on_device) {
-    if ((rc = ensure_staging(L, 3 * n))) return rc;
-    r = L->staging;
-    u = L->staging + n;
-    v = L->staging + 2 * n;
+    if (!mail && (rc = ensure_staging(L, 3 * n))) return rc;
+    r = mail ? mail : L->staging;
+    u = r + n;
+    v = r + 2 * n;
   }
   const int nx = L->cfg.nx, ny = L->cfg.ny;
   KSS_CUDA(L, with_storage(L->cfg.precision, [&](auto tag) {
@@ -864,13 +980,18 @@ int kss_read_moments(kss_lattice* L, double* rho, double* ux, double* uy, int on
              return kss::launch_moments<S>(static_cast<const S*>(L->f[L->cur]), L->plane,
                                            L->pitch, nx, ny, r, u, v, codec_of<S>(L), L->stream);
            }));
-  if (!on_device) {
+  if (!on_device && !mail) {
     KSS_CUDA(L, cudaMemcpyAsync(rho, r, n * 8, cudaMemcpyDeviceToHost, L->stream));
     KSS_CUDA(L, cudaMemcpyAsync(ux, u, n * 8, cudaMemcpyDeviceToHost, L->stream));
     KSS_CUDA(L, cudaMemcpyAsync(uy, v, n * 8, cudaMemcpyDeviceToHost, L->stream));
   }
-  KSS_CUDA(L, cudaStreamSynchronize(L->stream));
-  return device_error(L);
+  if ((rc = finish(L, lease))) return rc;
+  if (mail) {
+    std::memcpy(rho, r, n * 8);
+    std::memcpy(ux, u, n * 8);
+    std::memcpy(uy, v, n * 8);
+  }
+  return KSS_OK;
 }
 
 int kss_read_sensor(kss_lattice* L, int32_t sensor, double* out, int on_device) {
@@ -882,8 +1003,10 @@ int kss_read_sensor(kss_lattice* L, int32_t sensor, double* out, int on_device) 
   const void* field = nullptr;
   if ((rc = ensure_outputs(L, sensor, &field))) return rc;
   const size_t n = size_t(L->cfg.nx) * L->cfg.ny;
-  double* dst = out;
-  if (!on_device) {
+  const HostLease lease;
+  double* const mail = on_device ? nullptr : static_cast<double*>(lease.room(n * 8));
+  double* dst = mail ? mail : out;
+  if (!on_device && !mail) {
     if ((rc = ensure_staging(L, n))) return rc;
     dst = L->staging;
   }
@@ -894,9 +1017,12 @@ int kss_read_sensor(kss_lattice* L, int32_t sensor, double* out, int on_device) 
   else
     KSS_CUDA(L, kss::launch_pitched_to_dense<double>(static_cast<const double*>(field), L->plane,
                                                      L->pitch, nx, ny, 1, dst, L->stream));
-  if (!on_device)
+  if (!on_device && !mail)
     KSS_CUDA(L, cudaMemcpyAsync(out, L->staging, n * 8, cudaMemcpyDeviceToHost, L->stream));
-  return nonpos_status(L);
+  Status st;
+  if ((rc = finish(L, lease, &st))) return rc;
+  if (mail) std::memcpy(out, mail, n * 8);
+  return st.counts[2] > 0 ? KSS_WARN_NONPOSITIVE : KSS_OK;
 }
 
 int kss_read_flags(kss_lattice* L, uint8_t* flags, int32_t* tile_counts, int64_t counts[3],
@@ -905,20 +1031,33 @@ int kss_read_flags(kss_lattice* L, uint8_t* flags, int32_t* tile_counts, int64_t
   if (rc) return rc;
   DeviceGuard g(L->device);
   if ((rc = ensure_outputs(L, -1, nullptr))) return rc;
-  const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-  if (flags)
-    KSS_CUDA(L, cudaMemcpy2DAsync(flags, size_t(L->cfg.nx), L->flags, size_t(L->pitch),
-                                  size_t(L->cfg.nx), size_t(L->cfg.ny), kind, L->stream));
-  if (tile_counts)
-    KSS_CUDA(L, cudaMemcpyAsync(tile_counts, L->tiles,
-                                sizeof(int32_t) * 2 * size_t(L->ntx) * L->nty, kind, L->stream));
-  unsigned long long c[3];
-  KSS_CUDA(L, cudaMemcpyAsync(c, L->stat_counts, sizeof(c), cudaMemcpyDeviceToHost, L->stream));
-  KSS_CUDA(L, cudaStreamSynchronize(L->stream));
-  if ((rc = device_error(L))) return rc;
+  const size_t nf = flags ? size_t(L->cfg.nx) * L->cfg.ny : 0;
+  const size_t nt = tile_counts ? sizeof(int32_t) * 2 * size_t(L->ntx) * L->nty : 0;
+  const size_t at = (nf + 15) / 16 * 16;  // the tile counts' place after the flags
+  const HostLease lease;
+  unsigned char* const mail =
+      on_device ? nullptr : static_cast<unsigned char*>(lease.room(at + nt));
+  if (on_device || mail) {
+    uint8_t* const fo = !flags ? nullptr : mail ? mail : flags;
+    int32_t* const to = !tile_counts ? nullptr
+                        : mail       ? reinterpret_cast<int32_t*>(mail + at)
+                                     : tile_counts;
+    if (fo || to) KSS_CUDA(L, launch_flags_out(L, fo, to));
+  } else {
+    if (flags)
+      KSS_CUDA(L, cudaMemcpy2DAsync(flags, size_t(L->cfg.nx), L->flags, size_t(L->pitch),
+                                    size_t(L->cfg.nx), size_t(L->cfg.ny), cudaMemcpyDeviceToHost,
+                                    L->stream));
+    if (tile_counts)
+      KSS_CUDA(L, cudaMemcpyAsync(tile_counts, L->tiles, nt, cudaMemcpyDeviceToHost, L->stream));
+  }
+  Status st;
+  if ((rc = finish(L, lease, &st))) return rc;
+  if (mail && nf) std::memcpy(flags, mail, nf);
+  if (mail && nt) std::memcpy(tile_counts, mail + at, nt);
   if (counts)
-    for (int k = 0; k < 3; ++k) counts[k] = int64_t(c[k]);
-  return c[2] > 0 ? KSS_WARN_NONPOSITIVE : KSS_OK;
+    for (int k = 0; k < 3; ++k) counts[k] = int64_t(st.counts[k]);
+  return st.counts[2] > 0 ? KSS_WARN_NONPOSITIVE : KSS_OK;
 }
 
 int kss_read_stats(kss_lattice* L, double sums[3], int64_t counts[3], int64_t* step) {
@@ -926,18 +1065,15 @@ int kss_read_stats(kss_lattice* L, double sums[3], int64_t counts[3], int64_t* s
   if (rc) return rc;
   DeviceGuard g(L->device);
   if ((rc = ensure_outputs(L, -1, nullptr))) return rc;
-  double s[3];
-  unsigned long long c[3];
-  KSS_CUDA(L, cudaMemcpyAsync(s, L->stat_sums, sizeof(s), cudaMemcpyDeviceToHost, L->stream));
-  KSS_CUDA(L, cudaMemcpyAsync(c, L->stat_counts, sizeof(c), cudaMemcpyDeviceToHost, L->stream));
-  KSS_CUDA(L, cudaStreamSynchronize(L->stream));
-  if ((rc = device_error(L))) return rc;
+  const HostLease lease;
+  Status st;
+  if ((rc = finish(L, lease, &st))) return rc;
   if (sums)
-    for (int k = 0; k < 3; ++k) sums[k] = s[k];
+    for (int k = 0; k < 3; ++k) sums[k] = st.sums[k];
   if (counts)
-    for (int k = 0; k < 3; ++k) counts[k] = int64_t(c[k]);
+    for (int k = 0; k < 3; ++k) counts[k] = int64_t(st.counts[k]);
   if (step) *step = L->out_step;
-  return c[2] > 0 ? KSS_WARN_NONPOSITIVE : KSS_OK;
+  return st.counts[2] > 0 ? KSS_WARN_NONPOSITIVE : KSS_OK;
 }
 
 int kss_set_aar_region(kss_lattice* L, const uint8_t* region, int on_device) {
@@ -968,7 +1104,6 @@ int kss_get_aar_region(kss_lattice* L, uint8_t* region, int on_device) {
                                 size_t(L->cfg.nx), size_t(L->cfg.ny),
                                 on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                                 L->stream));
-  KSS_CUDA(L, cudaStreamSynchronize(L->stream));
   return device_error(L);
 }
 
@@ -1063,7 +1198,6 @@ int kss_sync(kss_lattice* L) {
   int rc = enter(L);
   if (rc) return rc;
   DeviceGuard g(L->device);
-  KSS_CUDA(L, cudaStreamSynchronize(L->stream));
   return device_error(L);
 }
 

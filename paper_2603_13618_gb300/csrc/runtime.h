@@ -249,8 +249,38 @@ inline int enter(kss_lattice* L) {
 // Free a lattice's device buffers and stream after its stream drains (kss_runtime.cu).
 void release(kss_lattice* L);
 
-// After a stream synchronisation: did a bounded device wait run out?  (sticky)
+// Page-locked host memory that kernels read and write in place, borrowed for the length of
+// one call: the first kMailBytes take the lattice's status block, the rest small arrays on
+// their way from or to pageable memory.  A call that needs it takes a lease from a pool,
+// shared by all threads and lattices, which keeps at most kKeptLeases buffers between calls
+// and frees the others.  `p` is nullptr if page-locked memory could not be had (the calls
+// then copy through the driver as for large arrays).
+struct HostLease {
+  static constexpr size_t kMailBytes = 256, kBytes = size_t(1) << 20;
+  static constexpr int kKeptLeases = 4;
+  unsigned char* p;
+  explicit HostLease(bool wanted = true);
+  ~HostLease();
+  HostLease(const HostLease&) = delete;
+  HostLease& operator=(const HostLease&) = delete;
+  // room for `bytes` of array data, or nullptr
+  void* room(size_t bytes) const { return p && bytes <= kBytes - kMailBytes ? p + kMailBytes : nullptr; }
+};
+
+// A lattice's status block (kss_lattice::small) as of a stream synchronisation.
+struct Status {
+  double sums[3];
+  unsigned long long counts[3];
+  uint32_t err;
+};
+// Wait for the lattice's stream and read its status block, in one synchronisation: a kernel
+// at the end of the queued work writes the block into the lease.  Did a bounded device wait
+// run out?  (sticky)
+int finish(kss_lattice* L, const HostLease& lease, Status* st = nullptr);
+// The same without a status to return.
 int device_error(kss_lattice* L);
+// Evaluate the flags, tile counts, sums and counts of the current step if it had no outputs.
+int ensure_flags(kss_lattice* L);
 
 // Free a lattice's regridding workspace, if any (kss_regrid.cu).
 void regrid_release(kss_lattice* L);
