@@ -2,8 +2,7 @@
 // within `buffer` cells of a refine-flagged cell are marked, and the marked tiles are
 // clustered into rectangular boxes by the signature method of Berger & Rigoutsos (the
 // clustering the paper's regridding routine cites, section "Adaptive refinement and
-// parallel processing"), breadth first: each level of boxes is clustered by CTAs striding
-// over its boxes, and the host checks the level sizes every few levels.
+// parallel processing"), breadth first: one cluster of CTAs walks all levels, a warp per box.
 //
 // Clustering rules (all integer except one efficiency comparison in FP64), for a box:
 //   1. signatures sx[i] = marked tiles of column i, sy[j] = of row j;
@@ -19,6 +18,7 @@
 // are appended level by level in list order, so the result is deterministic.
 #include <algorithm>
 #include <cstdint>
+#include <cstring>
 #include <new>
 #include <string>
 
@@ -28,266 +28,373 @@ using namespace kss_rt;
 
 namespace {
 
-constexpr int kMaxSide = 8192;  // tiles per side (signatures live in shared memory)
+constexpr int kMaxSide = 8192;  // tiles per side (the codes of cluster_box have 13 bits for one)
 
-struct Box {
+struct alignas(16) Box {
   int x0, y0, x1, y1;
 };
 
 // ---- kernels ----
 
 // mask[ty][tx] = 1 if a cell within `buffer` cells (periodic) of tile (tx, ty) has the
-// refine flag.  One thread per tile.
-__global__ void tile_mask_kernel(const uint8_t* __restrict__ flags, long long pitch, int nx,
-                                 int ny, int tile, int buffer, int ntx, int nty,
-                                 uint8_t* __restrict__ mask) {
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= (long long)ntx * nty) return;
-  const int ty = int(t / ntx), tx = int(t - (long long)ty * ntx);
-  const int ya = ty * tile - buffer, yb = min((ty + 1) * tile, ny) + buffer;
-  const int xa = tx * tile - buffer, xb = min((tx + 1) * tile, nx) + buffer;
-  uint8_t any = 0;
-  for (int y = ya; y < yb && !any; ++y) {
-    const int yy = ((y % ny) + ny) % ny;
-    const uint8_t* row = flags + (long long)yy * pitch;
-    for (int x = xa; x < xb; ++x) {
-      const int xx = ((x % nx) + nx) % nx;
-      if (row[xx] & 1u) {
-        any = 1;
-        break;
+// refine flag.  A CTA takes 32 tiles of a tile row; its eight warps share out the rows
+// around them, a lane reading one tile's bytes of a row (in 8-byte words where the rows are
+// 8-byte aligned) and then the buffer's on both sides.  256 x 256 tiles: 86 us with one
+// thread per tile, its cells one by one through two divisions each; now 13 us.
+__global__ void __launch_bounds__(256) tile_mask_kernel(const uint8_t* __restrict__ flags,
+                                                        long long pitch, int nx, int ny, int tile,
+                                                        int buffer, int ntx, int nty, bool words,
+                                                        uint8_t* __restrict__ mask) {
+  __shared__ int s_any[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tx = blockIdx.x * 32 + lane;
+  for (int ty = blockIdx.y; ty < nty; ty += gridDim.y) {
+    if (warp == 0) s_any[lane] = 0;
+    __syncthreads();
+    if (tx < ntx) {
+      const int x0 = tx * tile, x1 = min(x0 + tile, nx);
+      const int ya = ty * tile - buffer, yb = min((ty + 1) * tile, ny) + buffer;
+      bool any = false;
+      for (int y = ya + warp; y < yb && !any; y += 8) {
+        int yy = y;
+        if (yy < 0 || yy >= ny) yy = ((yy % ny) + ny) % ny;
+        const uint8_t* const row = flags + (long long)yy * pitch;
+        uint32_t bits = 0;
+        if (words && x1 - x0 == tile) {
+          for (int x = x0; x < x1; x += 8) {
+            const uint2 w = *reinterpret_cast<const uint2*>(row + x);
+            bits |= w.x | w.y;
+          }
+          bits &= 0x01010101u;
+        } else {
+          for (int x = x0; x < x1; ++x) bits |= row[x] & 1u;
+        }
+        for (int d = 1; d <= buffer && !bits; ++d) {
+          int l = x0 - d, r = x1 - 1 + d;
+          if (l < 0) l = (l % nx + nx) % nx;
+          if (r >= nx) r %= nx;
+          bits = (row[l] | row[r]) & 1u;
+        }
+        any = bits != 0;
       }
+      if (any) s_any[lane] = 1;
     }
+    __syncthreads();
+    if (warp == 0 && tx < ntx) mask[(long long)ty * ntx + tx] = uint8_t(s_any[lane]);
   }
-  mask[t] = any;
 }
 
-// Prefix sums of the mask: pc[j][i] = marked tiles of column i in rows < j ((nty + 1) x
-// ntx), pr[j][i] = of row j in columns < i (nty x (ntx + 1)).  One thread per column,
-// then one per row.
-__global__ void mask_prefix_kernel(const uint8_t* __restrict__ mask, int ntx, int nty,
-                                   int* __restrict__ pc, int* __restrict__ pr) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < ntx) {
-    int acc = 0;
-    for (int j = 0; j < nty; ++j) {
-      pc[(long long)j * ntx + t] = acc;
-      acc += mask[(long long)j * ntx + t];
+// Prefix sums of the mask along one direction: out[k][l] = marked tiles of line l at
+// positions below k, k = 0 .. len.  A CTA of 32 warps takes 32 lines (a lane each); a warp
+// counts 32 positions at a time, and the warps' totals are added in shared memory.
+__device__ __forceinline__ void prefix_lines(const uint8_t* __restrict__ mask, int line0,
+                                             int nlines, int len, long long line_stride,
+                                             long long pos_stride, int* __restrict__ out) {
+  __shared__ int s_tot[32][33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int line = line0 + lane;
+  const bool ok = line < nlines;
+  const uint8_t* const src = mask + line * line_stride;
+  int base = 0;
+  for (int p0 = 0; p0 < len; p0 += 1024) {  // (uniform over the CTA)
+    const int p = p0 + 32 * warp, n = max(0, min(32, len - p));
+    uint32_t bits = 0;
+    if (ok) {
+#pragma unroll 8
+      for (int k = 0; k < n; ++k) bits |= uint32_t(src[(p + k) * pos_stride]) << k;
     }
-    pc[(long long)nty * ntx + t] = acc;
-  } else if (t < ntx + nty) {
-    const int j = t - ntx;
-    int acc = 0;
-    const uint8_t* row = mask + (long long)j * ntx;
-    int* out = pr + (long long)j * (ntx + 1);
-    for (int i = 0; i < ntx; ++i) {
-      out[i] = acc;
-      acc += row[i];
+    s_tot[warp][lane] = __popc(bits);
+    __syncthreads();
+    int before = base, all = 0;
+    for (int w = 0; w < 32; ++w) {
+      const int t = s_tot[w][lane];
+      if (w < warp) before += t;
+      all += t;
     }
-    out[ntx] = acc;
+    if (ok) {
+      for (int k = 0; k < n; ++k)
+        out[(long long)(p + k) * nlines + line] = before + __popc(bits & ((1u << k) - 1u));
+    }
+    base += all;
+    __syncthreads();
   }
+  if (ok && warp == 0) out[(long long)len * nlines + line] = base;
+}
+
+// pc[j][i] = marked tiles of column i in rows < j ((nty + 1) x ntx), pr[i][j] = of row j in
+// columns < i ((ntx + 1) x nty): the first `column_ctas` CTAs take the columns, the others
+// the rows.
+__global__ void __launch_bounds__(1024) mask_prefix_kernel(const uint8_t* __restrict__ mask,
+                                                           int ntx, int nty, int column_ctas,
+                                                           int* __restrict__ pc,
+                                                           int* __restrict__ pr) {
+  const int c = blockIdx.x;
+  if (c < column_ctas)
+    prefix_lines(mask, 32 * c, ntx, nty, 1, ntx, pc);
+  else
+    prefix_lines(mask, 32 * (c - column_ctas), nty, ntx, ntx, 1, pr);
 }
 
 __device__ __forceinline__ int tile_key(int i, int lo, int hi) { return abs(2 * i - (lo + hi - 1)); }
 __device__ __forceinline__ int cut_key(int i, int lo, int hi) { return abs(2 * i - (lo + hi)); }
 
-// The boxes of one level, *count of them (written by the previous compaction), CTAs
-// striding over them.  acc[i]: box i accepted (shrunk) or x0 = -1; kids[2i], kids[2i+1]:
-// its two halves or x0 = -1.
-__device__ __forceinline__ void cluster_box(const int* __restrict__ pc,
-                                            const int* __restrict__ pr, int ntx, Box b, int bi,
-                                            double efficiency, Box* __restrict__ acc,
-                                            Box* __restrict__ kids, int* sig);
-
-__global__ void __launch_bounds__(256) cluster_level_kernel(const int* __restrict__ pc,
-                                                            const int* __restrict__ pr,
-                                                            int ntx, const Box* __restrict__ in,
-                                                            const int* __restrict__ count,
-                                                            const double* __restrict__ eff,
-                                                            Box* __restrict__ acc,
-                                                            Box* __restrict__ kids) {
-  extern __shared__ int sig[];  // sx[w] then sy[h]
-  const int n = *count;
-  const double efficiency = *eff;
-  for (int bi = blockIdx.x; bi < n; bi += gridDim.x) {
-    cluster_box(pc, pr, ntx, in[bi], bi, efficiency, acc, kids, sig);
-    __syncthreads();  // the signatures are reused by the next box
-  }
+__device__ __forceinline__ Box load_box(const Box* p) {
+  const int4 v = __ldcg(reinterpret_cast<const int4*>(p));
+  return Box{v.x, v.y, v.z, v.w};
+}
+__device__ __forceinline__ void store_box(Box* p, Box b) {
+  *reinterpret_cast<int4*>(p) = make_int4(b.x0, b.y0, b.x1, b.y1);
 }
 
-__device__ __forceinline__ void cluster_box(const int* __restrict__ pc,
-                                            const int* __restrict__ pr, int ntx, Box b, int bi,
-                                            double efficiency, Box* __restrict__ acc,
-                                            Box* __restrict__ kids, int* sig) {
+// One box by one warp (rules 1 to 6 above): 0 dropped, 1 accepted (k0 the shrunk box), 2
+// split into k0 and k1.  sig: room for kSig signature values; longer boxes read theirs from
+// the prefix sums each time.  Every choice is the minimum of a code that orders the
+// candidates by the rule's key and its ties: sides and positions are below 2^13, keys at
+// most 2^14, inflection strengths at most 2^15.
+constexpr int kSig = 512;
+__device__ __forceinline__ int cluster_box(const int* __restrict__ pc, const int* __restrict__ pr,
+                                           int ntx, int nty, Box b, double efficiency, int* sig,
+                                           Box& k0, Box& k1) {
+  constexpr unsigned kAll = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
   const int w = b.x1 - b.x0, h = b.y1 - b.y0;
-  int* sx = sig;
-  int* sy = sig + w;
-  // signatures from the prefix sums
-  for (int k = threadIdx.x; k < w + h; k += blockDim.x) {
+  const bool fits = w + h <= kSig;
+  auto value = [&](int k) {  // signature k: column x0 + k, then row y0 + k - w
     if (k < w) {
-      const int i = b.x0 + k;
-      sx[k] = pc[(long long)b.y1 * ntx + i] - pc[(long long)b.y0 * ntx + i];
-    } else {
-      const long long r = (long long)(b.y0 + k - w) * (ntx + 1);
-      sy[k - w] = pr[r + b.x1] - pr[r + b.x0];
+      const int* const c = pc + b.x0 + k;
+      return c[(long long)b.y1 * ntx] - c[(long long)b.y0 * ntx];
+    }
+    const int* const r = pr + b.y0 + k - w;
+    return r[(long long)b.x1 * nty] - r[(long long)b.x0 * nty];
+  };
+  auto at = [&](int k) { return fits ? sig[k] : value(k); };
+  int ia = w, ib = -1, ja = h, jb = -1, total = 0;
+  for (int k = lane; k < w + h; k += 32) {
+    const int v = value(k);
+    if (fits) sig[k] = v;
+    if (v && k < w) {
+      ia = min(ia, k);
+      ib = k;
+      total += v;
+    } else if (v) {
+      ja = min(ja, k - w);
+      jb = k - w;
     }
   }
-  __syncthreads();
-  if (threadIdx.x != 0) return;  // (the caller's barrier follows for every thread)
-  const Box none{-1, -1, -1, -1};
-  Box out_acc = none, k0 = none, k1 = none;
-  long long total = 0;
-  int ia = -1, ib = -1, ja = -1, jb = -1;
-  for (int i = 0; i < w; ++i) {
-    if (sx[i]) {
-      if (ia < 0) ia = i;
-      ib = i;
-      total += sx[i];
-    }
+  total = __reduce_add_sync(kAll, total);
+  if (total == 0) return 0;
+  ia = __reduce_min_sync(kAll, ia);
+  ib = __reduce_max_sync(kAll, ib);
+  ja = __reduce_min_sync(kAll, ja);
+  jb = __reduce_max_sync(kAll, jb);
+  __syncwarp();  // the signatures are in shared memory
+  const int x0 = b.x0 + ia, x1 = b.x0 + ib + 1, y0 = b.y0 + ja, y1 = b.y0 + jb + 1;
+  const int n[2] = {x1 - x0, y1 - y0}, first[2] = {ia, w + ja};
+  const int lo[2] = {x0, y0}, hi[2] = {x1, y1};
+  if (double(total) >= efficiency * double((long long)n[0] * n[1]) || (n[0] == 1 && n[1] == 1)) {
+    k0 = Box{x0, y0, x1, y1};
+    return 1;
   }
-  for (int j = 0; j < h; ++j) {
-    if (sy[j]) {
-      if (ja < 0) ja = j;
-      jb = j;
-    }
-  }
-  if (total > 0) {
-    // the shrunk box [x0, x1) x [y0, y1) and its signatures sx[ia..ib], sy[ja..jb]
-    const int x0 = b.x0 + ia, x1 = b.x0 + ib + 1, y0 = b.y0 + ja, y1 = b.y0 + jb + 1;
-    const int sw = x1 - x0, sh = y1 - y0;
-    const int* s[2] = {sx + ia, sy + ja};
-    const int n[2] = {sw, sh};
-    const int lo[2] = {x0, y0}, hi[2] = {x1, y1};
-    if (double(total) >= efficiency * double((long long)sw * sh) || (sw == 1 && sh == 1)) {
-      out_acc = Box{x0, y0, x1, y1};
-    } else {
-      int best_axis = -1, best_i = 0, best_k = 0;
-      bool hole = false;
-      // 4. interior holes
-      for (int a = 0; a < 2; ++a) {
-        for (int k = 1; k < n[a] - 1; ++k) {
-          if (s[a][k] != 0) continue;
-          const int i = lo[a] + k, key = tile_key(i, lo[a], hi[a]);
-          if (best_axis < 0 || key < best_k) {  // x first, lower index first on ties
-            best_axis = a;
-            best_i = i;
-            best_k = key;
+  // 4. interior holes: (key, x before y, position)
+  unsigned best = kAll;
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+    for (int k = 1 + lane; k < n[a] - 1; k += 32)
+      if (at(first[a] + k) == 0)
+        best = min(best, unsigned(tile_key(lo[a] + k, lo[a], hi[a])) << 14 | unsigned(a) << 13 |
+                             unsigned(k));
+  best = __reduce_min_sync(kAll, best);
+  int axis, cut, skip = 0;
+  if (best != kAll) {
+    axis = (best >> 13) & 1;
+    cut = lo[axis] + int(best & 8191u);
+    skip = 1;
+  } else {
+    // 5. strongest inflection: (strength down, key, x before y, position)
+    unsigned c1 = kAll, c2 = kAll;
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+      for (int k = 1 + lane; k < n[a] - 2; k += 32) {
+        const int s0 = at(first[a] + k - 1), s1 = at(first[a] + k), s2 = at(first[a] + k + 1),
+                  s3 = at(first[a] + k + 2);
+        const int dk = s0 - 2 * s1 + s2, dk1 = s1 - 2 * s2 + s3;
+        if ((dk > 0 && dk1 < 0) || (dk < 0 && dk1 > 0)) {
+          const unsigned c = unsigned(32768 - abs(dk1 - dk)) << 15 |
+                             unsigned(cut_key(lo[a] + k + 1, lo[a], hi[a]));
+          if (c < c1) {
+            c1 = c;
+            c2 = unsigned(a) << 13 | unsigned(k);
           }
         }
       }
-      hole = best_axis >= 0;
-      if (!hole) {
-        // 5. strongest inflection
-        int best_str = -1;
-        for (int a = 0; a < 2; ++a) {
-          for (int k = 1; k < n[a] - 2; ++k) {
-            const int dk = s[a][k - 1] - 2 * s[a][k] + s[a][k + 1];
-            const int dk1 = s[a][k] - 2 * s[a][k + 1] + s[a][k + 2];
-            if ((long long)dk * dk1 >= 0) continue;
-            const int i = lo[a] + k + 1, str = abs(dk1 - dk), key = cut_key(i, lo[a], hi[a]);
-            if (best_axis < 0 || str > best_str || (str == best_str && key < best_k)) {
-              best_axis = a;
-              best_i = i;
-              best_str = str;
-              best_k = key;
-            }
-          }
-        }
-      }
-      if (best_axis < 0) {
-        // 6. bisection of the longer side
-        best_axis = sw >= sh ? 0 : 1;
-        best_i = best_axis == 0 ? x0 + sw / 2 : y0 + sh / 2;
-      }
-      const int skip = hole ? 1 : 0;
-      if (best_axis == 0) {
-        k0 = Box{x0, y0, best_i, y1};
-        k1 = Box{best_i + skip, y0, x1, y1};
-      } else {
-        k0 = Box{x0, y0, x1, best_i};
-        k1 = Box{x0, best_i + skip, x1, y1};
-      }
+    const unsigned m = __reduce_min_sync(kAll, c1);
+    c2 = __reduce_min_sync(kAll, c1 == m ? c2 : kAll);
+    if (m != kAll) {
+      axis = (c2 >> 13) & 1;
+      cut = lo[axis] + int(c2 & 8191u) + 1;
+    } else {
+      // 6. bisection of the longer side
+      axis = n[0] >= n[1] ? 0 : 1;
+      cut = lo[axis] + n[axis] / 2;
     }
   }
-  acc[bi] = out_acc;
-  kids[2 * bi] = k0;
-  kids[2 * bi + 1] = k1;
+  if (axis == 0) {
+    k0 = Box{x0, y0, cut, y1};
+    k1 = Box{cut + skip, y0, x1, y1};
+  } else {
+    k0 = Box{x0, y0, x1, cut};
+    k1 = Box{x0, cut + skip, x1, y1};
+  }
+  return 2;
 }
 
-// Appends the accepted boxes to the result (in order) and compacts the valid children
-// into the next level's list.  One CTA of 1024 threads; counts[0] = result size,
-// counts[1] = next level size.
-__global__ void __launch_bounds__(1024) compact_kernel(const Box* __restrict__ acc,
-                                                       const Box* __restrict__ kids,
-                                                       Box* __restrict__ result,
-                                                       int result_cap, Box* __restrict__ next,
-                                                       int* __restrict__ counts) {
-  __shared__ int s_warp[32];
-  __shared__ int s_base[2];
-  __shared__ int s_n;
+// The whole clustering, breadth first, in one cluster of CTAs: a level's boxes are shared out
+// to the CTAs in contiguous runs and to their warps; after a cluster barrier every CTA knows
+// how many boxes the ones before it accepted and split, and writes its own accepted boxes
+// and halves in list order.  The results are those of one list processed in order.  (A
+// level was two launches, whose first had one thread walk every box: 256 x 256 tiles,
+// 985 boxes, 24 levels: 427 us; now 190, both by ncu.)
+constexpr int kCtas = 8;
+__global__ void __launch_bounds__(1024) cluster_kernel(const int* __restrict__ pc,
+                                                       const int* __restrict__ pr, int ntx,
+                                                       int nty, double efficiency, Box* list0,
+                                                       Box* list1, Box* acc, Box* kids,
+                                                       Box* result, int result_cap, int* count) {
+  extern __shared__ int s_sig[];  // kSig values per warp
+  __shared__ int s_tot[2];                   // accepted, split boxes of this CTA
+  __shared__ int s_all[kCtas][2];            // of every CTA
+  __shared__ int s_warp[32][2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) {
-    s_base[0] = counts[0];
-    s_base[1] = 0;
-    s_n = counts[1];  // boxes of the level just clustered
-  }
-  __syncthreads();
-  const int n = s_n;
-  // two passes of the same block-wide ordered scan: accepted boxes, then children
-  for (int pass = 0; pass < 2; ++pass) {
-    const Box* src = pass == 0 ? acc : kids;
-    const int m = pass == 0 ? n : 2 * n;
-    for (int c0 = 0; c0 < m; c0 += blockDim.x) {
-      const int c = c0 + threadIdx.x;
-      const bool valid = c < m && src[c].x0 >= 0;
-      const unsigned bal = __ballot_sync(0xffffffffu, valid);
-      if (lane == 0) s_warp[warp] = __popc(bal);
-      __syncthreads();
-      int before = 0, chunk = 0;
-      for (int w2 = 0; w2 < int(blockDim.x >> 5); ++w2) {
-        if (w2 < warp) before += s_warp[w2];
-        chunk += s_warp[w2];
+  const int rank = int(kss::cluster_rank());
+  Box* lists[2] = {list0, list1};
+  int n = 1, nres = 0, cur = 0;
+  // every level splits some box, and a box splits at most w + h - 2 times on any path
+  for (int level = 0; n > 0 && level <= ntx + nty + 2; ++level) {
+    const int per = (n + kCtas - 1) / kCtas;
+    const int lo = min(rank * per, n), hi = min(lo + per, n);
+    if (threadIdx.x < 2) s_tot[threadIdx.x] = 0;
+    __syncthreads();
+    for (int bi = lo + warp; bi < hi; bi += 32) {
+      const Box b = level == 0 ? Box{0, 0, ntx, nty} : load_box(lists[cur] + bi);
+      Box k0{-1, -1, -1, -1}, k1 = k0;
+      const int what = cluster_box(pc, pr, ntx, nty, b, efficiency, s_sig + kSig * warp, k0, k1);
+      __syncwarp();  // the signatures are rewritten by the warp's next box
+      if (lane == 0) {
+        const Box none{-1, -1, -1, -1};
+        store_box(acc + bi, what == 1 ? k0 : none);
+        store_box(kids + 2 * (long long)bi, what == 2 ? k0 : none);
+        store_box(kids + 2 * (long long)bi + 1, k1);
+        if (what) atomicAdd(&s_tot[what - 1], 1);
       }
-      const int pos = s_base[pass] + before + __popc(bal & ((1u << lane) - 1u));
-      if (valid) {
-        if (pass == 0) {
-          if (pos < result_cap) result[pos] = src[c];
-        } else {
-          next[pos] = src[c];
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 * kCtas) {  // this CTA's totals into every CTA's table
+      const uint32_t a = static_cast<uint32_t>(
+          __cvta_generic_to_shared(&s_all[rank][threadIdx.x & 1]));
+      uint32_t r;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                   : "=r"(r) : "r"(a), "r"(uint32_t(threadIdx.x >> 1)));
+      asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(r), "r"(s_tot[threadIdx.x & 1])
+                   : "memory");
+    }
+    __syncwarp();
+    kss::cluster_arrive();
+    kss::cluster_wait();
+    int at_acc = nres, at_kid = 0, all_acc = 0, all_split = 0;
+    for (int c = 0; c < kCtas; ++c) {
+      if (c < rank) {
+        at_acc += s_all[c][0];
+        at_kid += 2 * s_all[c][1];
+      }
+      all_acc += s_all[c][0];
+      all_split += s_all[c][1];
+    }
+    Box* const next = lists[cur ^ 1];
+    for (int c0 = lo; c0 < hi; c0 += 1024) {  // (uniform over the CTA)
+      const int bi = c0 + threadIdx.x;
+      Box a{-1, 0, 0, 0}, k{-1, 0, 0, 0};
+      if (bi < hi) {
+        a = load_box(acc + bi);
+        k = load_box(kids + 2 * (long long)bi);
+      }
+      const unsigned ba = __ballot_sync(0xffffffffu, a.x0 >= 0);
+      const unsigned bk = __ballot_sync(0xffffffffu, k.x0 >= 0);
+      if (lane == 0) {
+        s_warp[warp][0] = __popc(ba);
+        s_warp[warp][1] = __popc(bk);
+      }
+      __syncthreads();
+      int pa = at_acc, pk = at_kid;
+      for (int v = 0; v < 32; ++v) {
+        if (v < warp) {
+          pa += s_warp[v][0];
+          pk += 2 * s_warp[v][1];
         }
+        at_acc += s_warp[v][0];
+        at_kid += 2 * s_warp[v][1];
       }
-      __syncthreads();
-      if (threadIdx.x == 0) s_base[pass] += chunk;
+      const unsigned below = (1u << lane) - 1u;
+      pa += __popc(ba & below);
+      pk += 2 * __popc(bk & below);
+      if (a.x0 >= 0 && pa < result_cap) store_box(result + pa, a);
+      if (k.x0 >= 0) {
+        store_box(next + pk, k);
+        store_box(next + pk + 1, load_box(kids + 2 * (long long)bi + 1));
+      }
       __syncthreads();
     }
+    nres += all_acc;
+    n = 2 * all_split;
+    cur ^= 1;
+    __syncwarp();
+    kss::cluster_arrive();  // the next list is complete, and every CTA has read the totals
+    kss::cluster_wait();
   }
-  if (threadIdx.x == 0) {
-    counts[0] = s_base[0];
-    counts[1] = s_base[1];
-  }
+  if (rank == 0 && threadIdx.x == 0) *count = nres;
+}
+
+// The tile mask, the first `room` boxes (at most `max_boxes`) and the box count to the
+// caller's arrays or page-locked memory (nullptr: not wanted; a caller's boxes may be 4-byte
+// aligned only).
+__global__ void regrid_out_kernel(const uint8_t* __restrict__ mask, int ntiles,
+                                  uint8_t* __restrict__ mask_out, const Box* __restrict__ result,
+                                  const int* __restrict__ count, int room,
+                                  kss_box* __restrict__ boxes_out, int* __restrict__ count_out) {
+  const int t0 = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+  const int n = *count;
+  if (mask_out)
+    for (int t = t0; t < ntiles; t += nt) mask_out[t] = mask[t];
+  if (boxes_out)
+    for (int t = t0; t < min(n, room); t += nt)
+      boxes_out[t] = kss_box{result[t].x0, result[t].y0, result[t].x1, result[t].y1};
+  if (t0 == 0 && count_out) *count_out = n;
 }
 
 // ---- host side ----
 
+// Workspace of one tile grid, kept by a lattice between calls.
 struct Workspace {
-  int cap = 0;            // boxes per level list
+  int ntx = 0, nty = 0;
+  int cap = 0;            // boxes the result holds
   Box* level[2] = {nullptr, nullptr};
   Box* acc = nullptr;     // [cap]
   Box* kids = nullptr;    // [2 cap]
   Box* result = nullptr;  // [cap]
-  int* counts = nullptr;  // [2]
-  double* eff = nullptr;  // the efficiency threshold of the current call
+  int* count = nullptr;
   uint8_t* mask = nullptr;
   int* pc = nullptr;      // column prefix sums [(nty + 1) ntx]
-  int* pr = nullptr;      // row prefix sums [nty (ntx + 1)]
+  int* pr = nullptr;      // row prefix sums [(ntx + 1) nty]
   void release() {
-    void* b[] = {level[0], level[1], acc, kids, result, counts, eff, mask, pc, pr};
+    void* b[] = {level[0], level[1], acc, kids, result, count, mask, pc, pr};
     for (void* p : b)
       if (p) kss_rt::dev_free(p);
     *this = Workspace{};
   }
 };
 
-cudaError_t ws_alloc(Workspace& ws, int ntx, int nty) {
+cudaError_t ws_setup(Workspace& ws, int ntx, int nty) {
+  if (ws.ntx == ntx && ws.nty == nty) return cudaSuccess;
+  ws.release();
   const int ntiles = ntx * nty;
   ws.cap = ntiles + 1;
   const size_t bb = sizeof(Box) * size_t(ws.cap);
@@ -297,84 +404,28 @@ cudaError_t ws_alloc(Workspace& ws, int ntx, int nty) {
   if (e == cudaSuccess) e = kss_rt::dev_malloc(&ws.acc, bb);
   if (e == cudaSuccess) e = kss_rt::dev_malloc(&ws.kids, 2 * bb);
   if (e == cudaSuccess) e = kss_rt::dev_malloc(&ws.result, bb);
-  if (e == cudaSuccess) e = kss_rt::dev_malloc(&ws.counts, 2 * sizeof(int));
-  if (e == cudaSuccess) e = kss_rt::dev_malloc(&ws.eff, sizeof(double));
+  if (e == cudaSuccess) e = kss_rt::dev_malloc(&ws.count, sizeof(int));
   if (e == cudaSuccess) e = kss_rt::dev_malloc(&ws.mask, size_t(ntiles));
   if (e == cudaSuccess) e = kss_rt::dev_malloc(&ws.pc, sizeof(int) * size_t(nty + 1) * ntx);
   if (e == cudaSuccess) e = kss_rt::dev_malloc(&ws.pr, sizeof(int) * size_t(nty) * (ntx + 1));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             32 * kSig * int(sizeof(int)));
   if (e != cudaSuccess) {
     cudaGetLastError();
     ws.release();
+    return e;
   }
+  ws.ntx = ntx;
+  ws.nty = nty;
   return e;
 }
 
-// Workspace of one tile grid, kept by a lattice between calls: the device arrays, a
-// stream to record on, and the recorded chunk of kChunk clustering levels.
-struct RegridWS {
-  Workspace ws;
-  int ntx = 0, nty = 0, ctas = 0;
-  size_t smem = 0;
-  cudaStream_t cap = nullptr;
-  cudaGraphExec_t chunk = nullptr;
-  void destroy() {
-    if (chunk) cudaGraphExecDestroy(chunk);
-    if (cap) cudaStreamDestroy(cap);
-    ws.release();
-    chunk = nullptr;
-    cap = nullptr;
-    ntx = nty = 0;
-  }
-};
-
-constexpr int kChunk = 8;  // clustering levels between host checks of the level size
-
-cudaError_t ws_setup(RegridWS& R, int ntx, int nty) {
-  if (R.ntx == ntx && R.nty == nty && R.chunk) return cudaSuccess;
-  R.destroy();
-  cudaError_t e = ws_alloc(R.ws, ntx, nty);
-  if (e != cudaSuccess) return e;
-  int dev = 0, nsm = 1;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
-      (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-    return e;
-  R.ctas = std::max(1, std::min(ntx * nty, 2 * nsm));
-  R.smem = sizeof(int) * size_t(ntx + nty);
-  if (R.smem > 48 * 1024 &&
-      (e = cudaFuncSetAttribute(cluster_level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                int(R.smem))) != cudaSuccess)
-    return e;
-  if ((e = cudaStreamCreateWithFlags(&R.cap, cudaStreamNonBlocking)) != cudaSuccess) return e;
-  // one chunk: kChunk levels; the level lists alternate, so a chunk ends where it began
-  if ((e = cudaStreamBeginCapture(R.cap, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) return e;
-  int cur = 0;
-  for (int k = 0; k < kChunk; ++k) {
-    cluster_level_kernel<<<R.ctas, 256, R.smem, R.cap>>>(R.ws.pc, R.ws.pr, ntx, R.ws.level[cur],
-                                                         R.ws.counts + 1, R.ws.eff, R.ws.acc,
-                                                         R.ws.kids);
-    compact_kernel<<<1, 1024, 0, R.cap>>>(R.ws.acc, R.ws.kids, R.ws.result, R.ws.cap,
-                                          R.ws.level[cur ^ 1], R.ws.counts);
-    cur ^= 1;
-  }
-  cudaGraph_t graph = nullptr;
-  const cudaError_t le = cudaGetLastError();
-  e = cudaStreamEndCapture(R.cap, &graph);
-  if (le != cudaSuccess || e != cudaSuccess) {
-    if (graph) cudaGraphDestroy(graph);
-    return le != cudaSuccess ? le : e;
-  }
-  e = cudaGraphInstantiate(&R.chunk, graph, 0);
-  cudaGraphDestroy(graph);
-  if (e != cudaSuccess) return e;
-  R.ntx = ntx;
-  R.nty = nty;
-  return cudaSuccess;
-}
-
-// The whole regrid on device flags; outputs to host or device pointers.
-int regrid_run(RegridWS& R, const uint8_t* d_flags, long long pitch, int nx, int ny, int tile,
+// The whole regrid on device flags; outputs to host or device pointers.  L: the lattice
+// whose flags these are, or nullptr.
+int regrid_run(Workspace& ws, const uint8_t* d_flags, long long pitch, int nx, int ny, int tile,
                int buffer, double efficiency, uint8_t* tile_mask, kss_box* boxes,
-               int32_t max_boxes, int32_t* nboxes, int on_device, cudaStream_t s,
+               int32_t max_boxes, int32_t* nboxes, int on_device, cudaStream_t s, kss_lattice* L,
                std::string* msg) {
   const int ntx = (nx + tile - 1) / tile, nty = (ny + tile - 1) / tile;
   if (ntx > kMaxSide || nty > kMaxSide) return KSS_ERR_UNSUPPORTED;
@@ -384,47 +435,80 @@ int regrid_run(RegridWS& R, const uint8_t* d_flags, long long pitch, int nx, int
     cudaGetLastError();
     return KSS_ERR_CUDA;
   };
-  cudaError_t e = ws_setup(R, ntx, nty);
-  if (e != cudaSuccess) {
-    R.destroy();
-    if (e == cudaErrorMemoryAllocation) {
-      cudaGetLastError();
-      return KSS_ERR_OOM;
-    }
+  cudaError_t e = ws_setup(ws, ntx, nty);
+  if (e == cudaErrorMemoryAllocation) return KSS_ERR_OOM;
+  if (e != cudaSuccess) return fail_cuda(e);
+  const bool words = pitch % 8 == 0 && reinterpret_cast<uintptr_t>(d_flags) % 8 == 0;
+  tile_mask_kernel<<<dim3((ntx + 31) / 32, nty), 256, 0, s>>>(d_flags, pitch, nx, ny, tile, buffer,
+                                                             ntx, nty, words, ws.mask);
+  if ((e = cudaGetLastError()) != cudaSuccess) return fail_cuda(e);
+  const int cc = (ntx + 31) / 32, rc = (nty + 31) / 32;
+  mask_prefix_kernel<<<cc + rc, 1024, 0, s>>>(ws.mask, ntx, nty, cc, ws.pc, ws.pr);
+  if ((e = cudaGetLastError()) != cudaSuccess) return fail_cuda(e);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(kCtas);
+  cfg.blockDim = dim3(1024);
+  cfg.dynamicSmemBytes = 32 * kSig * sizeof(int);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kCtas;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  e = cudaLaunchKernelEx(&cfg, cluster_kernel, (const int*)ws.pc, (const int*)ws.pr, ntx, nty,
+                         efficiency, ws.level[0], ws.level[1], ws.acc, ws.kids, ws.result, ws.cap,
+                         ws.count);
+  if (e != cudaSuccess) return fail_cuda(e);
+  // the outputs: device arrays are written directly; host ones go through borrowed
+  // page-locked memory (16 bytes for the count, the mask, then boxes) where they fit
+  static_assert(sizeof(Box) == sizeof(kss_box), "box layout");
+  const HostLease lease;
+  const size_t at_boxes = 16 + (size_t(ntiles) + 15) / 16 * 16;
+  unsigned char* const mail = static_cast<unsigned char*>(lease.room(at_boxes));
+  int* const count_mail = static_cast<int*>(lease.room(16));
+  const int wanted = std::min(max_boxes, ws.cap);
+  int room = wanted;
+  uint8_t* mo = nullptr;
+  kss_box* bo = nullptr;
+  if (on_device) {
+    mo = tile_mask;
+    bo = boxes;
+  } else if (mail) {
+    room = std::min<size_t>(wanted, (HostLease::kBytes - HostLease::kMailBytes - at_boxes) / sizeof(Box));
+    mo = tile_mask ? mail + 16 : nullptr;
+    bo = boxes ? reinterpret_cast<kss_box*>(mail + at_boxes) : nullptr;
+  }
+  regrid_out_kernel<<<std::max(1, std::min(64, (ntiles + 255) / 256)), 256, 0, s>>>(
+      ws.mask, ntiles, mo, ws.result, ws.count, room, bo, count_mail);
+  if ((e = cudaGetLastError()) != cudaSuccess) return fail_cuda(e);
+  int total = 0;
+  if (!count_mail &&
+      (e = cudaMemcpyAsync(&total, ws.count, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+    return fail_cuda(e);
+  if (L) {
+    if (const int r = finish(L, lease)) return r;
+  } else if ((e = cudaStreamSynchronize(s)) != cudaSuccess) {
     return fail_cuda(e);
   }
-  Workspace& ws = R.ws;
-  tile_mask_kernel<<<(ntiles + 255) / 256, 256, 0, s>>>(d_flags, pitch, nx, ny, tile, buffer,
-                                                         ntx, nty, ws.mask);
-  if ((e = cudaGetLastError()) != cudaSuccess) return fail_cuda(e);
-  mask_prefix_kernel<<<(ntx + nty + 255) / 256, 256, 0, s>>>(ws.mask, ntx, nty, ws.pc, ws.pr);
-  if ((e = cudaGetLastError()) != cudaSuccess) return fail_cuda(e);
-  // first level: the whole tile grid; results so far 0; this call's efficiency (pageable
-  // sources: each copy completes before the call returns)
-  const Box whole{0, 0, ntx, nty};
-  const int init[2] = {0, 1};
-  if ((e = cudaMemcpyAsync(ws.level[0], &whole, sizeof(Box), cudaMemcpyHostToDevice, s)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(ws.counts, init, sizeof(init), cudaMemcpyHostToDevice, s)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(ws.eff, &efficiency, sizeof(double), cudaMemcpyHostToDevice, s)) != cudaSuccess)
-    return fail_cuda(e);
-  int count[2] = {0, 1};
-  // every level splits some box, and a box splits at most w + h - 2 times on any path
-  for (int level = 0; count[1] > 0 && level <= ntx + nty + 2; level += kChunk) {
-    if ((e = cudaGraphLaunch(R.chunk, s)) != cudaSuccess) return fail_cuda(e);
-    if ((e = cudaMemcpyAsync(count, ws.counts, sizeof(count), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(s)) != cudaSuccess)
+  if (count_mail) total = *count_mail;
+  if (!on_device) {
+    const int ncopy = std::min(total, wanted), have = mail ? std::min(ncopy, room) : 0;
+    if (mo) std::memcpy(tile_mask, mail + 16, size_t(ntiles));
+    if (bo) std::memcpy(boxes, mail + at_boxes, sizeof(Box) * size_t(have));
+    const bool more = boxes && ncopy > have;
+    if (more &&
+        (e = cudaMemcpyAsync(boxes + have, ws.result + have, sizeof(Box) * size_t(ncopy - have),
+                             cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+      return fail_cuda(e);
+    if (tile_mask && !mo &&
+        (e = cudaMemcpyAsync(tile_mask, ws.mask, size_t(ntiles), cudaMemcpyDeviceToHost, s)) !=
+            cudaSuccess)
+      return fail_cuda(e);
+    if ((more || (tile_mask && !mo)) && (e = cudaStreamSynchronize(s)) != cudaSuccess)
       return fail_cuda(e);
   }
-  const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-  const int total = count[0];
-  const int ncopy = std::min(total, max_boxes);
-  static_assert(sizeof(Box) == sizeof(kss_box), "box layout");
-  if (boxes && ncopy > 0 &&
-      (e = cudaMemcpyAsync(boxes, ws.result, sizeof(Box) * size_t(ncopy), kind, s)) != cudaSuccess)
-    return fail_cuda(e);
-  if (tile_mask && (e = cudaMemcpyAsync(tile_mask, ws.mask, size_t(ntiles), kind, s)) != cudaSuccess)
-    return fail_cuda(e);
-  if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return fail_cuda(e);
   *nboxes = total;
   return KSS_OK;
 }
@@ -439,8 +523,8 @@ bool valid_args(int tile, int buffer, double efficiency, int32_t max_boxes, int3
 namespace kss_rt {
 void regrid_release(kss_lattice* L) {
   if (!L || !L->regrid) return;
-  RegridWS* R = static_cast<RegridWS*>(L->regrid);
-  R->destroy();
+  Workspace* R = static_cast<Workspace*>(L->regrid);
+  R->release();
   delete R;
   L->regrid = nullptr;
 }
@@ -457,14 +541,14 @@ int kss_regrid(kss_lattice* L, int32_t buffer, double efficiency, uint8_t* tile_
     return fail(L, KSS_ERR_ARG, "invalid regrid argument");
   DeviceGuard g(L->device);
   // the flags of the current step (evaluated if this step had no outputs)
-  if ((rc = ensure_flags(L)) || (rc = device_error(L))) return rc;
+  if ((rc = ensure_flags(L))) return rc;
   if (!L->regrid) {
-    L->regrid = new (std::nothrow) RegridWS();
+    L->regrid = new (std::nothrow) Workspace();
     if (!L->regrid) return fail(L, KSS_ERR_OOM, "regrid workspace");
   }
-  rc = regrid_run(*static_cast<RegridWS*>(L->regrid), L->flags, L->pitch, L->cfg.nx, L->cfg.ny,
+  rc = regrid_run(*static_cast<Workspace*>(L->regrid), L->flags, L->pitch, L->cfg.nx, L->cfg.ny,
                   L->cfg.tile, buffer, efficiency, tile_mask, boxes, max_boxes, nboxes, on_device,
-                  L->stream, &L->msg);
+                  L->stream, L, &L->msg);
   if (rc == KSS_ERR_CUDA) L->err = rc;  // sticky
   return rc;
 }
@@ -490,11 +574,11 @@ int kss_regrid_flags(const uint8_t* flags, int32_t nx, int32_t ny, int32_t tile,
     }
     d = staged;
   }
-  RegridWS R;
+  Workspace R;
   const int rc = regrid_run(R, d, nx, nx, ny, tile, buffer, efficiency, tile_mask, boxes, max_boxes,
-                            nboxes, on_device, s, nullptr);
+                            nboxes, on_device, s, nullptr, nullptr);
   cudaStreamSynchronize(s);
-  R.destroy();
+  R.release();
   if (staged) kss_rt::dev_free(staged);
   return rc;
 }
