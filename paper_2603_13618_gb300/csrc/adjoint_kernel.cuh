@@ -59,7 +59,7 @@ struct AdjParams {
 
 // Nine populations of V cells of row j pulled from src: forward (REV = false)
 // v_q(i, j) = src_q(i - cx_q, j - cy_q); reverse v_q(i, j) = src_q(i + cx_q, j + cy_q).
-template <class T, bool REV, bool CG = false>
+template <class T, bool REV>
 __device__ __forceinline__ void adj_pull_row(const T* src, long long plane, int pitch, int nx,
                                              int ny, int j, int i0, int lane, bool cv,
                                              T (&v)[9][kAdjV]) {
@@ -79,16 +79,16 @@ __device__ __forceinline__ void adj_pull_row(const T* src, long long plane, int 
                    base + 7 * plane + rm,
                    base + 8 * plane + rm};
 #pragma unroll
-  for (int q = 0; q < 9; ++q) vload<T, V, CG>(r[q] + i0, cv, v[q]);
+  for (int q = 0; q < 9; ++q) vload<T, V>(r[q] + i0, cv, v[q]);
   // cx = +1 planes (1, 5, 8) take column i - 1 forward, i + 1 in reverse; cx = -1
   // planes (3, 6, 7) the opposite
   if (!REV) {
-    const T h1 = load_left_halo<T, CG>(r[1], i0, nx, lane, cv);
-    const T h5 = load_left_halo<T, CG>(r[5], i0, nx, lane, cv);
-    const T h8 = load_left_halo<T, CG>(r[8], i0, nx, lane, cv);
-    const T h3 = load_right_halo<T, V, CG>(r[3], i0, nx, lane, cv);
-    const T h6 = load_right_halo<T, V, CG>(r[6], i0, nx, lane, cv);
-    const T h7 = load_right_halo<T, V, CG>(r[7], i0, nx, lane, cv);
+    const T h1 = load_left_halo<T>(r[1], i0, nx, lane, cv);
+    const T h5 = load_left_halo<T>(r[5], i0, nx, lane, cv);
+    const T h8 = load_left_halo<T>(r[8], i0, nx, lane, cv);
+    const T h3 = load_right_halo<T, V>(r[3], i0, nx, lane, cv);
+    const T h6 = load_right_halo<T, V>(r[6], i0, nx, lane, cv);
+    const T h7 = load_right_halo<T, V>(r[7], i0, nx, lane, cv);
     assemble_from_left<T, V>(v[1], h1, lane);
     assemble_from_left<T, V>(v[5], h5, lane);
     assemble_from_left<T, V>(v[8], h8, lane);
@@ -96,12 +96,12 @@ __device__ __forceinline__ void adj_pull_row(const T* src, long long plane, int 
     assemble_from_right<T, V>(v[6], h6, i0, nx, lane);
     assemble_from_right<T, V>(v[7], h7, i0, nx, lane);
   } else {
-    const T h3 = load_left_halo<T, CG>(r[3], i0, nx, lane, cv);
-    const T h6 = load_left_halo<T, CG>(r[6], i0, nx, lane, cv);
-    const T h7 = load_left_halo<T, CG>(r[7], i0, nx, lane, cv);
-    const T h1 = load_right_halo<T, V, CG>(r[1], i0, nx, lane, cv);
-    const T h5 = load_right_halo<T, V, CG>(r[5], i0, nx, lane, cv);
-    const T h8 = load_right_halo<T, V, CG>(r[8], i0, nx, lane, cv);
+    const T h3 = load_left_halo<T>(r[3], i0, nx, lane, cv);
+    const T h6 = load_left_halo<T>(r[6], i0, nx, lane, cv);
+    const T h7 = load_left_halo<T>(r[7], i0, nx, lane, cv);
+    const T h1 = load_right_halo<T, V>(r[1], i0, nx, lane, cv);
+    const T h5 = load_right_halo<T, V>(r[5], i0, nx, lane, cv);
+    const T h8 = load_right_halo<T, V>(r[8], i0, nx, lane, cv);
     assemble_from_left<T, V>(v[3], h3, lane);
     assemble_from_left<T, V>(v[6], h6, lane);
     assemble_from_left<T, V>(v[7], h7, lane);
@@ -342,7 +342,7 @@ __device__ __forceinline__ void adj_step_row(const AdjParams<T>& p, int j, int i
   constexpr int cy[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
   const T om = p.omega, om1 = T(1) - p.omega;
   T l[9][V];
-  adj_pull_row<T, true, CG>(p.lam_in, p.plane, p.pitch, p.nx, p.ny, j, i0, lane, cv, l);
+  adj_pull_row<T, true>(p.lam_in, p.plane, p.pitch, p.nx, p.ny, j, i0, lane, cv, l);
   adj_pad<T>(ft, nvalid, T(1));
   adj_pad<T>(l, nvalid, T(0));
   if constexpr (KSS_ADJ_PAIRED && std::is_same<T, float>::value && V == 2) {

@@ -41,13 +41,14 @@ cudaError_t launch_step(const StepParams<T>& p, int mode, bool pull, bool store,
 
 // CTAs (ranks) that share each block of an output step or evaluation pass of `nblocks`
 // blocks of `rows` rows (step_kernel_split), or 0 where a block is one CTA's.  Blocks are
-// shared where the ranks, at one row per warp of eight, all fit on the GPU at once (two CTAs
-// of 256 threads per SM); beyond that line the cluster's barriers cost more than the idle
-// SMs.  {Kn, KL, neq} steps of the density step, unsplit / split, us: FP32 256^2 (16 blocks)
-// 15.4 / 9.2, 512^2 (64) 17.5 / 10.9, 1021x517 (136) 17.1 / 18.9, 1024^2 (256) 21.7 / 32.8;
-// FP64 64^2 (2) 322 / 24, 128^2 (8) 243 / 37, 512x256 (64) 227 / 100; FP16 512^2 (32 blocks
-// of 256 columns) 21.0 / 11.7, 1021x517 (68) 20.3 / 14.2, 1024^2 (128) 19.9 / 26.4.  All of
-// Table 1, FP32: 256^2 44.7 / 15.1, 512^2 44.1 / 19.1.
+// shared where the ranks, at one row per warp of eight (FP32 arithmetic: or two), all fit on
+// the GPU at once (two CTAs of 256 threads per SM); beyond that line the cluster's barriers
+// cost more than the idle SMs.  {Kn, KL, neq} steps of the density step, unsplit / split,
+// us: FP32 256^2 (16 blocks) 15.4 / 9.2, 512^2 (64) 17.5 / 10.9, 1021x517 (136) 17.1 / 13.5
+// (18.9 at one row per warp), 1024^2 (256) 21.7 / 32.8; FP64 64^2 (2) 322 / 24, 128^2 (8)
+// 243 / 37, 512x256 (64) 227 / 100; FP16 512^2 (32 blocks of 256 columns) 21.0 / 11.7,
+// 1021x517 (68) 20.3 / 14.2, 1024^2 (128) 19.9 / 26.4.  All of Table 1, FP32: 256^2
+// 44.7 / 15.1, 512^2 44.1 / 19.1, 768^2 46.4 / 33.0.
 template <class T>
 int split_ranks(long long nblocks, int rows);
 

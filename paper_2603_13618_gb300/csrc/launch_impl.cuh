@@ -44,6 +44,31 @@ cudaError_t allow_dynamic_smem() {
   }
 }
 
+// kernel<<<grid, threads, dyn, stream>>>(args...), launched while the stream's previous kernel
+// still runs if that one allows it (see previous_done), in clusters of `cluster` CTAs along z.
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, int dyn,
+                           cudaStream_t stream, int cluster, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(unsigned(threads));
+  cfg.dynamicSmemBytes = size_t(dyn);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 1;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = unsigned(cluster);
+  // (FP64: a split step launched into SMs that its predecessor still occupies has its
+  // clusters doubled up on the free ones; FP64 128^2 with outputs every 10 steps 7.5 -> 11.3 us)
+  const int first = std::is_same<KSS_T, double>::value ? 1 : 0;
+  cfg.attrs = attr + first;
+  cfg.numAttrs = (cluster > 1 ? 2 : 1) - first;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // Let `kernel` run in clusters of more than eight CTAs on the current device, once per
 // device (as above).
 template <auto kernel>
@@ -114,8 +139,13 @@ inline int sm_count() {
 
 template <>
 int split_ranks<KSS_T>(long long nblocks, int rows) {
-  if (nblocks * (rows / kWarps) > 2LL * sm_count()) return 0;
-  const int ranks = std::min(rows / split_rows<KSS_T>(), 16);
+  const long long slots = 2LL * sm_count();
+  int ranks = std::min(rows / split_rows<KSS_T>(), 16);
+  if (nblocks * (rows / kWarps) > slots) {
+    // (FP32 arithmetic: two rows per warp where one each would not fit)
+    if (std::is_same<KSS_T, double>::value || nblocks * (rows / (2 * kWarps)) > slots) return 0;
+    ranks /= 2;
+  }
   return ranks >= 2 && ranks * split_rows<KSS_T>() * kSplitTurns >= rows ? ranks : 0;
 }
 
@@ -128,30 +158,21 @@ cudaError_t launch_split(const StepParams<KSS_T>& p, dim3 grid, int ranks, cudaS
   cudaError_t e = allow_dynamic_smem<kern, split_smem<KSS_T, MODE, VC>(64)>();  // any height
   if (e == cudaSuccess && ranks > 8) e = allow_large_clusters<kern>();
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(grid.x, grid.y, unsigned(ranks));
-  cfg.blockDim = dim3(32 * split_warps<KSS_T>());
-  cfg.dynamicSmemBytes = dyn;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 1;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = unsigned(ranks);
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, p);
+  return launch_chained(kern, dim3(grid.x, grid.y, unsigned(ranks)), 32 * split_warps<KSS_T>(),
+                        dyn, stream, ranks, p);
 }
 
 // A plain FP64 step of a lattice whose 8-row CTAs leave SMs idle (step_plain_f64_kernel:
 // 128^2 13.0 -> 5.1 us); true if launched.
 template <bool AAR>
-bool launch_plain_f64(const StepParams<KSS_T>& p, dim3 grid, cudaStream_t stream) {
+bool launch_plain_f64(const StepParams<KSS_T>& p, dim3 grid, cudaStream_t stream,
+                      cudaError_t& e) {
   if constexpr (std::is_same<KSS_T, double>::value) {
     if (p.tile * p.bands != 8 || (long long)grid.x * grid.y >= sm_count()) return false;
     const dim3 g((p.nx + 63) / 64, (p.ny + 1) / 2);
     if (g.y > 65535) return false;
     step_plain_f64_kernel<AAR><<<g, 128, 0, stream>>>(p);
+    e = cudaGetLastError();
     return true;
   }
   return false;
@@ -161,7 +182,8 @@ template <int MODE>
 cudaError_t launch_step_mode(const StepParams<KSS_T>& p, dim3 grid, cudaStream_t stream) {
   const int nblocks = int(grid.x * grid.y);
   if constexpr (MODE == MODE_PLAIN) {
-    if (launch_plain_f64<false>(p, grid, stream)) return cudaGetLastError();
+    cudaError_t e = cudaSuccess;
+    if (launch_plain_f64<false>(p, grid, stream, e)) return e;
   }
   if constexpr (MODE != MODE_PLAIN) {
     const int rows = p.tile * p.bands;
@@ -195,8 +217,8 @@ cudaError_t launch_step_mode(const StepParams<KSS_T>& p, dim3 grid, cudaStream_t
     constexpr int dyn = step_prefetch_smem<KSS_T, MODE, true>();
     const cudaError_t e = allow_dynamic_smem<step_kernel<KSS_T, MODE, true, true, false, true>, dyn>();
     if (e != cudaSuccess) return e;
-    step_kernel<KSS_T, MODE, true, true, false, true><<<grid, kThreads, dyn, stream>>>(p);
-    return cudaGetLastError();
+    return launch_chained(step_kernel<KSS_T, MODE, true, true, false, true>, grid, kThreads, dyn,
+                          stream, 1, p);
   }
   if constexpr (std::is_same<KSS_T, __half>::value && KSS_F16_PREFETCH &&
                 step_prefetch_smem<KSS_T, MODE, true>() > 0) {
@@ -215,18 +237,21 @@ cudaError_t launch_step_mode(const StepParams<KSS_T>& p, dim3 grid, cudaStream_t
         constexpr int dyn8 = step_prefetch_smem<KSS_T, MODE, true, 8, NW>();
         const cudaError_t e = allow_dynamic_smem<kern, dyn8>();
         if (e != cudaSuccess) return e;
-        kern<<<g8, 32 * NW, dyn8, stream>>>(q);
-        return cudaGetLastError();
+        return launch_chained(kern, g8, 32 * NW, dyn8, stream, 1, q);
       }
     }
     constexpr int dyn = step_prefetch_smem<KSS_T, MODE, true>();
     const cudaError_t e = allow_dynamic_smem<step_kernel<KSS_T, MODE, true, true, false, true>, dyn>();
     if (e != cudaSuccess) return e;
-    step_kernel<KSS_T, MODE, true, true, false, true><<<grid, kThreads, dyn, stream>>>(p);
-    return cudaGetLastError();
+    return launch_chained(step_kernel<KSS_T, MODE, true, true, false, true>, grid, kThreads, dyn,
+                          stream, 1, p);
   }
-  step_kernel<KSS_T, MODE, true, true><<<grid, kThreads, 0, stream>>>(p);
-  return cudaGetLastError();
+  if constexpr (MODE == MODE_PLAIN) {
+    step_kernel<KSS_T, MODE, true, true><<<grid, kThreads, 0, stream>>>(p);
+    return cudaGetLastError();
+  } else {
+    return launch_chained(step_kernel<KSS_T, MODE, true, true>, grid, kThreads, 0, stream, 1, p);
+  }
 }
 
 template <>
@@ -271,14 +296,20 @@ cudaError_t launch_step_aar<KSS_T>(const StepParams<KSS_T>& p, int mode, cudaStr
     return mode == MODE_STD ? launch_split<MODE_STD, true, true, true, V>(p, grid, ranks, stream)
                             : launch_split<MODE_FULL, true, true, true, V>(p, grid, ranks, stream);
   }
-  if (mode == MODE_PLAIN && launch_plain_f64<true>(p, grid, stream)) return cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+  if (mode == MODE_PLAIN && launch_plain_f64<true>(p, grid, stream, e)) return e;
   switch (mode) {
-    case MODE_PLAIN: step_kernel<KSS_T, MODE_PLAIN, true, true, true><<<grid, kThreads, 0, stream>>>(p); break;
-    case MODE_STD: step_kernel<KSS_T, MODE_STD, true, true, true><<<grid, kThreads, 0, stream>>>(p); break;
-    case MODE_FULL: step_kernel<KSS_T, MODE_FULL, true, true, true><<<grid, kThreads, 0, stream>>>(p); break;
+    case MODE_PLAIN:
+      step_kernel<KSS_T, MODE_PLAIN, true, true, true><<<grid, kThreads, 0, stream>>>(p);
+      return cudaGetLastError();
+    case MODE_STD:
+      return launch_chained(step_kernel<KSS_T, MODE_STD, true, true, true>, grid, kThreads, 0,
+                            stream, 1, p);
+    case MODE_FULL:
+      return launch_chained(step_kernel<KSS_T, MODE_FULL, true, true, true>, grid, kThreads, 0,
+                            stream, 1, p);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 template <>

@@ -270,26 +270,39 @@ __device__ __forceinline__ void row_neighbours(const StepParams<S>& p, int j, lo
   dn = (long long)((hi ? 0 : j + 1) - j) * p.pitch;
 }
 
+// ---------------------------------------------------------------- launch overlap ----
+// One-step kernels with outputs are launched with programmatic stream serialization (launch_chained).
+// Each waits, before it touches memory, until the kernels before it have completed and their
+// writes are visible (previous_done: every thread of every such kernel calls it first, so
+// completion is transitive), and then lets the next kernel be launched as soon as all of its
+// own CTAs run (next_launch; only after the wait, so that no kernel starts while an older one
+// than its predecessor still runs).  What overlaps is the launch itself: 64^2 FP32 output
+// steps 10.8 -> 9.0 us in separate calls and 8.8 -> 8.4 in a graph, 2048^2 66.4 -> 64.2.
+// Plain steps gain nothing from it in graphs and are launched as usual, and so are FP64 steps
+// (launch_chained).  Without the launch attribute both functions do nothing.
+__device__ __forceinline__ void previous_done() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void next_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- loads ----
-// Population loads: through the read-only data path (CG = false; the source buffer is
-// not written during the launch), or as ordinary cached loads (CG = true: the multi-step
-// kernel, whose source buffers other CTAs write during the launch; its loads follow an
-// acquire of the writers' release, which the read-only path would not honour).
-template <bool CG, class VT>
+// Population loads: ordinary cached loads.  The read-only path would not do: in the
+// multi-step kernels other CTAs write the source buffers during the launch (loads follow an
+// acquire of the writers' release), and a chained kernel may be launched while its
+// predecessor still writes them (loads follow previous_done).
+template <class VT>
 __device__ __forceinline__ VT ld_pop(const VT* p) {
-  if constexpr (CG) {
-    return __ldca(p);
-  } else {
-    return __ldg(p);
-  }
+  return __ldca(p);
 }
 
 // V cells per thread (default: the fused step's Vec<T>::N).
-template <class T, int V = Vec<T>::N, bool CG = false>
+template <class T, int V = Vec<T>::N>
 __device__ __forceinline__ void vload(const T* p, bool ok, T (&v)[V]) {
   using VT = typename VecT<T, V>::type;
   if (ok) {
-    const VT a = ld_pop<CG>(reinterpret_cast<const VT*>(p));
+    const VT a = ld_pop(reinterpret_cast<const VT*>(p));
     if constexpr (V == 4) {
       v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
     } else {
@@ -307,17 +320,17 @@ __device__ __forceinline__ void vload(const T* p, bool ok, T (&v)[V]) {
 //
 // Halo element of a cx = +1 population (source column i - 1): lane 0 of each warp
 // needs the element left of its vector (column nx-1 at the periodic seam).
-template <class T, bool CG = false>
+template <class T>
 __device__ __forceinline__ T load_left_halo(const T* row, int i0, int nx, int lane, bool cv) {
-  return (lane == 0 && cv) ? ld_pop<CG>(row + (i0 == 0 ? nx - 1 : i0 - 1)) : T(0);
+  return (lane == 0 && cv) ? ld_pop(row + (i0 == 0 ? nx - 1 : i0 - 1)) : T(0);
 }
 
 // Halo element of a cx = -1 population (source column i + 1): lane 31, and any lane
 // whose vector reaches the row end (then the element is column 0, periodic seam).
-template <class T, int V = Vec<T>::N, bool CG = false>
+template <class T, int V = Vec<T>::N>
 __device__ __forceinline__ T load_right_halo(const T* row, int i0, int nx, int lane, bool cv) {
   const bool tail = i0 + V >= nx;
-  return (cv && (lane == 31 || tail)) ? ld_pop<CG>(row + (tail ? 0 : i0 + V)) : T(0);
+  return (cv && (lane == 31 || tail)) ? ld_pop(row + (tail ? 0 : i0 + V)) : T(0);
 }
 
 // Cells i0..i0+V-1 pulled from column i - 1: the left neighbour's last element by
@@ -453,7 +466,7 @@ __device__ __forceinline__ void vstore(T* p, const T (&v)[V]) {
 
 // Populations of plane q: V cells loaded and decoded to the arithmetic type, or encoded
 // and stored (streaming stores).  FP16 deviations move as 8- (V = 4) or 4-byte vectors.
-template <class S, int V = Vec<S>::N, bool CG = false>
+template <class S, int V = Vec<S>::N>
 __device__ __forceinline__ void pop_vload(const S* p, bool ok, arith_t<S> (&v)[V], int q,
                                           const codec_t<S>& c) {
   if constexpr (std::is_same<S, __half>::value) {
@@ -463,7 +476,7 @@ __device__ __forceinline__ void pop_vload(const S* p, bool ok, arith_t<S> (&v)[V
       return;
     }
     using VT = typename VecT<S, V>::type;
-    const VT raw = ld_pop<CG>(reinterpret_cast<const VT*>(p));
+    const VT raw = ld_pop(reinterpret_cast<const VT*>(p));
     const __half2* h = reinterpret_cast<const __half2*>(&raw);
     // two codes per paired FMA (each half rounded as fmaf rounds it)
     const F2 inv = pack2(c.inv[q], c.inv[q]), base = pack2(c.base[q], c.base[q]);
@@ -473,7 +486,7 @@ __device__ __forceinline__ void pop_vload(const S* p, bool ok, arith_t<S> (&v)[V
       unpack2(fma2(pack2(a.x, a.y), inv, base), v[2 * k], v[2 * k + 1]);
     }
   } else {
-    vload<S, V, CG>(p, ok, v);
+    vload<S, V>(p, ok, v);
   }
 }
 
@@ -745,7 +758,7 @@ struct Pick3 {
 
 // The nine populations of cell (i, j) as the step sees them (pulled when PULL), for the
 // exact recomputation of deferred cells.
-template <class S, bool PULL, bool CG = false>
+template <class S, bool PULL>
 __device__ __forceinline__ void reload_cell(const StepParams<S>& p, int i, int j,
                                             arith_t<S> (&c)[9]) {
   constexpr int cx[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
@@ -759,7 +772,7 @@ __device__ __forceinline__ void reload_cell(const StepParams<S>& p, int i, int j
       si = si < 0 ? si + p.nx : (si >= p.nx ? si - p.nx : si);
       if (!p.slab) sj = sj < 0 ? sj + p.ny : (sj >= p.ny ? sj - p.ny : sj);
     }
-    c[q] = decode<S>(ld_pop<CG>(p.src + q * p.plane + (long long)sj * p.pitch + si), q, p.codec);
+    c[q] = decode<S>(ld_pop(p.src + q * p.plane + (long long)sj * p.pitch + si), q, p.codec);
   }
 }
 
@@ -904,12 +917,12 @@ __host__ __device__ constexpr bool mode_has(int s) {
 // the pass's source buffer (which the pass does not modify) with the exact per-cell
 // arithmetic of the full sensor set (cell_update).  Returns the refine/switch/non-
 // positive tags; the tile counts are corrected here.
-template <class S, bool PULL, bool CG = false>
+template <class S, bool PULL>
 __device__ __forceinline__ uint32_t fix_cell(const StepParams<S>& p, const Pick3& pr,
                                              const Pick3& ps, int i, int j) {
   using T = arith_t<S>;
   T cell[9], dummy[9];
-  reload_cell<S, PULL, CG>(p, i, j, cell);
+  reload_cell<S, PULL>(p, i, j, cell);
   CellOut<T> co;
   cell_update<T, MODE_STD, false>(cell, p.omega, p.tau, dummy, co, p.trt);
   const T kn = co.sv[S_KN], kl = co.sv[S_KL], neq = co.sv[S_NEQ], qe = co.sv[S_QE];
@@ -1454,7 +1467,6 @@ __device__ __forceinline__ void half_rows(const StepParams<__half>& p, int j,
 // The lane's code vectors w[q] of row j and the halo codes h[q] of the populations with
 // cx = +1 (q = 1, 5, 8: column i0 - 1, periodic; lane 0) and cx = -1 (q = 3, 6, 7: column
 // i0 + 4, or 0 at the row end; lane 31 and the lanes whose vector reaches the row end).
-template <bool CG>
 __device__ __forceinline__ void gather_half_row(const StepParams<__half>& p, int j, int i0,
                                                 int lane, bool cv, uint2 (&w)[9],
                                                 uint32_t (&h)[9]) {
@@ -1462,16 +1474,16 @@ __device__ __forceinline__ void gather_half_row(const StepParams<__half>& p, int
   half_rows(p, j, r);
 #pragma unroll
   for (int q = 0; q < 9; ++q)
-    w[q] = cv ? ld_pop<CG>(reinterpret_cast<const uint2*>(r[q] + i0)) : make_uint2(0u, 0u);
+    w[q] = cv ? ld_pop(reinterpret_cast<const uint2*>(r[q] + i0)) : make_uint2(0u, 0u);
   const bool tail = i0 + 4 >= p.nx;
   const int cl = i0 == 0 ? p.nx - 1 : i0 - 1, cr = tail ? 0 : i0 + 4;
   const bool hl = lane == 0 && cv, hr = cv && (lane == 31 || tail);
-  h[1] = hl ? half_bits(ld_pop<CG>(r[1] + cl)) : 0u;
-  h[5] = hl ? half_bits(ld_pop<CG>(r[5] + cl)) : 0u;
-  h[8] = hl ? half_bits(ld_pop<CG>(r[8] + cl)) : 0u;
-  h[3] = hr ? half_bits(ld_pop<CG>(r[3] + cr)) : 0u;
-  h[6] = hr ? half_bits(ld_pop<CG>(r[6] + cr)) : 0u;
-  h[7] = hr ? half_bits(ld_pop<CG>(r[7] + cr)) : 0u;
+  h[1] = hl ? half_bits(ld_pop(r[1] + cl)) : 0u;
+  h[5] = hl ? half_bits(ld_pop(r[5] + cl)) : 0u;
+  h[8] = hl ? half_bits(ld_pop(r[8] + cl)) : 0u;
+  h[3] = hr ? half_bits(ld_pop(r[3] + cr)) : 0u;
+  h[6] = hr ? half_bits(ld_pop(r[6] + cr)) : 0u;
+  h[7] = hr ? half_bits(ld_pop(r[7] + cr)) : 0u;
 }
 
 // Pull along x and decode: w and h as gather_half_row leaves them.
@@ -1688,7 +1700,7 @@ __host__ __device__ constexpr int step_prefetch_smem() {
 // The populations of row j's V-cell vectors at column i0 after the pull (loads of the nine
 // source rows, the halo values of the cx != 0 planes, the shifts along x): the direct-load
 // path of step_block, and one row of a plain step on its own (the adjoint's recomputation).
-template <class S, bool CG>
+template <class S>
 __device__ __forceinline__ void pull_row(const StepParams<S>& p, int j, int i0, int lane,
                                          bool cv, arith_t<S> (&ft)[9][Vec<S>::N]) {
   using T = arith_t<S>;
@@ -1706,21 +1718,21 @@ __device__ __forceinline__ void pull_row(const StepParams<S>& p, int j, int i0, 
   const S* r6 = base + 6 * p.plane + up;
   const S* r7 = base + 7 * p.plane + dn;
   const S* r8 = base + 8 * p.plane + dn;
-  pop_vload<S, V, CG>(r0 + i0, cv, ft[0], 0, p.codec);
-  pop_vload<S, V, CG>(r1 + i0, cv, ft[1], 1, p.codec);
-  pop_vload<S, V, CG>(r2 + i0, cv, ft[2], 2, p.codec);
-  pop_vload<S, V, CG>(r3 + i0, cv, ft[3], 3, p.codec);
-  pop_vload<S, V, CG>(r4 + i0, cv, ft[4], 4, p.codec);
-  pop_vload<S, V, CG>(r5 + i0, cv, ft[5], 5, p.codec);
-  pop_vload<S, V, CG>(r6 + i0, cv, ft[6], 6, p.codec);
-  pop_vload<S, V, CG>(r7 + i0, cv, ft[7], 7, p.codec);
-  pop_vload<S, V, CG>(r8 + i0, cv, ft[8], 8, p.codec);
-  const T h1 = decode<S>(load_left_halo<S, CG>(r1, i0, p.nx, lane, cv), 1, p.codec);
-  const T h5 = decode<S>(load_left_halo<S, CG>(r5, i0, p.nx, lane, cv), 5, p.codec);
-  const T h8 = decode<S>(load_left_halo<S, CG>(r8, i0, p.nx, lane, cv), 8, p.codec);
-  const T h3 = decode<S>(load_right_halo<S, V, CG>(r3, i0, p.nx, lane, cv), 3, p.codec);
-  const T h6 = decode<S>(load_right_halo<S, V, CG>(r6, i0, p.nx, lane, cv), 6, p.codec);
-  const T h7 = decode<S>(load_right_halo<S, V, CG>(r7, i0, p.nx, lane, cv), 7, p.codec);
+  pop_vload<S, V>(r0 + i0, cv, ft[0], 0, p.codec);
+  pop_vload<S, V>(r1 + i0, cv, ft[1], 1, p.codec);
+  pop_vload<S, V>(r2 + i0, cv, ft[2], 2, p.codec);
+  pop_vload<S, V>(r3 + i0, cv, ft[3], 3, p.codec);
+  pop_vload<S, V>(r4 + i0, cv, ft[4], 4, p.codec);
+  pop_vload<S, V>(r5 + i0, cv, ft[5], 5, p.codec);
+  pop_vload<S, V>(r6 + i0, cv, ft[6], 6, p.codec);
+  pop_vload<S, V>(r7 + i0, cv, ft[7], 7, p.codec);
+  pop_vload<S, V>(r8 + i0, cv, ft[8], 8, p.codec);
+  const T h1 = decode<S>(load_left_halo<S>(r1, i0, p.nx, lane, cv), 1, p.codec);
+  const T h5 = decode<S>(load_left_halo<S>(r5, i0, p.nx, lane, cv), 5, p.codec);
+  const T h8 = decode<S>(load_left_halo<S>(r8, i0, p.nx, lane, cv), 8, p.codec);
+  const T h3 = decode<S>(load_right_halo<S, V>(r3, i0, p.nx, lane, cv), 3, p.codec);
+  const T h6 = decode<S>(load_right_halo<S, V>(r6, i0, p.nx, lane, cv), 6, p.codec);
+  const T h7 = decode<S>(load_right_halo<S, V>(r7, i0, p.nx, lane, cv), 7, p.codec);
   assemble_from_left<T>(ft[1], h1, lane);
   assemble_from_left<T>(ft[5], h5, lane);
   assemble_from_left<T>(ft[8], h8, lane);
@@ -1750,7 +1762,7 @@ struct FullRow {
 
 // The nine populations of cell (i, j), one cell per lane (pulled when PULL); ones where !ok
 // (finite: nothing of such a cell is stored or added).
-template <class S, bool PULL, bool CG>
+template <class S, bool PULL>
 __device__ __forceinline__ void pull_cell(const StepParams<S>& p, int i, int j, bool ok,
                                           arith_t<S> (&f)[9]) {
   constexpr int cx[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
@@ -1765,20 +1777,20 @@ __device__ __forceinline__ void pull_cell(const StepParams<S>& p, int i, int j, 
     if (ok) {
       const int col = !PULL || cx[q] == 0 ? i : (cx[q] > 0 ? l : r);
       const long long off = !PULL || cy[q] == 0 ? 0 : (cy[q] > 0 ? up : dn);
-      f[q] = decode<S>(ld_pop<CG>(src + q * p.plane + off + col), q, p.codec);
+      f[q] = decode<S>(ld_pop(src + q * p.plane + off + col), q, p.codec);
     }
   }
 }
 
 // One cell per lane of an all-sensor step: stores the new populations and the recorded
 // sensors, returns the flag byte and the moments.
-template <class S, bool PULL, bool STORE, bool AAR, bool CG>
+template <class S, bool PULL, bool STORE, bool AAR>
 __device__ __forceinline__ uint32_t full_cell(const StepParams<S>& p, int i, int j, bool ok,
                                               arith_t<S> (&m)[3]) {
   using T = arith_t<S>;
   const long long off = (long long)j * p.pitch + i;
   T f[9], fo[9];
-  pull_cell<S, PULL, CG>(p, i, j, ok, f);
+  pull_cell<S, PULL>(p, i, j, ok, f);
   // (in a batch, a member without the model has no region: it steps as BGK)
   const bool switched = AAR && STORE && ok && p.region && p.region[off];
   CellOut<T> co;
@@ -1802,7 +1814,7 @@ __device__ __forceinline__ uint32_t full_cell(const StepParams<S>& p, int i, int
   return uint32_t(rf) | (uint32_t(sw) << 1) | (uint32_t(ok && co.nonpos) << 7);
 }
 
-template <class S, bool PULL, bool STORE, bool AAR, bool CG>
+template <class S, bool PULL, bool STORE, bool AAR>
 __device__ __forceinline__ uint32_t full_row(const StepParams<S>& p, FullRow<S>& row, int c0,
                                              int j, int lane) {
   using T = arith_t<S>;
@@ -1812,7 +1824,7 @@ __device__ __forceinline__ uint32_t full_row(const StepParams<S>& p, FullRow<S>&
     const int t = 32 * c + lane;
     T m[3];
     row.flags[t] =
-        uint8_t(full_cell<S, PULL, STORE, AAR, CG>(p, c0 + t, j, c0 + t < p.nx, m));
+        uint8_t(full_cell<S, PULL, STORE, AAR>(p, c0 + t, j, c0 + t < p.nx, m));
     row.m[0][t] = m[0];
     row.m[1][t] = m[1];
     row.m[2][t] = m[2];
@@ -1857,7 +1869,7 @@ __device__ __forceinline__ void full_row_sums(const StepParams<S>& p, const Full
 // lane (the storage's vector width, or 8 for the FP16 {Kn, KL, neq} step with the row
 // prefetch, whose CTA rows are 256 columns).  NW: warps per CTA (8; the eight-cell kernel
 // may take fewer, at most 8 rows per warp).
-template <class S, int MODE, bool PULL, bool STORE, bool CG = false, bool AAR = false,
+template <class S, int MODE, bool PULL, bool STORE, bool MULTI = false, bool AAR = false,
           bool PREFETCH = false, int VC = Vec<S>::N, int NW = kWarps>
 __device__ __forceinline__ void step_block(const StepParams<S>& p, const int bx, const int by,
                                            const int gx, double* part_sum, uint32_t* part_cnt) {
@@ -1868,7 +1880,7 @@ __device__ __forceinline__ void step_block(const StepParams<S>& p, const int bx,
   // eight cells per lane: two groups of four on the paired FP16 row, staged by pf_issue_h8
   constexpr bool kH8 = VC == 8;
   static_assert(VC == V || (kH8 && std::is_same<S, __half>::value && MODE == MODE_STD &&
-                            PULL && STORE && PREFETCH && !AAR && !CG && KSS_ROW_PAIRED),
+                            PULL && STORE && PREFETCH && !AAR && !MULTI && KSS_ROW_PAIRED),
                 "eight cells per lane: the one-step FP16 {Kn, KL, neq} kernel only");
   static_assert(NW == kWarps || (kH8 && NW >= 1 && NW < kWarps), "warps per CTA");
   const int lane = threadIdx.x & 31, warp = __shfl_sync(kFull, int(threadIdx.x >> 5), 0);
@@ -1996,12 +2008,12 @@ __device__ __forceinline__ void step_block(const StepParams<S>& p, const int bx,
         __syncwarp();  // the row's reads precede the copies of the next row into the slots
         if (j + kWarps < j1) pf_issue_half(p, pwh, j + kWarps, i0, lane, cv);
       } else {
-        gather_half_row<CG>(p, j, i0, lane, cv, w, h);
+        gather_half_row(p, j, i0, lane, cv, w, h);
       }
       assemble_half_row(p, i0, lane, w, h, f);
       fbits = fused_row_paired<S, MODE, STORE>(p, f, i0, j, cv, a_rho, a_jx, a_jy);
     } else if constexpr (MODE == MODE_FULL) {
-      fbits = full_row<S, PULL, STORE, AAR, CG>(p, s_row[warp], bx * 32 * V, j, lane);
+      fbits = full_row<S, PULL, STORE, AAR>(p, s_row[warp], bx * 32 * V, j, lane);
       full_row_sums<S>(p, s_row[warp], bx * 32 * V, lane, a_rho, a_jx, a_jy);
     } else {
     T ft[9][V];
@@ -2046,15 +2058,15 @@ __device__ __forceinline__ void step_block(const StepParams<S>& p, const int bx,
         if (cv && p.region) mbits = load_bytes<V>(p.region + (long long)j * p.pitch + i0);
       }
       if (PULL) {
-        pull_row<S, CG>(p, j, i0, lane, cv, ft);
+        pull_row<S>(p, j, i0, lane, cv, ft);
       } else {
 #pragma unroll
         for (int q = 0; q < 9; ++q)
-          pop_vload<S, V, CG>(base + q * p.plane + i0, cv, ft[q], q, p.codec);
+          pop_vload<S, V>(base + q * p.plane + i0, cv, ft[q], q, p.codec);
       }
     }
 
-    fbits = fused_row<S, MODE, PULL, STORE, AAR, CG>(p, ft, i0, j, cv, a_rho, a_jx, a_jy, mbits);
+    fbits = fused_row<S, MODE, PULL, STORE, AAR, MULTI>(p, ft, i0, j, cv, a_rho, a_jx, a_jy, mbits);
     }
     if (OUT) {
       // (with eight cells per lane, the tags of cells 4-7 moved to bits no tag of cells
@@ -2153,7 +2165,7 @@ __device__ __forceinline__ void step_block(const StepParams<S>& p, const int bx,
         const int j = j0 + rl, i = bx * 32 * VC + cl;
         if (!bounds_ok(j < j1 && i < p.nx && rl / p.tile < kMaxBands && cl / p.tile < 32, p.err))
           continue;
-        const uint32_t tags = fix_cell<S, PULL, CG>(p, pr, ps, i, j);
+        const uint32_t tags = fix_cell<S, PULL>(p, pr, ps, i, j);
         if (AAR && STORE && p.region) p.region[(long long)j * p.pitch + i] = uint8_t((tags >> 1) & 1u);
         const int b = rl / p.tile, tl = cl / p.tile;
         if (tags & 1u) {
@@ -2243,6 +2255,10 @@ template <class S, int MODE, bool PULL, bool STORE, bool AAR = false, bool PF = 
 __global__ void __launch_bounds__(32 * NW, VC == 8 ? KSS_H8_MIN_BLOCKS
                                                    : step_min_blocks<S, MODE>())
 step_kernel(const StepParams<S> p) {
+  if (MODE != MODE_PLAIN) {
+    previous_done();
+    next_launch();
+  }
   step_cta<S, MODE, PULL, STORE, AAR, PF, VC, NW>(p, blockIdx.x, blockIdx.y, gridDim.x,
                                                   gridDim.x * gridDim.y);
 }
@@ -2361,7 +2377,7 @@ __device__ __forceinline__ uint32_t fix_cell_16(const StepParams<S>& p, const Pi
       si = si < 0 ? si + p.nx : (si >= p.nx ? si - p.nx : si);
       if (!p.slab) sj = sj < 0 ? sj + p.ny : (sj >= p.ny ? sj - p.ny : sj);
     }
-    own = decode<S>(ld_pop<false>(p.src + q * p.plane + (long long)sj * p.pitch + si), q, p.codec);
+    own = decode<S>(ld_pop(p.src + q * p.plane + (long long)sj * p.pitch + si), q, p.codec);
   }
   T c[9];
 #pragma unroll
@@ -2458,6 +2474,8 @@ step_kernel_split(const StepParams<S> p) {
   if (threadIdx.x < 3) s_cx[threadIdx.x] = 0;
   __syncwarp();
   cluster_arrive();  // rank 0's counters are zero (waited for before the first push)
+  previous_done();
+  next_launch();
   const uint32_t tiles0 = in_rank0(&s_tiles[0][0][0]), cx0 = in_rank0(s_cx);
   const uint32_t val0 = in_rank0(s_val);
   auto add_tile = [&](int set, int band, int tl, uint32_t n) {
@@ -2475,14 +2493,14 @@ step_kernel_split(const StepParams<S> p) {
     T mom[3];  // (one value per lane and row)
     Acc<T> a[3], b[3];
     if constexpr (FULL && kF64) {
-      fbits = full_cell<S, PULL, STORE, AAR, false>(p, i0, j, cv, mom);
+      fbits = full_cell<S, PULL, STORE, AAR>(p, i0, j, cv, mom);
       if (cv) {
         const long long off = (long long)j * p.pitch + i0;
         store_flags<1>(p.flags + off, fbits);
         if (AAR && STORE && p.region) store_flags<1>(p.region + off, (fbits >> 1) & 1u);
       }
     } else if constexpr (FULL) {
-      fbits = full_row<S, PULL, STORE, AAR, false>(p, s_row[warp], c0, j, lane);
+      fbits = full_row<S, PULL, STORE, AAR>(p, s_row[warp], c0, j, lane);
     } else if constexpr (kH8) {
       PfWarpH8* const pw = reinterpret_cast<PfWarpH8*>(kss_dyn_smem) + warp;
       const bool tail = cv && i0 + 8 >= p.nx;
@@ -2502,7 +2520,7 @@ step_kernel_split(const StepParams<S> p) {
       F2 f[9][2];
       uint2 w[9];
       uint32_t h[9];
-      gather_half_row<false>(p, j, i0, lane, cv, w, h);
+      gather_half_row(p, j, i0, lane, cv, w, h);
       assemble_half_row(p, i0, lane, w, h, f);
       fbits = fused_row_paired<S, MODE, STORE>(p, f, i0, j, cv, a[0], a[1], a[2]);
     } else {
@@ -2513,15 +2531,15 @@ step_kernel_split(const StepParams<S> p) {
       }
       if constexpr (kF64) {
         T f[9];
-        pull_cell<S, PULL, false>(p, i0, j, cv, f);
+        pull_cell<S, PULL>(p, i0, j, cv, f);
 #pragma unroll
         for (int q = 0; q < 9; ++q) ft[q][0] = f[q];
       } else if constexpr (PULL) {
-        pull_row<S, false>(p, j, i0, lane, cv, ft);
+        pull_row<S>(p, j, i0, lane, cv, ft);
       } else {
 #pragma unroll
         for (int q = 0; q < 9; ++q)
-          pop_vload<S, V, false>(p.src + (long long)j * p.pitch + q * p.plane + i0, cv, ft[q], q,
+          pop_vload<S, V>(p.src + (long long)j * p.pitch + q * p.plane + i0, cv, ft[q], q,
                                  p.codec);
       }
       fbits = fused_row<S, MODE, PULL, STORE, AAR, false, kCells>(p, ft, i0, j, cv, a[0], a[1],
@@ -2627,7 +2645,7 @@ step_kernel_split(const StepParams<S> p) {
           tags = fix_cell_16<S, PULL>(p, pr, ps, i, j, ok);
           if (threadIdx.x & 15) continue;
         } else if (ok) {
-          tags = fix_cell<S, PULL, false>(p, pr, ps, i, j);
+          tags = fix_cell<S, PULL>(p, pr, ps, i, j);
         }
         if (!ok) continue;
         if (AAR && STORE && p.region) p.region[(long long)j * p.pitch + i] = uint8_t((tags >> 1) & 1u);
@@ -2711,7 +2729,7 @@ __global__ void __launch_bounds__(128) step_plain_f64_kernel(const StepParams<do
   if (j >= p.ny) return;
   const bool ok = i < p.nx;
   double f[9], ft[9][1];
-  pull_cell<double, true, false>(p, i, j, ok, f);
+  pull_cell<double, true>(p, i, j, ok, f);
 #pragma unroll
   for (int q = 0; q < 9; ++q) ft[q][0] = f[q];
   const uint32_t mbits = AAR && ok && p.region ? p.region[(long long)j * p.pitch + i] : 0u;
@@ -2732,7 +2750,7 @@ __global__ void __launch_bounds__(128) step_plain_f64_kernel(const StepParams<do
 // sums; the last step's are the lattice's), and a slot is reused only after its previous
 // step's sums were formed.  Every wait is bounded by a clock64 deadline, after which the
 // CTA sets bit 1 of the error word and returns (its neighbours then run out too).
-// Population loads are ordinary cached loads after an acquire (CG).
+// Population loads are ordinary cached loads after an acquire.
 struct MultiState {
   uint32_t* done;      // [nblocks] steps each block has completed (0 at launch)
   uint32_t* ticket;    // [ring] blocks of the slot's step completed (0 when free)

@@ -48,6 +48,25 @@ def test_split_steps_equal_one_cta_per_block(kss, precision, tile, nx, ny):
     batch.close()
 
 
+@pytest.mark.parametrize("precision,nx,ny,record", [
+    ("fp32", 501, 801, ("kl",)), ("fp32", 512, 800, ("kl", "s")), ("fp16dev", 1021, 805, ("kl",))])
+def test_split_steps_of_two_rows_per_warp(kss, precision, nx, ny, record):
+    """Lattices of about 100 blocks: a rank's warps take two rows each."""
+    from paper_2603_13618_gb300 import inputs
+
+    fields = inputs.smooth_jump(nx, ny, seed=6, kmax=3)
+    kw = dict(precision=precision, tau=0.6, record=record)
+    batch = kss.Batch([dict(nx=nx, ny=ny)], **kw)
+    with kss.Lattice(nx, ny, **kw) as lat:
+        for x in (lat, batch[0]):
+            x.set_fields(*fields)
+            x.step(3) if x is lat else batch.step(3)
+        for a, b in zip(_outputs(lat, precision != "fp16dev"),
+                        _outputs(batch[0], precision != "fp16dev")):
+            np.testing.assert_array_equal(a, b)
+    batch.close()
+
+
 @pytest.mark.parametrize("precision", ["fp32", "fp64", "fp16dev"])
 @pytest.mark.parametrize("record,switch,at", [(("kl",), "neq", 1e-3), (("hr", "s"), "qe", 1e-5)])
 def test_split_two_relaxation_steps(kss, precision, record, switch, at):
