@@ -332,7 +332,7 @@ def adjoint_roofline(n, N, E, ms):
     pass keeps), the N - 1 reverse steps (108 B/LUP: f read, lambda read and written), the
     objective and the projection (72 B/LUP each).  The 512^2 working set (9.4 MB per
     state) lives mostly in L2, so HBM is not the limit: the latency of each dependent
-    reverse step is (the cooperative sweep's blocks wait on their neighbours)."""
+    reverse step is."""
     peak, kind = measured_peak()
     recompute = 0
     s0 = ((N - 2) // E) * E if N >= 2 else -1
@@ -352,23 +352,19 @@ def adjoint_roofline(n, N, E, ms):
                     "of the dependent reverse steps, not by HBM"}
 
 
-def adjoint_launches(N, E, multi=True):
+def adjoint_launches(N, E):
     """Kernel launches of one gradient: the forward pass (equilibrium, N - 1 plain steps,
     the last segment's states among them, and the objective), then per segment of the
-    reverse sweep, last first: one cooperative launch of its reverse steps that also
-    recomputes the previous segment, and the ordered addition of its totals (multi); or
-    its recomputed plain steps (all but the last segment) and one launch per reverse step.
-    Then the final projection."""
+    reverse sweep, last first: its recomputed plain steps (all but the last segment), one
+    launch per reverse step, and the ordered addition of its totals.  Then the final
+    projection."""
     fwd = 1 + (N - 1) + 1
     bwd = 1
     s0 = ((N - 2) // E) * E if N >= 2 else -1
     first = True
     while s0 >= 0:
         last = min(s0 + E - 1, N - 2)
-        if multi:
-            bwd += 2
-        else:
-            bwd += (0 if first else last - s0) + (last - s0 + 1)
+        bwd += (0 if first else last - s0) + (last - s0 + 1) + 1
         first = False
         s0 -= E
     return fwd + bwd
@@ -416,8 +412,7 @@ def run_adjoint(args):
     g, gt = gradient()
 
     # the same gradient with one segment (checkpoint_every = N): the forward pass keeps every
-    # state (N x 9.4 MB in HBM), the reverse sweep is one cooperative launch and recomputes
-    # nothing; reported beside the workload's checkpoint interval, not in place of it
+    # state (N x 9.4 MB in HBM), the reverse sweep is one segment and recomputes nothing; reported beside the workload's checkpoint interval, not in place of it
     adj_all = kss.Adjoint(n, n, N, precision="fp32", checkpoint_every=N)
 
     def gradient_all():
@@ -439,8 +434,7 @@ def run_adjoint(args):
         "roofline": adjoint_roofline(n, N, E, t_adj),
         "ms_gradient": t_adj, "ms_forward_plain": t_fwd, "adjoint_over_forward": t_adj / t_fwd,
         "grad_tau": gt, "grad_rho0_norm": float(torch.linalg.vector_norm(g)),
-        "gpu_launches_per_gradient": adjoint_launches(N, E, multi=True),
-        "gpu_launches_per_gradient_one_launch_per_reverse_step": adjoint_launches(N, E, False),
+        "gpu_launches_per_gradient": adjoint_launches(N, E),
         "every_state_kept": {"checkpoint_every": N, "ms_gradient": t_all,
                              "adjoint_over_forward": t_all / t_fwd,
                              "state_bytes": 9 * 4 * cells * N,

@@ -9,7 +9,7 @@
 // C the BGK collision, J = sum W KL(S f^{N-1}).  With ft^n = S f^n the reverse sweep is
 //   lt^{N-1} = W dKL/dft (ft^{N-1})                            adj_objective_kernel
 //   l^{n+1} = S^T lt^{n+1},   lt^n = (dC/dft (ft^n))^T l^{n+1},
-//   dJ/dtau += sum_x l^{n+1} . (ft^n - f^eq(ft^n)) / tau^2      adj_step_kernel
+//   dJ/dtau += sum_x l^{n+1} . (ft^n - f^eq(ft^n)) / tau^2      adj_reverse_kernel
 //   dJ/drho0 = sum_q (S^T lt^0)_q f^eq_q(1, u0)                 adj_final_kernel
 // where S^T is the pull in the opposite direction, (S^T l)_q(x) = l_q(x + c_q).
 //
@@ -46,13 +46,14 @@ struct AdjParams {
   const double* ux0;     // u0, dense [ny][nx] (final kernel)
   const double* uy0;
   double* grad;          // dJ/drho0, dense [ny][nx] (final kernel)
-  double* part;          // per-CTA partial sums [nblocks]
+  double* part;          // partial sums: per CTA [nblocks] (objective), per warp (reverse step)
   uint32_t* done;        // CTA completion counter, 0 between launches
   double* acc;           // the launch's total is added to *acc (FP64)
   uint32_t* err;         // error word (bit 2: a debug bounds check failed)
   long long plane;
   int pitch, nx, ny;
-  int rows;              // rows per CTA (grid adj_grid(nx, ny, rows))
+  int rows;              // rows per CTA (grid adj_grid(nx, ny, rows)), or per warp of a
+                         // reverse step (grid adj_reverse_grid)
   T omega;
   T zero;                // 0, read at run time (see product2)
 };
@@ -331,9 +332,7 @@ __device__ __forceinline__ void adj_cell_pairs(const F2 (&c)[9], const F2 (&y)[9
 
 // One row j of the reverse step: lt^n from l^{n+1} = S^T lt^{n+1} (pulled here) and
 // ft^n = S f^n (pulled by the caller into ft); adds the row's l^{n+1} . f^neq to sum.
-// CG: the adjoint buffers are written by other CTAs of the same launch (the multi-step
-// reverse sweep), so they are read with ordinary cached loads.
-template <class T, bool CG>
+template <class T>
 __device__ __forceinline__ void adj_step_row(const AdjParams<T>& p, int j, int i0, int lane,
                                              bool cv, int nvalid, T (&ft)[9][kAdjV],
                                              Acc<T>& sum) {
@@ -393,267 +392,57 @@ __device__ __forceinline__ void adj_step_row(const AdjParams<T>& p, int j, int i
   }
 }
 
-// The reverse step for the block (bx, by) of the adjoint grid; returns the block's sum
-// l^{n+1} . f^neq per thread (dJ/dtau = that sum over all steps / tau^2).  PRE: the
-// warp's first row of ft^n was pulled by the caller into ft0 (the multi-step sweep issues
-// those loads before it waits for its neighbours: the forward state is not written in
-// the launch).
-template <class T, bool CG, bool PRE = false>
-__device__ __forceinline__ Acc<T> adj_step_block(const AdjParams<T>& p, int bx, int by,
-                                                 T (*ft0)[kAdjV] = nullptr) {
+// One reverse step.  A warp takes p.rows rows of 64 columns, one after the other, and writes
+// its partial of the dJ/dtau sum (l^{n+1} . f^neq; dJ/dtau = that sum over all steps / tau^2)
+// to part[]: nothing in the launch waits for another warp.  The launches of a segment are
+// chained (launch_chained): a warp pulls the forward state, which no launch of the segment
+// writes, before it waits for the previous reverse step, so that only the adjoint's own
+// loads follow that wait.  The sums are added after the segment (adj_iteration_totals).
+// FP32 takes 72 registers, so that the 4096 warps of a 512^2 step run at once (28 per SM).
+// One launch for a whole segment, whose blocks waited on their neighbours' previous step
+// through counters in memory, took 8.1 us per 512^2 step (the chain of a block's waits,
+// loads, stores, fence and release); a chained launch
+// takes 4.0.
+constexpr int kAdjWarps = 4;
+template <class T>
+__global__ void __launch_bounds__(32 * kAdjWarps, std::is_same<T, float>::value ? 7 : 4)
+adj_reverse_kernel(const AdjParams<T> p) {
   constexpr int V = kAdjV;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int i0 = (bx * 32 + lane) * V;
+  const int lane = threadIdx.x & 31, warp = __shfl_sync(kFull, int(threadIdx.x >> 5), 0);
+  const int i0 = (blockIdx.x * 32 + lane) * V;
   const bool cv = i0 < p.nx;
   const int nvalid = cv ? min(V, p.nx - i0) : 0;
-  const int j0 = by * p.rows, j1 = min(j0 + p.rows, p.ny);
+  const int w = blockIdx.y * kAdjWarps + warp;
+  const int j0 = w * p.rows;
+  const int j1 = bounds_ok(int(blockIdx.x) * 32 * V < p.pitch, p.err) ? min(j0 + p.rows, p.ny) : 0;
+  T ft[9][V];
+  if (j0 < j1) adj_pull_row<T, false>(p.f, p.plane, p.pitch, p.nx, p.ny, j0, i0, lane, cv, ft);
+  previous_done();
+  next_launch();
   Acc<T> sum;
-  if (!bounds_ok(bx >= 0 && by >= 0 && bx * 32 * V < p.pitch && j0 < p.ny, p.err)) return sum;
-  for (int j = j0 + warp; j < j1; j += kWarps) {
-    T ft[9][V];
-    if (PRE && j == j0 + warp) {
-#pragma unroll
-      for (int q = 0; q < 9; ++q)
-#pragma unroll
-        for (int k = 0; k < V; ++k) ft[q][k] = ft0[q][k];
-    } else {
-      adj_pull_row<T, false>(p.f, p.plane, p.pitch, p.nx, p.ny, j, i0, lane, cv, ft);
-    }
-    adj_step_row<T, CG>(p, j, i0, lane, cv, nvalid, ft, sum);
+  for (int j = j0; j < j1; ++j) {
+    if (j > j0) adj_pull_row<T, false>(p.f, p.plane, p.pitch, p.nx, p.ny, j, i0, lane, cv, ft);
+    adj_step_row<T>(p, j, i0, lane, cv, nvalid, ft, sum);
   }
-  return sum;
+  sum.warp_reduce();
+  if (lane == 0)
+    Red<T>::of(sum).store(p.part + (long long)w * gridDim.x + blockIdx.x);
 }
 
-template <class T>
-__global__ void __launch_bounds__(kThreads) adj_step_kernel(const AdjParams<T> p) {
-  Acc<T> sum = adj_step_block<T, false>(p, blockIdx.x, blockIdx.y);
-  adj_reduce<T>(p, sum);
-}
-
-// ---- the reverse sweep of one segment in one cooperative launch ----
-// Reverse iterations it = 0 .. nit - 1 (step k = last - it), each over the nblocks blocks of
-// the adjoint grid.  Block b of iteration it first waits until the blocks of its 3 x 3
-// neighbourhood (periodic) have completed iteration it - 1: they wrote the adjoint cells its
-// reverse pull reads, and have read the cells it overwrites (the buffers alternate).  Each
-// block's partial of the dJ/dtau sum goes to part[it][b].  After the launch,
-// adj_iteration_totals adds each iteration's partials as adj_reduce does, and the
-// iteration totals to the accumulator in iteration order, so the accumulator is that of
-// one launch per step bit for bit (and no block of the sweep waits for a counter of its
-// iteration before it takes its next item).
-//
-// The same launch recomputes the previous segment (fsteps > 0): its plain forward steps
-// t = 1 .. fsteps from the checkpoint fck into the states fseg + t (the forward step's own
-// CTA body over the forward grid, fnblocks blocks).  Those states are not read by the
-// reverse iterations of this launch (they belong to the next launch), and the reverse
-// sweep's latency-bound waits leave the SMs idle enough to take them.  Forward block fb of
-// step t waits until its 3 x 3 neighbourhood has completed step t - 1 (the rows its pull
-// reads); every state has a slot of its own, so nothing else is overwritten.
-//
-// Work items are handed out in order from an atomic counter, in rounds: round r holds the
-// reverse iteration r (if r < nit) and the forward step r + 1 (if r < fsteps).  Every item
-// waits only for items handed out before it (in its own chain), so the smallest unfinished
-// item can always proceed: no deadlock, given co-residency (the cooperative launch).  Every
-// wait is bounded (bit 1 of the error word on expiry).
-// Resident CTAs per SM requested from the register allocator for the FP32 adj_multi_kernel
-// (a build-time tuning knob; FP64 takes the registers it needs).  Measured at 512^2 with
-// the paired cell arithmetic: three (80 registers, a little spilling) 2.551 ms per
-// gradient, four (64) 2.618 ms; with the scalar arithmetic three 2.609, four 2.634-2.698,
-// two (128 registers) 3.144 and five (48 registers, 484 bytes of spills) 3.492 ms.  The
-// sweep is bound by the latency of its dependent items, so more of them in flight pays
-// more than registers, up to the point where spills lengthen each item.
-#ifndef KSS_ADJ_MULTI_MIN_BLOCKS
-#define KSS_ADJ_MULTI_MIN_BLOCKS 3
-#endif
-// Sleep between two polls of a neighbour's counter, in nanoseconds (0: poll back to back).
-#ifndef KSS_ADJ_POLL_NS
-#define KSS_ADJ_POLL_NS 64
-#endif
-// Order within a round of adj_multi_kernel's work items: the reverse iteration first (0) or
-// the forward step first (1); either order keeps each chain's items in order.
-#ifndef KSS_ADJ_FWD_FIRST
-#define KSS_ADJ_FWD_FIRST 0
-#endif
-
-template <class T>
-struct AdjMulti {
-  const T* ck;         // the segment's checkpoint state (step s0)
-  const T* seg;        // recomputed states of steps s0 + 1 .. last, state_elems apart
-  long long state_elems;
-  const T* lam0;       // adjoint ping-pong: iteration it reads lam(lc + it), writes
-  const T* lam1;       // lam(lc + it + 1), lam(k) = lam0 for even k, lam1 for odd
-  uint32_t* done;      // [nblocks] iterations each block completed (0 at launch)
-  uint32_t* ticket;    // adj_iteration_totals' block counter (0 at launch)
-  uint32_t* work;      // next work item (0 at launch)
-  double* part;        // [nit][nblocks]
-  double* totals;      // [nit]
-  uint32_t* err;       // bit 1: a wait ran out
-  long long deadline;  // clock64 cycles one wait may take
-  int s0, last, lc;
-  int gx, gy, nblocks;  // the adjoint grid (adj_grid): gx x gy blocks
-  // the previous segment's recomputation (fsteps = 0: none)
-  StepParams<T> fp;    // plain step parameters (src and dst are set per step)
-  const T* fck;        // its checkpoint (state 0)
-  T* fseg;             // its states 1 .. fsteps at fseg + t state_elems
-  uint32_t* fdone;     // [fnblocks] forward steps each block completed (0 at launch)
-  int fsteps;
-  int fgx, fgy, fnblocks;  // the forward step grid (step_grid)
-};
-
-// Orders this thread's earlier memory operations, and those it observed (through the
-// CTA barrier before it), before its later ones at GPU scope (a release fence).
-__device__ __forceinline__ void fence_acq_rel_gpu() {
-  asm volatile("fence.acq_rel.gpu;" ::: "memory");
-}
-
-__device__ __forceinline__ bool adj_wait_ge(const uint32_t* p, uint32_t want, uint32_t* err,
-                                            long long deadline) {
-  if (ld_acquire_u32(p) >= want) return true;
-  const long long t0 = clock64();
-  while (ld_acquire_u32(p) < want) {
-    if (clock64() - t0 > deadline) {
-      atomicOr(err, 2u);
-      return false;
-    }
-    if (KSS_ADJ_POLL_NS > 0) __nanosleep(KSS_ADJ_POLL_NS);
-  }
-  return true;
-}
-
-// Warp 0: lanes 0..8 wait (bounded) until the 3 x 3 neighbourhood of block (bx, by) of a
-// gx x gy grid has done[] >= want; lane 0 also takes the CTA's next work item.  Returns,
-// to every thread after the barrier, whether all waits succeeded.
-__device__ __forceinline__ bool adj_wait_neighbours(const uint32_t* done, int bx, int by,
-                                                    int gx, int gy, uint32_t want, bool wait,
-                                                    uint32_t* work, int* s_next, int* s_go,
-                                                    uint32_t* err, long long deadline) {
-  if (threadIdx.x < 32) {
-    const int t = threadIdx.x;
-    if (t == 0) *s_next = int(atomicAdd(work, 1u));
-    bool ok = true;
-    if (wait && t < 9) {
-      const int dy = t / 3 - 1, dx = t - 3 * (t / 3) - 1;
-      const int yy = by + dy < 0 ? gy - 1 : (by + dy == gy ? 0 : by + dy);
-      const int xx = bx + dx < 0 ? gx - 1 : (bx + dx == gx ? 0 : bx + dx);
-      ok = adj_wait_ge(done + yy * gx + xx, want, err, deadline);
-    }
-    ok = __all_sync(kFull, ok);
-    if (t == 0) *s_go = ok;
-  }
-  __syncthreads();
-  return *s_go != 0;
-}
-
-template <class T>
-__global__ void __launch_bounds__(kThreads,
-                                  std::is_same<T, float>::value ? KSS_ADJ_MULTI_MIN_BLOCKS : 1)
-adj_multi_kernel(const AdjParams<T> base, const AdjMulti<T> m) {
-  __shared__ int s_next, s_go;
-  __shared__ Red<T> s_red[kWarps];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int gx = m.gx, gy = m.gy;
-  const int nit = m.last - m.s0 + 1;
-  const int both = min(nit, m.fsteps);
-  const int round = m.nblocks + m.fnblocks;
-  const int total = nit * m.nblocks + m.fsteps * m.fnblocks;
-  if (threadIdx.x == 0) s_next = int(atomicAdd(m.work, 1u));
-  __syncthreads();
-  int w = s_next;
-  while (w < total) {
-    // the item: reverse iteration it, block b; or forward step t, block b
-    int it = -1, t = 0, b;
-    if (w < both * round) {
-      const int r = w / round, o = w - r * round;
-      if (KSS_ADJ_FWD_FIRST ? o >= m.fnblocks : o < m.nblocks) {
-        it = r;
-        b = KSS_ADJ_FWD_FIRST ? o - m.fnblocks : o;
-      } else {
-        t = r + 1;
-        b = KSS_ADJ_FWD_FIRST ? o : o - m.nblocks;
-      }
-    } else {
-      const int w2 = w - both * round;
-      if (nit > both) {
-        it = both + w2 / m.nblocks;
-        b = w2 - (it - both) * m.nblocks;
-      } else {
-        const int r = w2 / m.fnblocks;
-        t = both + 1 + r;
-        b = w2 - r * m.fnblocks;
-      }
-    }
-    if (it < 0) {  // ---- a forward step of the previous segment's recomputation
-      const int fby = b / m.fgx, fbx = b - fby * m.fgx;
-      __syncthreads();  // every thread has read s_next before thread 0 rewrites it
-      if (!adj_wait_neighbours(m.fdone, fbx, fby, m.fgx, m.fgy, uint32_t(t - 1), t > 1, m.work,
-                               &s_next, &s_go, m.err, m.deadline))
-        return;
-      StepParams<T> q = m.fp;
-      q.src = t == 1 ? m.fck : m.fseg + (long long)(t - 1) * m.state_elems;
-      q.dst = m.fseg + (long long)t * m.state_elems;
-      step_block<T, MODE_PLAIN, true, true, true>(q, fbx, fby, m.fgx, nullptr, nullptr);
-      __syncthreads();  // every store of the block precedes thread 0's release
-      w = s_next;
-      // (the other warps go on to their next item meanwhile; the barrier before its
-      // wait keeps s_next until everyone has read it)
-      if (threadIdx.x == 0) {
-        fence_acq_rel_gpu();
-        st_release_u32(m.fdone + b, uint32_t(t));
-      }
-      continue;
-    }
-    // ---- a reverse iteration of this segment
-    const int by = b / gx, bx = b - by * gx;
-    const int k = m.last - it;
-    AdjParams<T> p = base;
-    p.f = k == m.s0 ? m.ck : m.seg + (long long)(k - m.s0) * m.state_elems;
-    const bool odd = ((m.lc + it) & 1) != 0;
-    p.lam_in = odd ? m.lam1 : m.lam0;
-    p.lam_out = const_cast<T*>(odd ? m.lam0 : m.lam1);
-    // the warp's first row of the forward state (written before the launch), pulled
-    // while the block waits for its neighbours
-    T ft0[9][kAdjV];
-    {
-      const int i0 = (bx * 32 + lane) * kAdjV, jf = by * p.rows + warp;
-      if (jf < min(by * p.rows + p.rows, p.ny))
-        adj_pull_row<T, false>(p.f, p.plane, p.pitch, p.nx, p.ny, jf, i0, lane, i0 < p.nx,
-                               ft0);
-    }
-    __syncthreads();  // every thread has read s_next before thread 0 rewrites it
-    if (!adj_wait_neighbours(m.done, bx, by, gx, gy, uint32_t(it), it > 0, m.work, &s_next,
-                             &s_go, m.err, m.deadline))
-      return;
-    Acc<T> sum = adj_step_block<T, true, true>(p, bx, by, ft0);
-    // the neighbours wait only for the adjoint stores: the release comes first, then the
-    // block's partial (read after the launch), as adj_reduce forms it
-    sum.warp_reduce();
-    if (lane == 0) s_red[warp] = Red<T>::of(sum);
-    __syncthreads();  // every store of the block precedes thread 0's release
-    w = s_next;
-    // (as above; s_red is rewritten only after the next item's barriers)
-    if (threadIdx.x == 0) {
-      fence_acq_rel_gpu();
-      st_release_u32(m.done + b, uint32_t(it + 1));
-      Red<T> r;
-      for (int q = 0; q < kWarps; ++q) r.add(s_red[q]);
-      r.store(m.part + (long long)it * m.nblocks + b);
-    }
-  }
-}
-
-// Block it: the total of iteration it's per-block partials part[it][0 .. nblocks - 1],
-// added as adj_reduce adds one launch's partials, into totals[it].  The block finishing
-// last (count, 0 at launch) then does *acc += totals[0] + ... in iteration order, one
-// addition each (as one launch per step adds its total).
+// Block it: the total of iteration it's partials part[it][0 .. n - 1], added in order within
+// each thread and in a fixed tree across threads, into totals[it].  The block finishing
+// last (count, 0 at launch) then does *acc += totals[0] + ... in iteration order.
 template <class T>
 __global__ void __launch_bounds__(kThreads)
-adj_iteration_totals(const double* part, int nblocks, int nit, double* totals,
-                     uint32_t* count, double* acc) {
+adj_iteration_totals(const double* part, int n, int nit, double* totals, uint32_t* count,
+                     double* acc) {
   __shared__ Red<T> s_tot[kWarps];
   __shared__ int s_last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, it = blockIdx.x;
-  const double* pp = part + (long long)it * nblocks;
+  const double* pp = part + (long long)it * n;
   Red<T> r;
-  for (int q = threadIdx.x; q < nblocks; q += kThreads) r.add(Red<T>::load(pp + q));
+#pragma unroll 4
+  for (int q = threadIdx.x; q < n; q += kThreads) r.add(Red<T>::load(pp + q));
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) r.add(r.shfl_xor(off));
   if (lane == 0) s_tot[warp] = r;
@@ -671,6 +460,7 @@ adj_iteration_totals(const double* part, int nblocks, int nit, double* totals,
     double a = *acc;
     for (int i = 0; i < nit; ++i) a += __ldcg(totals + i);
     *acc = a;
+    *count = 0u;  // ready for the next segment (stream-ordered)
   }
 }
 

@@ -41,13 +41,11 @@ struct kss_adjoint {
   double* grad = nullptr;    // dense dJ/drho0
   double* part = nullptr;    // per-CTA partials
   unsigned char* small = nullptr;  // done counter @0, acc[2] @64, error word @128
-  // the reverse sweep of a segment in one cooperative launch (adj_multi_kernel): its
-  // counters (block progress, iteration tickets, work counter: zeroed before each launch),
-  // the per-block partials and the iteration totals
-  bool multi = true;
-  int multi_ctas = 0;
-  uint32_t* mcount = nullptr;  // [nblocks] done, [E] tickets, [1] work, [fnblocks] fdone
-  double* mpart = nullptr;     // [E][nblocks]
+  // the reverse steps of a segment: their warps' partials and each step's total
+  int rev_rows = 1;            // rows per warp of a reverse step
+  long long nparts = 0;        // partials per reverse step
+  bool overlap = true;         // the next segment recomputed beside the reverse steps
+  double* mpart = nullptr;     // [E][nparts]
   double* mtot = nullptr;      // [E]
   cudaStream_t stream = nullptr;
   bool own_stream = false;
@@ -58,9 +56,12 @@ struct kss_adjoint {
   // the forward and the backward launch sequences replayed as CUDA graphs, recorded on a
   // stream of their own for the (tau, weight) they were taken with
   cudaStream_t cap = nullptr;
+  cudaStream_t side = nullptr;          // the recomputation's branch while recording
+  cudaEvent_t fork = nullptr, join = nullptr;
   cudaGraphExec_t g_fwd = nullptr, g_bwd = nullptr;
   double g_tau = 0;
   int g_weight = -1;
+  bool expect_backward = true;  // false after a forward pass without its backward pass
   std::string msg;
 };
 
@@ -84,12 +85,15 @@ void free_all(kss_adjoint* A) {
   cudaStreamSynchronize(A->stream);
   void* bufs[] = {A->ck,     A->seg,    A->seg2,  A->work[0], A->work[1],
                   A->lam[0], A->lam[1], A->wplane, A->fields, A->grad,
-                  A->part,   A->small,  A->mcount, A->mpart,  A->mtot};
+                  A->part,   A->small,  A->mpart,  A->mtot};
   for (void* b : bufs)
     if (b) kss_rt::dev_free(b);
   if (A->g_fwd) cudaGraphExecDestroy(A->g_fwd);
   if (A->g_bwd) cudaGraphExecDestroy(A->g_bwd);
   if (A->cap) cudaStreamDestroy(A->cap);
+  if (A->side) cudaStreamDestroy(A->side);
+  if (A->fork) cudaEventDestroy(A->fork);
+  if (A->join) cudaEventDestroy(A->join);
   if (A->own_stream && A->stream) cudaStreamDestroy(A->stream);
   delete A;
 }
@@ -122,12 +126,6 @@ kss::StepParams<T> plain_params(const kss_adjoint* A, const void* src, void* dst
 template <class T>
 cudaError_t plain_step(const kss_adjoint* A, const void* src, void* dst, cudaStream_t s) {
   return kss::launch_step<T>(plain_params<T>(A, src, dst), kss::MODE_PLAIN, true, true, s);
-}
-
-// The forward step grid of the plain steps (plain_params: tile 8, step_rows rows).
-template <class T>
-dim3 plain_grid(const kss_adjoint* A) {
-  return kss::step_grid<T>(A->cfg.nx, A->cfg.ny, 8, A->step_rows / 8);
 }
 
 // First step of the last segment of states f^0 .. f^{N-2} that the reverse sweep needs.
@@ -192,82 +190,51 @@ cudaError_t backward_launches(kss_adjoint* A, cudaStream_t s) {
   const int N = A->cfg.nsteps, E = A->cfg.checkpoint_every;
   int lc = 0;
   kss::AdjParams<T> p = adj_params<T>(A);
-  p.acc = acc_at(A, 1);
   cudaError_t e = cudaSuccess;
   // segments [s0, last] of the states f^0 .. f^{N-2} that the reverse sweep needs,
   // last segment first (i = 0, 1, ...); slot 0 of a segment is its checkpoint, its other
   // states are in seg[i & 1]: the last segment's from the forward pass, each other one
-  // recomputed -- by the previous segment's cooperative launch (fused), or by plain steps
-  // before its own reverse steps
-  const bool fused = A->multi && A->multi_ctas > 0;
-  const dim3 g = kss::adj_grid(A->cfg.nx, A->cfg.ny, A->adj_rows);
-  const dim3 fg = plain_grid<T>(A);
-  const int nblocks = int(g.x * g.y), fnblocks = int(fg.x * fg.y);
-  auto segbuf = [&](int i) { return (i & 1) ? A->seg2 : A->seg; };
+  // recomputed by plain steps from its checkpoint, beside the reverse steps of the segment
+  // before it (overlap: a branch of its own in the graph, whose small launches fill the gaps
+  // between the reverse steps'), or after them
+  auto state = [&](int k, int i) -> void* {
+    const int s0 = k / E * E;
+    return k == s0 ? static_cast<void*>(state_at(A, A->ck, s0 / E))
+                   : static_cast<void*>(state_at(A, (i & 1) ? A->seg2 : A->seg, k - s0));
+  };
+  auto recompute = [&](int s0, int i, cudaStream_t on) {
+    cudaError_t r = cudaSuccess;
+    for (int k = s0 + 1; k < s0 + E && r == cudaSuccess; ++k)
+      r = plain_step<T>(A, state(k - 1, i), state(k, i), on);
+    return r;
+  };
+  p.rows = A->rev_rows;
   int i = 0;
   for (int s0 = last_segment(A); s0 >= 0 && e == cudaSuccess; s0 -= E, ++i) {
-    const int last = std::min(s0 + E - 1, N - 2);
-    unsigned char* sb = segbuf(i);
-    auto state = [&](int k) -> const void* {
-      return k == s0 ? static_cast<const void*>(state_at(A, A->ck, s0 / E))
-                     : static_cast<const void*>(state_at(A, sb, k - s0));
-    };
-    if (i > 0 && !fused)
-      for (int k = s0 + 1; k <= last && e == cudaSuccess; ++k)
-        e = plain_step<T>(A, state(k - 1), const_cast<void*>(state(k)), s);
-    if (fused && e == cudaSuccess) {
-      // the segment's reverse steps in one cooperative launch (adj_multi_kernel), which
-      // also recomputes the previous segment [s0 - E, s0 - 1] into seg[(i + 1) & 1]
-      const int nit = last - s0 + 1;
-      kss::AdjMulti<T> m{};
-      m.ck = static_cast<const T*>(state(s0));
-      m.seg = reinterpret_cast<const T*>(sb);
-      m.state_elems = (long long)(A->state_bytes / A->esz);
-      m.lam0 = reinterpret_cast<const T*>(A->lam[0]);
-      m.lam1 = reinterpret_cast<const T*>(A->lam[1]);
-      m.done = A->mcount;
-      m.ticket = A->mcount + nblocks;
-      m.work = A->mcount + nblocks + A->cfg.checkpoint_every;
-      m.fdone = m.work + 1;
-      m.part = A->mpart;
-      m.totals = A->mtot;
-      m.err = reinterpret_cast<uint32_t*>(A->small + 128);
-      m.deadline = 2000000000LL;  // about a second at 2 GHz
-      m.s0 = s0;
-      m.last = last;
-      m.lc = lc;
-      m.gx = int(g.x);
-      m.gy = int(g.y);
-      m.nblocks = nblocks;
-      if (s0 > 0) {
-        unsigned char* nb = segbuf(i + 1);
-        m.fp = plain_params<T>(A, nullptr, nullptr);
-        m.fck = reinterpret_cast<const T*>(state_at(A, A->ck, s0 / E - 1));
-        m.fseg = reinterpret_cast<T*>(nb);
-        m.fsteps = E - 1;
-        m.fgx = int(fg.x);
-        m.fgy = int(fg.y);
-        m.fnblocks = fnblocks;
-      }
-      e = cudaMemsetAsync(A->mcount, 0,
-                          sizeof(uint32_t) * (size_t(nblocks) + A->cfg.checkpoint_every + 1 +
-                                              size_t(fnblocks)),
-                          s);
-      const int items = nit * nblocks + m.fsteps * m.fnblocks;
-      const int ctas = std::min(A->multi_ctas, items);
-      if (e == cudaSuccess) e = kss::launch_adj_multi<T>(p, m, ctas, p.acc, s);
-      lc ^= nit & 1;
-      continue;
+    const int last = std::min(s0 + E - 1, N - 2), nit = last - s0 + 1;
+    const bool beside = A->overlap && s0 > 0;
+    if (beside) {  // (the buffer of segment i + 1 was read by segment i - 1: done by now)
+      e = cudaEventRecord(A->fork, s);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(A->side, A->fork, 0);
+      if (e == cudaSuccess) e = recompute(s0 - E, i + 1, A->side);
+      if (e == cudaSuccess) e = cudaEventRecord(A->join, A->side);
     }
     for (int k = last; k >= s0 && e == cudaSuccess; --k) {
-      p.f = static_cast<const T*>(state(k));
+      p.f = static_cast<const T*>(state(k, i));
       p.lam_in = reinterpret_cast<const T*>(A->lam[lc]);
       p.lam_out = reinterpret_cast<T*>(A->lam[lc ^ 1]);
-      e = kss::launch_adj_step<T>(p, s);
+      p.part = A->mpart + (last - k) * A->nparts;
+      e = kss::launch_adj_reverse<T>(p, k < last, s);
       lc ^= 1;
     }
+    if (e == cudaSuccess)
+      e = kss::launch_adj_totals<T>(A->mpart, int(A->nparts), nit, A->mtot,
+                                    reinterpret_cast<uint32_t*>(A->small), acc_at(A, 1), s);
+    if (beside && e == cudaSuccess) e = cudaStreamWaitEvent(s, A->join, 0);
+    if (!A->overlap && s0 > 0 && e == cudaSuccess) e = recompute(s0 - E, i + 1, s);
   }
   const size_t n = size_t(A->cfg.nx) * A->cfg.ny;
+  p.rows = A->adj_rows;
   p.lam_in = reinterpret_cast<const T*>(A->lam[lc]);
   p.ux0 = A->fields + n;
   p.uy0 = A->fields + 2 * n;
@@ -276,42 +243,58 @@ cudaError_t backward_launches(kss_adjoint* A, cudaStream_t s) {
   return e;
 }
 
-// Replay the graph of fn's launches (recorded when tau or the weight option changed).
-template <class F>
-int run_graph(kss_adjoint* A, cudaGraphExec_t* exec, F&& fn) {
-  if (A->g_tau != A->tau || A->g_weight != int(A->have_weight)) {
-    for (cudaGraphExec_t* g : {&A->g_fwd, &A->g_bwd})
-      if (*g) {
-        cudaGraphExecDestroy(*g);
-        *g = nullptr;
-      }
-    A->g_tau = A->tau;
-    A->g_weight = int(A->have_weight);
-  }
-  if (!*exec) {
-    if (!A->cap) KSS_ACUDA(A, cudaStreamCreateWithFlags(&A->cap, cudaStreamNonBlocking));
-    KSS_ACUDA(A, cudaStreamBeginCapture(A->cap, cudaStreamCaptureModeThreadLocal));
-    const cudaError_t le = fn(A->cap);
-    cudaGraph_t graph = nullptr;
-    const cudaError_t ee = cudaStreamEndCapture(A->cap, &graph);
-    if (le != cudaSuccess || ee != cudaSuccess) {
-      if (graph) cudaGraphDestroy(graph);
-      cudaGetLastError();
-      return afail(A, KSS_ERR_CUDA, std::string("graph capture: ") +
-                                        cudaGetErrorString(le != cudaSuccess ? le : ee));
+// Forget the graphs when tau or the weight option changed.
+void check_graphs(kss_adjoint* A) {
+  if (A->g_tau == A->tau && A->g_weight == int(A->have_weight)) return;
+  for (cudaGraphExec_t* g : {&A->g_fwd, &A->g_bwd})
+    if (*g) {
+      cudaGraphExecDestroy(*g);
+      *g = nullptr;
     }
-    const cudaError_t ie = cudaGraphInstantiate(exec, graph, 0);
-    cudaGraphDestroy(graph);
-    KSS_ACUDA(A, ie);
+  A->g_tau = A->tau;
+  A->g_weight = int(A->have_weight);
+}
+
+// Record fn's launches as a graph, unless that is done.
+template <class F>
+int record_graph(kss_adjoint* A, cudaGraphExec_t* exec, F&& fn) {
+  if (*exec) return KSS_OK;
+  if (!A->cap) KSS_ACUDA(A, cudaStreamCreateWithFlags(&A->cap, cudaStreamNonBlocking));
+  if (!A->side) KSS_ACUDA(A, cudaStreamCreateWithFlags(&A->side, cudaStreamNonBlocking));
+  for (cudaEvent_t* v : {&A->fork, &A->join})
+    if (!*v) KSS_ACUDA(A, cudaEventCreateWithFlags(v, cudaEventDisableTiming));
+  KSS_ACUDA(A, cudaStreamBeginCapture(A->cap, cudaStreamCaptureModeThreadLocal));
+  const cudaError_t le = fn(A->cap);
+  cudaGraph_t graph = nullptr;
+  const cudaError_t ee = cudaStreamEndCapture(A->cap, &graph);
+  if (le != cudaSuccess || ee != cudaSuccess) {
+    if (graph) cudaGraphDestroy(graph);
+    cudaGetLastError();
+    return afail(A, KSS_ERR_CUDA, std::string("graph capture: ") +
+                                      cudaGetErrorString(le != cudaSuccess ? le : ee));
   }
-  KSS_ACUDA(A, cudaGraphLaunch(*exec, A->stream));
+  const cudaError_t ie = cudaGraphInstantiate(exec, graph, 0);
+  cudaGraphDestroy(graph);
+  KSS_ACUDA(A, ie);
   return KSS_OK;
 }
 
 template <class T>
+int record_backward(kss_adjoint* A) {
+  return record_graph(A, &A->g_bwd, [&](cudaStream_t s) { return backward_launches<T>(A, s); });
+}
+
+template <class T>
 int forward_impl(kss_adjoint* A, double* J) {
-  int rc = run_graph(A, &A->g_fwd, [&](cudaStream_t s) { return forward_launches<T>(A, s); });
+  check_graphs(A);
+  int rc =
+      record_graph(A, &A->g_fwd, [&](cudaStream_t s) { return forward_launches<T>(A, s); });
   if (rc) return rc;
+  KSS_ACUDA(A, cudaGraphLaunch(A->g_fwd, A->stream));
+  // the reverse sweep is recorded while the forward pass runs (512^2, 200 steps: 0.9 ms of
+  // recording beside 0.7 ms; a first gradient 3.4 -> 2.7 ms), unless the caller has
+  // taken a forward pass without the backward one
+  if (A->expect_backward && (rc = record_backward<T>(A))) return rc;
   KSS_ACUDA(A, cudaMemcpyAsync(J, acc_at(A, 0), sizeof(double), cudaMemcpyDeviceToHost, A->stream));
   KSS_ACUDA(A, cudaStreamSynchronize(A->stream));
   A->lam_cur = 0;
@@ -320,8 +303,9 @@ int forward_impl(kss_adjoint* A, double* J) {
 
 template <class T>
 int backward_impl(kss_adjoint* A, double* grad_tau) {
-  int rc = run_graph(A, &A->g_bwd, [&](cudaStream_t s) { return backward_launches<T>(A, s); });
+  const int rc = record_backward<T>(A);
   if (rc) return rc;
+  KSS_ACUDA(A, cudaGraphLaunch(A->g_bwd, A->stream));
   double s = 0;
   uint32_t err = 0;
   KSS_ACUDA(A, cudaMemcpyAsync(&s, acc_at(A, 1), sizeof(double), cudaMemcpyDeviceToHost, A->stream));
@@ -329,7 +313,6 @@ int backward_impl(kss_adjoint* A, double* grad_tau) {
   KSS_ACUDA(A, cudaStreamSynchronize(A->stream));
   if (err & kss::kErrBounds)
     return afail(A, KSS_ERR_BOUNDS, "a device bounds check failed (debug build)");
-  if (err) return afail(A, KSS_ERR_TIMEOUT, "a bounded wait of the reverse sweep ran out");
   if (grad_tau) *grad_tau = s / (A->tau * A->tau);
   return KSS_OK;
 }
@@ -381,7 +364,12 @@ int kss_adjoint_create(const kss_adjoint_config* cfg, kss_adjoint** out) {
   A->adj_rows = KSS_ADJ_ROWS ? KSS_ADJ_ROWS : kss::fill_rows(cfg->nx, cfg->ny, 32 * kss::kAdjV, nsm);
   A->step_rows = kss::fill_rows(cfg->nx, cfg->ny, 32 * (A->fp32 ? kss::Vec<float>::N : kss::Vec<double>::N), nsm);
   const dim3 g = kss::adj_grid(cfg->nx, cfg->ny, A->adj_rows);
-  const dim3 fg = A->fp32 ? plain_grid<float>(A) : plain_grid<double>(A);
+  // one row per warp, or up to four where the reverse step still has four waves of warps (28
+  // per SM)
+  while (A->rev_rows < 4 &&
+         kss::adj_reverse_parts(cfg->nx, cfg->ny, 2 * A->rev_rows) >= 4LL * 28 * nsm)
+    A->rev_rows *= 2;
+  A->nparts = kss::adj_reverse_parts(cfg->nx, cfg->ny, A->rev_rows);
   struct {
     void** p;
     size_t bytes;
@@ -398,10 +386,8 @@ int kss_adjoint_create(const kss_adjoint_config* cfg, kss_adjoint** out) {
       {reinterpret_cast<void**>(&A->grad), n * sizeof(double)},
       {reinterpret_cast<void**>(&A->part), size_t(g.x) * g.y * sizeof(double)},
       {reinterpret_cast<void**>(&A->small), 256},
-      {reinterpret_cast<void**>(&A->mcount),
-       sizeof(uint32_t) * (size_t(g.x) * g.y + A->cfg.checkpoint_every + 1 + size_t(fg.x) * fg.y)},
       {reinterpret_cast<void**>(&A->mpart),
-       sizeof(double) * size_t(g.x) * g.y * A->cfg.checkpoint_every},
+       sizeof(double) * size_t(A->nparts) * A->cfg.checkpoint_every},
       {reinterpret_cast<void**>(&A->mtot), sizeof(double) * size_t(A->cfg.checkpoint_every)},
   };
   for (auto& a : allocs) {
@@ -424,8 +410,6 @@ int kss_adjoint_create(const kss_adjoint_config* cfg, kss_adjoint** out) {
     free_all(A);
     return KSS_ERR_CUDA;
   }
-  A->multi_ctas = A->fp32 ? kss::adj_multi_resident_ctas<float>()
-                          : kss::adj_multi_resident_ctas<double>();
   *out = A;
   return KSS_OK;
 }
@@ -434,11 +418,11 @@ void kss_adjoint_destroy(kss_adjoint* A) { free_all(A); }
 
 int kss_adjoint_set_multistep(kss_adjoint* A, int on) {
   if (!A || (on != 0 && on != 1)) return KSS_ERR_ARG;
-  if (A->multi != (on != 0) && A->g_bwd) {  // the recorded reverse sweep is the other form
+  if (A->overlap != (on != 0) && A->g_bwd) {  // the recorded reverse sweep is the other form
     cudaGraphExecDestroy(A->g_bwd);
     A->g_bwd = nullptr;
   }
-  A->multi = on != 0;
+  A->overlap = on != 0;
   return KSS_OK;
 }
 
@@ -470,6 +454,7 @@ int kss_adjoint_forward(kss_adjoint* A, const double* rho0, const double* ux0, c
                                                         A->stream));
   }
   A->tau = tau;
+  if (A->have_forward) A->expect_backward = false;
   A->have_forward = false;
   const int rc = A->fp32 ? forward_impl<float>(A, J) : forward_impl<double>(A, J);
   if (rc) return rc;
@@ -484,6 +469,7 @@ int kss_adjoint_backward(kss_adjoint* A, double* grad_rho0, double* grad_tau, in
   DeviceGuard g(A->device);
   // the sweep consumes the seed lt^{N-1}: one backward pass per forward pass
   A->have_forward = false;
+  A->expect_backward = true;
   const int rc = A->fp32 ? backward_impl<float>(A, grad_tau) : backward_impl<double>(A, grad_tau);
   if (rc) return rc;
   if (grad_rho0) {

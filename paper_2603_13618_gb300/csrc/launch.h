@@ -114,19 +114,26 @@ inline dim3 adj_grid(int nx, int ny, int rows = kAdjRows) {
 }
 template <class T>
 cudaError_t launch_adj_objective(const AdjParams<T>& p, cudaStream_t stream);
+// One reverse step (p.rows rows per warp); chained: its predecessor in the stream is another
+// reverse step of the segment, and nothing else writes the state p.f.
+inline dim3 adj_reverse_grid(int nx, int ny, int rows) {
+  return dim3((unsigned)((nx + 32 * kAdjV - 1) / (32 * kAdjV)),
+              (unsigned)((ny + kAdjWarps * rows - 1) / (kAdjWarps * rows)), 1u);
+}
+// (the partials of one step: a double per warp)
+inline long long adj_reverse_parts(int nx, int ny, int rows) {
+  const dim3 g = adj_reverse_grid(nx, ny, rows);
+  return (long long)g.x * g.y * kAdjWarps;
+}
 template <class T>
-cudaError_t launch_adj_step(const AdjParams<T>& p, cudaStream_t stream);
+cudaError_t launch_adj_reverse(const AdjParams<T>& p, bool chained, cudaStream_t stream);
+// *acc += the totals of nit reverse steps' n partials each, in step order (totals: [nit];
+// count: a counter, 0 before and after).
+template <class T>
+cudaError_t launch_adj_totals(const double* part, int n, int nit, double* totals,
+                              uint32_t* count, double* acc, cudaStream_t stream);
 template <class T>
 cudaError_t launch_adj_final(const AdjParams<T>& p, cudaStream_t stream);
-// The reverse sweep of one segment in one cooperative launch of `ctas` persistent CTAs
-// (adj_multi_kernel), then its iteration totals added to *acc in order; and the CTAs of
-// that kernel the device holds at once.
-template <class T>
-cudaError_t launch_adj_multi(const AdjParams<T>& base, const AdjMulti<T>& m, int ctas,
-                             double* acc, cudaStream_t stream);
-template <class T>
-int adj_multi_resident_ctas();
-
 // Population conversions for any storage S (float, double, __half deviations); the
 // codec is that of the lattice (empty for float and double).
 template <class S>

@@ -400,43 +400,25 @@ cudaError_t launch_adj_objective<KSS_T>(const AdjParams<KSS_T>& p, cudaStream_t 
 }
 
 template <>
-cudaError_t launch_adj_step<KSS_T>(const AdjParams<KSS_T>& p, cudaStream_t stream) {
-  adj_step_kernel<KSS_T><<<adj_grid(p.nx, p.ny, p.rows), kThreads, 0, stream>>>(p);
+cudaError_t launch_adj_reverse<KSS_T>(const AdjParams<KSS_T>& p, bool chained,
+                                      cudaStream_t stream) {
+  const dim3 g = adj_reverse_grid(p.nx, p.ny, p.rows);
+  if (chained)
+    return launch_chained(adj_reverse_kernel<KSS_T>, g, 32 * kAdjWarps, 0, stream, 1, p);
+  adj_reverse_kernel<KSS_T><<<g, 32 * kAdjWarps, 0, stream>>>(p);
+  return cudaGetLastError();
+}
+
+template <>
+cudaError_t launch_adj_totals<KSS_T>(const double* part, int n, int nit, double* totals,
+                                     uint32_t* count, double* acc, cudaStream_t stream) {
+  adj_iteration_totals<KSS_T><<<nit, kThreads, 0, stream>>>(part, n, nit, totals, count, acc);
   return cudaGetLastError();
 }
 
 template <>
 cudaError_t launch_adj_final<KSS_T>(const AdjParams<KSS_T>& p, cudaStream_t stream) {
   adj_final_kernel<KSS_T><<<adj_grid(p.nx, p.ny, p.rows), kThreads, 0, stream>>>(p);
-  return cudaGetLastError();
-}
-
-template <>
-int adj_multi_resident_ctas<KSS_T>() {
-  return resident_ctas<adj_multi_kernel<KSS_T>>();
-}
-
-template <>
-cudaError_t launch_adj_multi<KSS_T>(const AdjParams<KSS_T>& base, const AdjMulti<KSS_T>& m,
-                                    int ctas, double* acc, cudaStream_t stream) {
-  if (ctas < 1) return cudaErrorInvalidValue;
-  // a cooperative launch (all CTAs resident: the waits need it), recorded as such when the
-  // stream is being captured into a graph
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(ctas);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, adj_multi_kernel<KSS_T>, base, m);
-  if (e != cudaSuccess) return e;
-  const int nit = m.last - m.s0 + 1;
-  adj_iteration_totals<KSS_T><<<nit, kThreads, 0, stream>>>(m.part, m.nblocks, nit, m.totals,
-                                                             m.ticket, acc);
   return cudaGetLastError();
 }
 

@@ -106,6 +106,7 @@ struct kss_lattice {
   // step count, the buffer holding the state and the phase of the output steps; recorded
   // on a stream of their own
   static constexpr int kPlainGraphs = 8;
+  // (exec is nullptr for a run seen once and launched directly: see steps_graph)
   struct PlainGraph {
     int nsteps = 0, cur = 0;
     int64_t phase = 0;

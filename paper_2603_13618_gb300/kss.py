@@ -562,8 +562,8 @@ class Adjoint:
         return J.value
 
     def set_multistep(self, on: bool) -> None:
-        """Reverse sweep in one cooperative launch per segment (True, the default) or one
-        launch per reverse step; the gradients are the same bit for bit."""
+        """Recompute each segment beside the reverse steps of the one before it (True, the
+        default) or after them; the gradients are the same bit for bit."""
         self._check(self._lib.kss_adjoint_set_multistep(self._h, int(bool(on))))
 
     def backward(self, device: bool = False):
