@@ -61,11 +61,33 @@ bool use_tma(const kss_lattice* L, int mode) {
 // CTAs of the fixup pass (2 per SM, grid-striding over the deferred cells).
 int fixup_ctas(const kss_lattice* L) { return 2 * L->nsm; }
 
+// One step from buffer L->cur.  A run of output steps whose blocks are split (chain, the
+// run's state) leaves the sums of each step but the last to the next one: their partials
+// alternate between the two sets.  more: the run's next step is an output step too.
+struct StepChain {
+  int set = 0;         // the partials the next step writes
+  bool open = false;   // the previous step's sums are still to be formed
+};
 template <class S>
-cudaError_t launch_one_step(kss_lattice* L, bool out) {
+cudaError_t launch_one_step(kss_lattice* L, bool out, StepChain* chain = nullptr,
+                            bool more = false) {
   kss::StepParams<S> p = make_params<S>(L, L->f[L->cur], L->f[L->cur ^ 1]);
   const int mode = out ? mode_for(needed_mask(L, L->cfg.record_mask), L->region != nullptr)
                        : MODE_PLAIN;
+  if (chain && out && (L->region || !use_tma(L, mode)) &&
+      kss::step_split_ranks<S>(p, mode, L->region != nullptr, nullptr)) {
+    const size_t n = size_t(L->npart);
+    if (chain->open) {
+      p.prev_sum = L->part_sum + 3 * n * (chain->set ^ 1);
+      p.prev_cnt = L->part_cnt + 4 * n * (chain->set ^ 1);
+      p.prev_out = L->part_sum + 6 * n;
+    }
+    p.part_sum = L->part_sum + 3 * n * chain->set;
+    p.part_cnt = L->part_cnt + 4 * n * chain->set;
+    p.defer = more;
+    chain->open = more;
+    chain->set ^= 1;
+  }
   if (mode == MODE_PLAIN) {  // the tile only shapes the grid of a step without outputs
     p.tile = 8;
     p.bands = L->rows_plain / 8;
@@ -281,10 +303,12 @@ cudaError_t launch_steps(kss_lattice* L, int nsteps, cudaStream_t s) {
   const int cur0 = L->cur;
   L->stream = s;
   cudaError_t e = cudaSuccess;
+  StepChain chain;
   for (int k = 0; k < nsteps && e == cudaSuccess; ++k) {
     const bool out = is_output_step(L, L->step + k + 1);
+    const bool more = k + 1 < nsteps && is_output_step(L, L->step + k + 2);
     e = with_storage(L->cfg.precision, [&](auto tag) {
-      return launch_one_step<typename decltype(tag)::type>(L, out);
+      return launch_one_step<typename decltype(tag)::type>(L, out, &chain, more);
     });
     L->cur ^= 1;
   }
@@ -702,7 +726,7 @@ static int create_lattice(const kss_config* cfg, bool slab, kss_lattice** out) {
   }
   const dim3 g = grid_for(L->bands);
   L->nblocks = int(g.x * g.y);
-  const int npart = std::max(L->nblocks, L->nsm);  // partials of either step kernel
+  const int npart = L->npart = std::max(L->nblocks, L->nsm);  // partials of either step kernel
   // list of deferred cells: 1/8 of the lattice (a full scan takes over beyond that)
   L->defer_cap = uint32_t(std::max<long long>(4096, (long long)cfg->nx * cfg->ny / 8));
   int nrec = 0;
@@ -731,8 +755,8 @@ static int create_lattice(const kss_config* cfg, bool slab, kss_lattice** out) {
       {&L->evalplane, plane_bytes},
       {reinterpret_cast<void**>(&L->flags), size_t(L->pitch) * cfg->ny},
       {reinterpret_cast<void**>(&L->tiles), sizeof(int32_t) * 3 * size_t(L->ntx) * L->nty},
-      {reinterpret_cast<void**>(&L->part_sum), sizeof(double) * 3 * size_t(npart)},
-      {reinterpret_cast<void**>(&L->part_cnt), sizeof(uint32_t) * 4 * size_t(npart)},
+      {reinterpret_cast<void**>(&L->part_sum), sizeof(double) * (6 * size_t(npart) + 6)},
+      {reinterpret_cast<void**>(&L->part_cnt), sizeof(uint32_t) * 8 * size_t(npart)},
       {reinterpret_cast<void**>(&L->small), 256},
       {reinterpret_cast<void**>(&L->defer_list), sizeof(uint32_t) * size_t(L->defer_cap)},
   };

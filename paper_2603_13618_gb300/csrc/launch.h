@@ -44,13 +44,17 @@ cudaError_t launch_step(const StepParams<T>& p, int mode, bool pull, bool store,
 // shared where the ranks, at one row per warp of eight (FP32 arithmetic: or two), all fit on
 // the GPU at once (two CTAs of 256 threads per SM); beyond that line the cluster's barriers
 // cost more than the idle SMs.  {Kn, KL, neq} steps of the density step, unsplit / split,
-// us: FP32 256^2 (16 blocks) 15.4 / 9.2, 512^2 (64) 17.5 / 10.9, 1021x517 (136) 17.1 / 13.5
-// (18.9 at one row per warp), 1024^2 (256) 21.7 / 32.8; FP64 64^2 (2) 322 / 24, 128^2 (8)
-// 243 / 37, 512x256 (64) 227 / 100; FP16 512^2 (32 blocks of 256 columns) 21.0 / 11.7,
-// 1021x517 (68) 20.3 / 14.2, 1024^2 (128) 19.9 / 26.4.  All of Table 1, FP32: 256^2
-// 44.7 / 15.1, 512^2 44.1 / 19.1, 768^2 46.4 / 33.0.
+// us: FP32 256^2 (16 blocks) 15.4 / 6.8, 512^2 (64) 17.5 / 8.4, 768^2 (144) 18.4 / 11.2 (20.5
+// at one row per warp), 1024^2 (256) 21.7 / 32.8; FP64 64^2 (2) 322 / 21, 128^2 (8) 243 / 32,
+// 512x256 (64) 227 / 100; FP16 512^2 (32 blocks of 256 columns) 21.0 / 9.0, 768^2 (72)
+// 20.2 / 11.6, 1024^2 (128) 19.9 / 17.4.  All of Table 1, FP32, before the sums of a run's
+// steps were left to the next one: 256^2 44.7 / 15.1, 512^2 44.1 / 19.1, 768^2 46.4 / 33.0.
 template <class T>
 int split_ranks(long long nblocks, int rows);
+// The same for the step that launch_step (pull + store) or launch_step_aar takes with these
+// parameters; *cells8: it takes eight cells per lane.
+template <class T>
+int step_split_ranks(const StepParams<T>& p, int mode, bool aar, bool* cells8);
 
 // One step with adaptive algorithm refinement: the two-relaxation collision in the
 // region p.region (output steps rewrite it); mode as launch_step, always pull + store.

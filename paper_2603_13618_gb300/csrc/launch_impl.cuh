@@ -149,6 +149,25 @@ int split_ranks<KSS_T>(long long nblocks, int rows) {
   return ranks >= 2 && ranks * split_rows<KSS_T>() * kSplitTurns >= rows ? ranks : 0;
 }
 
+template <>
+int step_split_ranks<KSS_T>(const StepParams<KSS_T>& p, int mode, bool aar, bool* cells8) {
+  bool eight = false;
+  dim3 g = step_grid<KSS_T>(p.nx, p.ny, p.tile, p.bands);
+  if (std::is_same<KSS_T, __half>::value && mode == MODE_STD && !aar && KSS_F16_PREFETCH &&
+      KSS_F16_CELLS8) {
+    // (the sums of an FP16 lattice's steps are those of its eight-cell blocks)
+    dim3 g8;
+    int bands8 = 0;
+    if (step_grid8(p.nx, p.ny, p.tile, p.bands, KSS_H8_WARPS, g8, bands8)) {
+      if (bands8 != p.bands) return 0;
+      eight = true;
+      g = g8;
+    }
+  }
+  if (cells8) *cells8 = eight;
+  return mode == MODE_PLAIN ? 0 : split_ranks<KSS_T>((long long)g.x * g.y, p.tile * p.bands);
+}
+
 // One split step: a cluster of `ranks` CTAs per block of `grid` (the clusters of more than
 // eight CTAs of FP64 steps need an opt-in, once per device).
 template <int MODE, bool PULL, bool STORE, bool AAR, int VC>
@@ -186,19 +205,13 @@ cudaError_t launch_step_mode(const StepParams<KSS_T>& p, dim3 grid, cudaStream_t
     if (launch_plain_f64<false>(p, grid, stream, e)) return e;
   }
   if constexpr (MODE != MODE_PLAIN) {
-    const int rows = p.tile * p.bands;
-    if constexpr (std::is_same<KSS_T, __half>::value && MODE == MODE_STD && KSS_F16_CELLS8) {
-      // (the sums of an FP16 lattice's steps are those of its eight-cell blocks)
-      dim3 g8;
-      int bands8 = 0;
-      if (step_grid8(p.nx, p.ny, p.tile, p.bands, KSS_H8_WARPS, g8, bands8)) {
-        if (bands8 == p.bands)
-          if (const int ranks = split_ranks<KSS_T>((long long)g8.x * g8.y, rows))
-            return launch_split<MODE, true, true, false, 8>(p, g8, ranks, stream);
-      } else if (const int ranks = split_ranks<KSS_T>(nblocks, rows)) {
-        return launch_split<MODE, true, true, false, Vec<KSS_T>::N>(p, grid, ranks, stream);
+    bool cells8 = false;
+    if (const int ranks = step_split_ranks<KSS_T>(p, MODE, false, &cells8)) {
+      if constexpr (std::is_same<KSS_T, __half>::value && MODE == MODE_STD) {
+        if (cells8)
+          return launch_split<MODE, true, true, false, 8>(
+              p, dim3(unsigned((p.nx + 255) / 256), grid.y), ranks, stream);
       }
-    } else if (const int ranks = split_ranks<KSS_T>(nblocks, rows)) {
       return launch_split<MODE, true, true, false, Vec<KSS_T>::N>(p, grid, ranks, stream);
     }
   }
@@ -289,9 +302,7 @@ cudaError_t launch_step<KSS_T>(const StepParams<KSS_T>& p, int mode, bool pull, 
 template <>
 cudaError_t launch_step_aar<KSS_T>(const StepParams<KSS_T>& p, int mode, cudaStream_t stream) {
   const dim3 grid = step_grid<KSS_T>(p.nx, p.ny, p.tile, p.bands);
-  const int ranks =
-      mode == MODE_PLAIN ? 0 : split_ranks<KSS_T>((long long)grid.x * grid.y, p.tile * p.bands);
-  if (ranks) {
+  if (const int ranks = step_split_ranks<KSS_T>(p, mode, true, nullptr)) {
     constexpr int V = Vec<KSS_T>::N;
     return mode == MODE_STD ? launch_split<MODE_STD, true, true, true, V>(p, grid, ranks, stream)
                             : launch_split<MODE_FULL, true, true, true, V>(p, grid, ranks, stream);

@@ -76,6 +76,9 @@ struct kss_lattice {
   void* evalplane = nullptr;
   uint8_t* flags = nullptr;
   int32_t* tiles = nullptr;
+  // per-block partials: two sets of npart (runs of split output steps alternate between
+  // them, see launch_one_step), then six words for the sums and counts of a step but the last
+  int npart = 0;
   double* part_sum = nullptr;
   uint32_t* part_cnt = nullptr;
   unsigned char* small = nullptr;  // done counter + final sums + final counts

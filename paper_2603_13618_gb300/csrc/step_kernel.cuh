@@ -236,6 +236,12 @@ struct StepParams {
   double* part_sum;      // [nblocks][3]
   uint32_t* part_cnt;    // [nblocks][4]
   uint32_t* done;        // block-completion counter, 0 between launches
+  // split steps in a run of output steps: defer: the next step forms this one's sums;
+  // prev_*: the previous step's partials, and where their sums and counts go
+  int defer;
+  const double* prev_sum;
+  const uint32_t* prev_cnt;
+  double* prev_out;      // [3] sums, then [3] 64-bit counts
   double* stat_sums;     // [3]
   unsigned long long* stat_counts;  // [3]
   uint32_t* err;         // error word: bit 0 = a bounded device wait ran out
@@ -2664,7 +2670,13 @@ step_kernel_split(const StepParams<S> p) {
   }
   __syncwarp();
   cluster_arrive();  // everything this rank pushes has been pushed
-  if (rank != 0) return;
+  if (rank != 0) {
+    // the previous step's sums, by a rank that has nothing else to do (see below)
+    if (p.prev_sum && rank == cluster_size() - 1 && bx == 0 && by == 0)
+      finalize_sums<S, NT>(p.prev_sum, p.prev_cnt, gx * int(gridDim.y), p.prev_out,
+                           reinterpret_cast<unsigned long long*>(p.prev_out + 3));
+    return;
+  }
   cluster_wait();
   const int bid = by * gx + bx;
   // the moments in the order of the unsplit block: its warp w adds rows w, w + 8, ...
@@ -2716,6 +2728,10 @@ step_kernel_split(const StepParams<S> p) {
     sum.store(p.part_sum + 3 * bid + m);
     p.part_cnt[4 * bid + m] = s_cx[m];
   }
+  // (in a run of output steps only the last one's sums are formed here: a step's fence,
+  // ticket and final addition take about 2 us that the next step need not wait for; FP32
+  // 64^2 8.4 -> 6.5 us per step, 256^2 8.8 -> 6.8, 768^2 13.4 -> 11.2)
+  if (p.defer) return;
   __syncwarp();  // thread 0's fence covers the partials that threads 1 and 2 wrote
   ticket_and_finalize<S, NT>(p, gx * int(gridDim.y), gx * int(gridDim.y));
 }
