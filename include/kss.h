@@ -319,7 +319,9 @@ typedef struct {
                         /* {Kn, KL, neq} output steps runs as ONE cooperative launch: each */
                         /* block of a step waits (bounded, KSS_ERR_TIMEOUT) only for its  */
                         /* lattice's neighbouring blocks of the previous step; same results */
-                        /* bit for bit; ctas_per_sm and graph then do not apply            */
+                        /* bit for bit; ctas_per_sm and graph then do not apply.  Batches  */
+                        /* with too few blocks to fill the GPU (and ctas_per_sm = 0) take   */
+                        /* one launch per step instead, each block shared out to a cluster  */
 } kss_batch_tuning;
 
 /* Create n >= 1 lattices from cfgs[0..n-1] (each validated as by kss_create).  Members

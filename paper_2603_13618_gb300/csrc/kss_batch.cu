@@ -46,8 +46,11 @@ struct kss_batch {
   kss::BatchItem* items = nullptr;
   int nitems = 0;
   size_t items_cap = 0;
-  double* part_sum = nullptr;     // per member [nblocks][3] from off[k]
-  uint32_t* part_cnt = nullptr;   // per member [nblocks][4] from off[k]
+  // partials, one set per table: per member [nblocks][3] and [nblocks][4] from off[k]; after
+  // both sets six words per member for the sums and counts of a split run's earlier steps
+  double* part_sum = nullptr;
+  uint32_t* part_cnt = nullptr;
+  long long parts_cap = 0;        // blocks of a set
   std::vector<int> base_cur;      // members' cur when the tables were written (par = 0)
   std::vector<long long> off;     // first partial of each member
   std::vector<dim3> grids;        // each member's step grid at the current CTA height
@@ -226,8 +229,13 @@ void fill_params(const kss_batch* B, std::vector<kss::StepParams<S>>& t0,
       p.bands = B->tun.rows / L->cfg.tile;
       p.grid_x = int(B->grids[k].x);
       p.nblocks = int(B->grids[k].x * B->grids[k].y);
-      p.part_sum = B->part_sum + 3 * B->off[k];
-      p.part_cnt = B->part_cnt + 4 * B->off[k];
+      auto sums = [&](int set) { return B->part_sum + 3 * (set * B->parts_cap + B->off[k]); };
+      auto cnts = [&](int set) { return B->part_cnt + 4 * (set * B->parts_cap + B->off[k]); };
+      p.part_sum = sums(o);
+      p.part_cnt = cnts(o);
+      p.prev_sum = sums(o ^ 1);
+      p.prev_cnt = cnts(o ^ 1);
+      p.prev_out = B->part_sum + 6 * B->parts_cap + 6 * k;
       p.mode = mode_for(needed_mask(L, L->cfg.record_mask));
       (o == 0 ? t0 : t1)[k] = p;
     }
@@ -296,8 +304,28 @@ cudaError_t launch_multi(kss_batch* B, int nsteps) {
   });
 }
 
-cudaError_t launch_one(kss_batch* B, int tbl, int mode, cudaStream_t s) {
+// CTAs that share each block of a {Kn, KL, neq} step, or 0: batches without the
+// two-relaxation model whose blocks would leave the GPU idle, unless the tuning asks for
+// persistent CTAs.
+int batch_ranks(const kss_batch* B) {
+  if (B->mode_out != kss::MODE_STD || B->aar || B->tun.ctas_per_sm > 0) return 0;
+  return with_storage(B->prec, [&](auto tag) {
+    return kss::split_ranks<typename decltype(tag)::type>(B->nitems, B->tun.rows);
+  });
+}
+
+// One step.  before, after: the run's previous and next steps have the same outputs (a split
+// run leaves the sums of each step but the last to the next one).
+cudaError_t launch_one(kss_batch* B, int tbl, int mode, cudaStream_t s, bool before = false,
+                       bool after = false) {
   const int ctas = launch_ctas(B);
+  const int ranks = mode == kss::MODE_STD ? batch_ranks(B) : 0;
+  if (ranks)
+    return with_storage(B->prec, [&](auto tag) {
+      using S = typename decltype(tag)::type;
+      return kss::launch_batch_split<S>(static_cast<const kss::StepParams<S>*>(B->table[tbl]),
+                                        B->items, B->nitems, B->tun.rows, ranks, after, before, s);
+    });
   return with_storage(B->prec, [&](auto tag) {
     using S = typename decltype(tag)::type;
     return kss::launch_batch_step<S>(static_cast<const kss::StepParams<S>*>(B->table[tbl]),
@@ -318,7 +346,8 @@ int graph_for(kss_batch* B, int nsteps, const std::string& modes, cudaGraphExec_
   KSS_BCUDA(B, cudaStreamBeginCapture(B->cap, cudaStreamCaptureModeThreadLocal));
   cudaError_t le = cudaSuccess;
   for (int s = 0; s < nsteps && le == cudaSuccess; ++s)
-    le = launch_one(B, B->par ^ (s & 1), char_mode(modes[s]), B->cap);
+    le = launch_one(B, B->par ^ (s & 1), char_mode(modes[s]), B->cap,
+                    s > 0 && modes[s - 1] == modes[s], s + 1 < nsteps && modes[s + 1] == modes[s]);
   cudaGraph_t graph = nullptr;
   const cudaError_t ee = cudaStreamEndCapture(B->cap, &graph);
   if (le != cudaSuccess || ee != cudaSuccess) {
@@ -493,6 +522,7 @@ int kss_batch_create(int32_t n, const kss_config* cfgs, kss_batch** out) {
     parts += (long long)g.x * g.y;
     nb_max.push_back((long long)g.x * g.y);
   }
+  B->parts_cap = parts;
   const size_t pb = param_bytes(B) * size_t(n);
   struct {
     void** p;
@@ -500,8 +530,8 @@ int kss_batch_create(int32_t n, const kss_config* cfgs, kss_batch** out) {
   } allocs[] = {
       {&B->table[0], pb},
       {&B->table[1], pb},
-      {reinterpret_cast<void**>(&B->part_sum), sizeof(double) * 3 * size_t(parts)},
-      {reinterpret_cast<void**>(&B->part_cnt), sizeof(uint32_t) * 4 * size_t(parts)},
+      {reinterpret_cast<void**>(&B->part_sum), sizeof(double) * (6 * size_t(parts) + 6 * size_t(n))},
+      {reinterpret_cast<void**>(&B->part_cnt), sizeof(uint32_t) * 8 * size_t(parts)},
       {&B->multi, multi_bytes(nb_max, nullptr)},
       {reinterpret_cast<void**>(&B->mtab), sizeof(kss::MultiState) * size_t(n)},
   };
@@ -585,16 +615,19 @@ int kss_batch_step(kss_batch* B, int32_t nsteps) {
   }
   const bool all_std = B->mode_out == kss::MODE_STD && !B->aar &&
                        modes.find_first_not_of('S') == std::string::npos;
-  if (B->tun.multi_step && nsteps >= 2 && all_std &&
+  const bool split = all_std && batch_ranks(B) > 0;
+  if (B->tun.multi_step && nsteps >= 2 && all_std && !split &&
       (long long)nsteps * B->nitems < (1LL << 30)) {
     KSS_BCUDA(B, launch_multi(B, nsteps));
-  } else if (B->tun.graph && nsteps >= 2) {
+  } else if (B->tun.graph && nsteps >= 2 && !split) {
     cudaGraphExec_t exec = nullptr;
     if ((rc = graph_for(B, nsteps, modes, &exec))) return rc;
     KSS_BCUDA(B, cudaGraphLaunch(exec, B->stream));
-  } else {
+  } else {  // (split runs gain nothing from a graph: 9.6 us per step either way)
     for (int s = 0; s < nsteps; ++s)
-      KSS_BCUDA(B, launch_one(B, B->par ^ (s & 1), char_mode(modes[s]), B->stream));
+      KSS_BCUDA(B, launch_one(B, B->par ^ (s & 1), char_mode(modes[s]), B->stream,
+                              s > 0 && modes[s - 1] == modes[s],
+                              s + 1 < nsteps && modes[s + 1] == modes[s]));
   }
   for (kss_lattice* L : B->mem) {
     for (int s = 0; s < nsteps; ++s) {
@@ -699,6 +732,7 @@ int kss_batch_autotune(kss_batch* B, const char* cache_path, int32_t steps,
       t.ctas_per_sm = 0;
       t.multi_step = 1;
       if ((rc = kss_batch_set_tuning(B, &t))) break;
+      if (batch_ranks(B)) continue;  // its runs take split launches, timed above
       cudaError_t e = launch_multi(B, 2);
       if (e == cudaSuccess) e = cudaEventRecord(e0, B->stream);
       if (e == cudaSuccess) e = launch_multi(B, std::max(2, int(steps)));

@@ -68,6 +68,13 @@ template <class T>
 cudaError_t launch_batch_step(const StepParams<T>* table, const BatchItem* items, int nitems,
                               int ctas, int mode, cudaStream_t stream, bool aar = false);
 
+// One batched {Kn, KL, neq} step whose items' blocks (`rows` rows each) are shared out to
+// `ranks` CTAs (batch_step_kernel_split, split_ranks); defer: the next step of the run forms
+// this one's sums; prev: this one forms the previous one's.
+template <class T>
+cudaError_t launch_batch_split(const StepParams<T>* table, const BatchItem* items, int nitems,
+                               int rows, int ranks, bool defer, bool prev, cudaStream_t stream);
+
 // nsteps batched steps in one cooperative launch (batch_kernel_multi): ta / tb are the
 // parameter tables of even / odd steps, mtab each lattice's MultiState, work the shared
 // work counter (0 at launch); mode MODE_STD; ctas <= batch_multi_resident_ctas.

@@ -380,6 +380,20 @@ cudaError_t launch_batch_multi<KSS_T>(const StepParams<KSS_T>* ta, const StepPar
 }
 
 template <>
+cudaError_t launch_batch_split<KSS_T>(const StepParams<KSS_T>* table, const BatchItem* items,
+                                      int nitems, int rows, int ranks, bool defer, bool prev,
+                                      cudaStream_t stream) {
+  constexpr auto kern = batch_step_kernel_split<KSS_T>;
+  constexpr int V = Vec<KSS_T>::N;
+  cudaError_t e = allow_dynamic_smem<kern, split_smem<KSS_T, MODE_STD, V>(64)>();
+  if (e == cudaSuccess && ranks > 8) e = allow_large_clusters<kern>();
+  if (e != cudaSuccess) return e;
+  return launch_chained(kern, dim3(unsigned(nitems), 1u, unsigned(ranks)),
+                        32 * split_warps<KSS_T>(), split_smem<KSS_T, MODE_STD, V>(rows), stream,
+                        ranks, table, items, defer, prev);
+}
+
+template <>
 cudaError_t launch_batch_step<KSS_T>(const StepParams<KSS_T>* table, const BatchItem* items,
                                      int nitems, int ctas, int mode, cudaStream_t stream,
                                      bool aar) {

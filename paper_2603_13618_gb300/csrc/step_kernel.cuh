@@ -2437,9 +2437,12 @@ __device__ __forceinline__ uint32_t fix_cell_16(const StepParams<S>& p, const Pi
   return uint32_t(rr) | (uint32_t(ss) << 1) | (uint32_t(nonpos) << 2);
 }
 
+// Block (bx, by) of a lattice whose step grid is gx blocks wide, nblocks in all, by the CTAs
+// of one cluster.  defer, prev: see the end.
 template <class S, int MODE, bool PULL, bool STORE, bool AAR, int VC>
-__global__ void __launch_bounds__(32 * split_warps<S>(), std::is_same<S, double>::value ? 4 : 2)
-step_kernel_split(const StepParams<S> p) {
+__device__ __forceinline__ void split_block(const StepParams<S>& p, const int bx, const int by,
+                                            const int gx, const int nblocks, const bool defer,
+                                            const bool prev) {
   using T = arith_t<S>;
   constexpr int V = Vec<S>::N, NW = split_warps<S>(), NT = 32 * NW;
   constexpr bool kH8 = VC == 8, FULL = MODE == MODE_FULL, kF64 = std::is_same<S, double>::value;
@@ -2450,7 +2453,6 @@ step_kernel_split(const StepParams<S> p) {
   constexpr int kCells = kF64 ? 1 : VC;   // cells per lane of a row
   constexpr int kShare = VC / kCells;     // warps per row
   static_assert(NW == split_rows<S>() * kShare, "warps of a rank");
-  const int bx = blockIdx.x, by = blockIdx.y, gx = gridDim.x;
   const uint32_t rank = cluster_rank();
   const int lane = threadIdx.x & 31, warp = __shfl_sync(kFull, int(threadIdx.x >> 5), 0);
   const int rows = p.tile * p.bands, stride = int(cluster_size()) * split_rows<S>();
@@ -2672,8 +2674,8 @@ step_kernel_split(const StepParams<S> p) {
   cluster_arrive();  // everything this rank pushes has been pushed
   if (rank != 0) {
     // the previous step's sums, by a rank that has nothing else to do (see below)
-    if (p.prev_sum && rank == cluster_size() - 1 && bx == 0 && by == 0)
-      finalize_sums<S, NT>(p.prev_sum, p.prev_cnt, gx * int(gridDim.y), p.prev_out,
+    if (prev && rank == cluster_size() - 1 && bx == 0 && by == 0)
+      finalize_sums<S, NT>(p.prev_sum, p.prev_cnt, nblocks, p.prev_out,
                            reinterpret_cast<unsigned long long*>(p.prev_out + 3));
     return;
   }
@@ -2731,9 +2733,17 @@ step_kernel_split(const StepParams<S> p) {
   // (in a run of output steps only the last one's sums are formed here: a step's fence,
   // ticket and final addition take about 2 us that the next step need not wait for; FP32
   // 64^2 8.4 -> 6.5 us per step, 256^2 8.8 -> 6.8, 768^2 13.4 -> 11.2)
-  if (p.defer) return;
+  if (defer) return;
   __syncwarp();  // thread 0's fence covers the partials that threads 1 and 2 wrote
-  ticket_and_finalize<S, NT>(p, gx * int(gridDim.y), gx * int(gridDim.y));
+  ticket_and_finalize<S, NT>(p, nblocks, nblocks);
+}
+
+template <class S, int MODE, bool PULL, bool STORE, bool AAR, int VC>
+__global__ void __launch_bounds__(32 * split_warps<S>(), std::is_same<S, double>::value ? 4 : 2)
+step_kernel_split(const StepParams<S> p) {
+  split_block<S, MODE, PULL, STORE, AAR, VC>(p, blockIdx.x, blockIdx.y, gridDim.x,
+                                             gridDim.x * gridDim.y, p.defer != 0,
+                                             p.prev_sum != nullptr);
 }
 
 // A plain FP64 step of a small lattice: CTAs of two rows of 64 columns, one cell per lane
@@ -2924,6 +2934,32 @@ batch_step_kernel(const StepParams<S>* __restrict__ table, const BatchItem* __re
                                               sp.nblocks);
     __syncthreads();  // the CTA's shared memory is reused by the next item
   }
+}
+
+// The batched {Kn, KL, neq} step with each item's block shared out to a cluster of CTAs
+// (split_block; grid nitems x 1 x ranks), for batches with too few blocks to fill the GPU,
+// bound by a block's chain of rows: 25 steps, us, the multi-step launch's one CTA per block /
+// here: FP32 four of 64^2 606 / 225, eight of 256^2 607 / 357; FP16 four of 64^2 577 / 221;
+// FP64 two of 64^2 9280 / 689, eight of 96x80 12026 / 2672.
+// The table's entries of even and odd steps hold the two sets of partials (prev_*: the
+// other's); defer, prev: see split_block.
+template <class S>
+__global__ void __launch_bounds__(32 * split_warps<S>(), std::is_same<S, double>::value ? 4 : 2)
+batch_step_kernel_split(const StepParams<S>* __restrict__ table,
+                        const BatchItem* __restrict__ items, bool defer, bool prev) {
+  static_assert(sizeof(StepParams<S>) % 8 == 0, "parameter copy in 8-byte words");
+  __shared__ __align__(16) unsigned long long s_raw[sizeof(StepParams<S>) / 8];
+  const BatchItem it = items[blockIdx.x];
+  const unsigned long long* src = reinterpret_cast<const unsigned long long*>(table + it.lat);
+  for (int k = threadIdx.x; k < int(sizeof(StepParams<S>) / 8); k += 32 * split_warps<S>())
+    s_raw[k] = src[k];
+  __syncthreads();
+  // (FP32: the parameters in registers, 9.6 -> 9.0 us per step of four 64^2 lattices; FP16 and
+  // FP64 have none to spare, 9.2 -> 9.4 and 44.6 -> 46.6 us; read from the table: 10.5 us)
+  using P = StepParams<S>;
+  const std::conditional_t<std::is_same<S, float>::value, P, P&> p = *reinterpret_cast<P*>(s_raw);
+  split_block<S, MODE_STD, true, true, false, Vec<S>::N>(p, int(it.bx), int(it.by), p.grid_x,
+                                                         p.nblocks, defer, prev);
 }
 
 // ---------------------------------------------------------------- batched multi-step ----

@@ -88,3 +88,31 @@ def test_split_two_relaxation_steps(kss, precision, record, switch, at):
                         _outputs(batch[0]) + [batch[0].get_aar_region()]):
             np.testing.assert_array_equal(a, b)
     batch.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64", "fp16dev"])
+@pytest.mark.parametrize("rows", [16, 32, 64])
+@pytest.mark.parametrize("shapes", [[(1, 1)], [(64, 64), (33, 17), (200, 90)],
+                                    [(128, 65)] * 7, [(300, 64), (129, 1), (128, 33), (5, 200)]])
+def test_split_batches_equal_one_cta_per_block(kss, precision, rows, shapes):
+    """Batches with few blocks, against the same batch with persistent CTAs (one per block);
+    the second set's sums are those of the last step of each run."""
+    from paper_2603_13618_gb300 import inputs
+
+    kw = dict(precision=precision, tau=0.56, record=("kl",), output_every=1)
+    a = kss.Batch([dict(nx=nx, ny=ny) for nx, ny in shapes], **kw)
+    b = kss.Batch([dict(nx=nx, ny=ny) for nx, ny in shapes], **kw)
+    a.set_tuning(rows=rows)
+    b.set_tuning(rows=rows, ctas_per_sm=1, multi_step=0)
+    for k, (nx, ny) in enumerate(shapes):
+        fields = inputs.smooth_jump(nx, ny, seed=20 + k, kmax=2)
+        a[k].set_fields(*fields)
+        b[k].set_fields(*fields)
+    for steps in (1, 5, 2):
+        a.step(steps)
+        b.step(steps)
+        for x, y in zip(a.members, b.members):
+            for u, v in zip(_outputs(x), _outputs(y)):
+                np.testing.assert_array_equal(u, v)
+    a.close()
+    b.close()
