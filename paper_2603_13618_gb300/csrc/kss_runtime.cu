@@ -122,7 +122,8 @@ cudaError_t launch_one_step(kss_lattice* L, bool out, StepChain* chain = nullptr
 
 // Multi-step launches (KSS_MULTISTEP, default on): kss_step(n >= 2) with every step an
 // output step of the {Kn, KL, neq} set runs as one cooperative launch of
-// step_kernel_multi (the kernel also takes plain steps).
+// step_kernel_multi (the kernel also takes plain steps), except on the lattices that
+// one_launch_per_step names.
 #ifndef KSS_MULTISTEP
 #define KSS_MULTISTEP 1
 #endif
@@ -324,7 +325,17 @@ cudaError_t launch_steps(kss_lattice* L, int nsteps, cudaStream_t s) {
 // Plain steps (2 to 3 us each) would wait for their launches without it; a run of output
 // steps only (8 us and more each) does not, and is launched directly the first time: 50 of
 // a 256^2 lattice 0.36 ms, 0.48 when recorded, 0.34 replayed.
+// A stream under capture takes no graph launch, and its caller keeps the launches anyway: a
+// run of output steps is launched directly into it.
 int steps_graph(kss_lattice* L, int nsteps) {
+  if (L->cfg.output_every == 1) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(L->stream, &st) != cudaSuccess) cudaGetLastError();
+    if (st == cudaStreamCaptureStatusActive) {
+      KSS_CUDA(L, launch_steps(L, nsteps, L->stream));
+      return KSS_OK;
+    }
+  }
   const int64_t phase = L->cfg.output_every > 0 ? L->step % L->cfg.output_every : 0;
   kss_lattice::PlainGraph* slot = nullptr;
   for (auto& g : L->plain_graphs)
@@ -955,8 +966,8 @@ int kss_step(kss_lattice* L, int32_t nsteps) {
   if (injected_launch_error() != cudaSuccess)
     return fail(L, KSS_ERR_CUDA, "injected launch failure (kss_testing_fail_after)");
   DeviceGuard g(L->device);
-  // several output steps of the {Kn, KL, neq} set on FP32 or FP64 storage: one multi-step
-  // launch (measured on GB300 at 4096^2 FP32: 0.232 vs 0.244 ms per step; plain steps and
+  // several output steps of the {Kn, KL, neq} set on FP32 or FP64 storage, of a lattice above
+  // the line of one_launch_per_step: one multi-step launch (measured on GB300 at 4096^2 FP32: 0.232 vs 0.244 ms per step; plain steps and
   // FP16-deviation storage gain nothing from it: 0.179 vs 0.179, 0.224 vs 0.221 ms)
   const int every = L->cfg.output_every;
   const int mode =

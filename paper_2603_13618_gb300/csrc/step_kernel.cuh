@@ -1705,7 +1705,7 @@ __host__ __device__ constexpr int step_prefetch_smem() {
 
 // The populations of row j's V-cell vectors at column i0 after the pull (loads of the nine
 // source rows, the halo values of the cx != 0 planes, the shifts along x): the direct-load
-// path of step_block, and one row of a plain step on its own (the adjoint's recomputation).
+// path of step_block.
 template <class S>
 __device__ __forceinline__ void pull_row(const StepParams<S>& p, int j, int i0, int lane,
                                          bool cv, arith_t<S> (&ft)[9][Vec<S>::N]) {

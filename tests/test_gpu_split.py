@@ -116,3 +116,30 @@ def test_split_batches_equal_one_cta_per_block(kss, precision, rows, shapes):
                 np.testing.assert_array_equal(u, v)
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(64, 64), (300, 200), (900, 1000)])
+def test_runs_under_capture(kss, nx, ny):
+    """A run of output steps recorded into the caller's graph: one replay equals the call."""
+    import torch
+    from paper_2603_13618_gb300 import inputs
+
+    fields = inputs.smooth_jump(nx, ny, seed=9, kmax=2)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        a = kss.Lattice(nx, ny, precision="fp32", tau=0.6, record=("kl",))
+        b = kss.Lattice(nx, ny, precision="fp32", tau=0.6, record=("kl",))
+        for x in (a, b):
+            x.set_fields(*fields)
+            for _ in range(3):
+                x.step(4)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            a.step(4)
+        graph.replay()
+        b.step(4)
+        for u, v in zip(_outputs(a), _outputs(b)):
+            np.testing.assert_array_equal(u, v)
+        a.close()
+        b.close()
