@@ -353,18 +353,18 @@ def adjoint_roofline(n, N, E, ms):
 
 
 def adjoint_launches(N, E):
-    """Kernel launches of one gradient: the forward pass (equilibrium, N - 1 plain steps,
-    the last segment's states among them, and the objective), then per segment of the
-    reverse sweep, last first: its recomputed plain steps (all but the last segment), one
-    launch per reverse step, and the ordered addition of its totals.  Then the final
-    projection."""
-    fwd = 1 + (N - 1) + 1
+    """Kernel launches of one FP32 gradient: the forward pass (equilibrium, N - 1 plain
+    steps, two to a launch, the last segment's states among them, and the objective), then
+    per segment of the reverse sweep, last first: its recomputed plain steps (all but the
+    last segment), one launch per reverse step, and the ordered addition of its totals.
+    Then the final projection."""
+    fwd = 1 + N // 2 + 1
     bwd = 1
     s0 = ((N - 2) // E) * E if N >= 2 else -1
     first = True
     while s0 >= 0:
         last = min(s0 + E - 1, N - 2)
-        bwd += (0 if first else last - s0) + (last - s0 + 1) + 1
+        bwd += (0 if first else (last - s0 + 1) // 2) + (last - s0 + 1) + 1
         first = False
         s0 -= E
     return fwd + bwd

@@ -43,6 +43,7 @@ struct kss_adjoint {
   unsigned char* small = nullptr;  // done counter @0, acc[2] @64, error word @128
   // the reverse steps of a segment: their warps' partials and each step's total
   int rev_rows = 1;            // rows per warp of a reverse step
+  bool twice = false;          // plain steps go two to a launch
   long long nparts = 0;        // partials per reverse step
   bool overlap = true;         // the next segment recomputed beside the reverse steps
   double* mpart = nullptr;     // [E][nparts]
@@ -128,6 +129,13 @@ cudaError_t plain_step(const kss_adjoint* A, const void* src, void* dst, cudaStr
   return kss::launch_step<T>(plain_params<T>(A, src, dst), kss::MODE_PLAIN, true, true, s);
 }
 
+// Two from src to dst, the state in between to mid (or nowhere: null).
+template <class T>
+cudaError_t plain_steps2(const kss_adjoint* A, const void* src, void* mid, void* dst,
+                         cudaStream_t s) {
+  return kss::launch_plain_twice<T>(plain_params<T>(A, src, dst), static_cast<T*>(mid), s);
+}
+
 // First step of the last segment of states f^0 .. f^{N-2} that the reverse sweep needs.
 int last_segment(const kss_adjoint* A) {
   const int N = A->cfg.nsteps, E = A->cfg.checkpoint_every;
@@ -166,11 +174,18 @@ cudaError_t forward_launches(kss_adjoint* A, cudaStream_t s) {
   // work[]
   const int sl = last_segment(A);
   const void* cur = A->ck;
-  for (int k = 1; k < N && e == cudaSuccess; ++k) {
-    void* dst = (k % E == 0)         ? state_at(A, A->ck, k / E)
-                : (sl >= 0 && k > sl && k <= N - 2) ? state_at(A, A->seg, k - sl)
-                                                    : A->work[k & 1];
-    e = plain_step<T>(A, cur, dst, s);
+  auto kept = [&](int k) -> void* {
+    return (k % E == 0)                        ? state_at(A, A->ck, k / E)
+           : (sl >= 0 && k > sl && k <= N - 2) ? state_at(A, A->seg, k - sl)
+                                               : nullptr;
+  };
+  for (int k = 1, w = 0; k < N && e == cudaSuccess; ++k) {
+    const bool two = A->twice && k + 1 < N;
+    void* const mid = two ? kept(k) : nullptr;
+    k += two;
+    void* dst = kept(k);
+    if (!dst) dst = A->work[w ^= 1];
+    e = two ? plain_steps2<T>(A, cur, mid, dst, s) : plain_step<T>(A, cur, dst, s);
     cur = dst;
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(A->small + 64, 0, 2 * sizeof(double), s);
@@ -204,8 +219,12 @@ cudaError_t backward_launches(kss_adjoint* A, cudaStream_t s) {
   };
   auto recompute = [&](int s0, int i, cudaStream_t on) {
     cudaError_t r = cudaSuccess;
-    for (int k = s0 + 1; k < s0 + E && r == cudaSuccess; ++k)
-      r = plain_step<T>(A, state(k - 1, i), state(k, i), on);
+    for (int k = s0 + 1; k < s0 + E && r == cudaSuccess; ++k) {
+      const bool two = A->twice && k + 1 < s0 + E;
+      r = two ? plain_steps2<T>(A, state(k - 1, i), state(k, i), state(k + 1, i), on)
+              : plain_step<T>(A, state(k - 1, i), state(k, i), on);
+      k += two;
+    }
     return r;
   };
   p.rows = A->rev_rows;
@@ -366,6 +385,7 @@ int kss_adjoint_create(const kss_adjoint_config* cfg, kss_adjoint** out) {
   const dim3 g = kss::adj_grid(cfg->nx, cfg->ny, A->adj_rows);
   // one row per warp, or up to four where the reverse step still has four waves of warps (28
   // per SM)
+  A->twice = cfg->precision == KSS_FP32 && kss::can_step_twice<float>(cfg->nx, cfg->ny);
   while (A->rev_rows < 4 &&
          kss::adj_reverse_parts(cfg->nx, cfg->ny, 2 * A->rev_rows) >= 4LL * 28 * nsm)
     A->rev_rows *= 2;

@@ -298,7 +298,25 @@ bool is_output_step(const kss_lattice* L, int64_t n) {
   return L->cfg.output_every > 0 && n % L->cfg.output_every == 0;
 }
 
-// The next nsteps steps from buffer L->cur, one launch each, on stream s (L->cur unchanged).
+// Do the steps k + 1 and k + 2 from now go as one launch (launch_plain_twice): two plain steps
+// of an FP32 lattice, and not the last of the run, whose source the other buffer has to hold
+// afterwards (launch_eval streams it).
+bool two_steps(const kss_lattice* L, int k, int nsteps) {
+  return k + 2 < nsteps && L->cfg.precision == KSS_FP32 && !L->region && !L->slab &&
+         !use_tma(L, MODE_PLAIN) && !is_output_step(L, L->step + k + 1) &&
+         !is_output_step(L, L->step + k + 2) &&
+         kss::can_step_twice<float>(L->cfg.nx, L->cfg.ny);
+}
+
+// Launches of the next nsteps steps as launch_steps makes them (each swaps the buffers).
+int step_launches(const kss_lattice* L, int nsteps) {
+  int n = 0;
+  for (int k = 0; k < nsteps; ++k, ++n) k += two_steps(L, k, nsteps);
+  return n;
+}
+
+// The next nsteps steps from buffer L->cur, one launch each (two plain FP32 steps: one for
+// both), on stream s (L->cur unchanged).
 cudaError_t launch_steps(kss_lattice* L, int nsteps, cudaStream_t s) {
   const cudaStream_t keep = L->stream;
   const int cur0 = L->cur;
@@ -306,6 +324,13 @@ cudaError_t launch_steps(kss_lattice* L, int nsteps, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
   StepChain chain;
   for (int k = 0; k < nsteps && e == cudaSuccess; ++k) {
+    if (two_steps(L, k, nsteps)) {
+      e = kss::launch_plain_twice<float>(
+          make_params<float>(L, L->f[L->cur], L->f[L->cur ^ 1]), nullptr, s);
+      L->cur ^= 1;
+      ++k;
+      continue;
+    }
     const bool out = is_output_step(L, L->step + k + 1);
     const bool more = k + 1 < nsteps && is_output_step(L, L->step + k + 2);
     e = with_storage(L->cfg.precision, [&](auto tag) {
@@ -986,7 +1011,8 @@ int kss_step(kss_lattice* L, int32_t nsteps) {
   }
   // any other run of steps: one launch each, replayed as graphs of at most kGraphChunk
   // steps; longer runs go in chunks of whole output periods and an even step count, so that
-  // every chunk has the same (count, buffer, phase) key and replays the same graph
+  // the chunks have the same (count, buffer, phase) key, or two in turn, and replay the same
+  // graphs
   int32_t left = nsteps;
   while (left > 0) {
     int32_t c = 1;
@@ -995,7 +1021,9 @@ int kss_step(kss_lattice* L, int32_t nsteps) {
       const int64_t period = every > 0 ? std::lcm<int64_t>(2, every) : 2;
       if (c < left && period <= kGraphChunk) c = int32_t(c / period * period);
     }
+    int swaps = 1;
     if (c >= 2) {
+      swaps = step_launches(L, c);
       if ((rc = steps_graph(L, c))) return rc;
     } else {
       const bool out = is_output_step(L, L->step + 1);
@@ -1005,7 +1033,7 @@ int kss_step(kss_lattice* L, int32_t nsteps) {
     }
     for (int32_t s = 0; s < c; ++s)
       if (is_output_step(L, L->step + s + 1)) L->out_step = L->rec_step = L->step + s + 1;
-    L->cur ^= c & 1;
+    L->cur ^= swaps & 1;
     L->step += c;
     left -= c;
   }

@@ -56,6 +56,15 @@ int split_ranks(long long nblocks, int rows);
 template <class T>
 int step_split_ranks(const StepParams<T>& p, int mode, bool aar, bool* cells8);
 
+// Two plain steps in one launch, from p.src to p.dst (step_plain_twice_kernel: FP32 storage,
+// no two-relaxation model, no slab; faster at every size measured, 64^2 to 8192^2, so that
+// only the grid's limit of rows bounds it); mid: where the state in between goes, or null.
+constexpr int kTwiceRows = 8;  // rows per CTA
+template <class T>
+bool can_step_twice(int nx, int ny);
+template <class T>
+cudaError_t launch_plain_twice(const StepParams<T>& p, T* mid, cudaStream_t stream);
+
 // One step with adaptive algorithm refinement: the two-relaxation collision in the
 // region p.region (output steps rewrite it); mode as launch_step, always pull + store.
 template <class T>

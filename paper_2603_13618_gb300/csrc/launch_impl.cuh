@@ -300,6 +300,31 @@ cudaError_t launch_step<KSS_T>(const StepParams<KSS_T>& p, int mode, bool pull, 
 }
 
 template <>
+bool can_step_twice<KSS_T>(int nx, int ny) {
+  return std::is_same<KSS_T, float>::value && (ny + kTwiceRows - 1) / kTwiceRows <= 65535 && nx > 0;
+}
+
+template <class S>
+cudaError_t launch_twice(const StepParams<S>& p, S* mid, cudaStream_t stream) {
+  if constexpr (std::is_same<S, float>::value) {
+    constexpr auto kern = step_plain_twice_kernel<kTwiceRows>;
+    constexpr int dyn = 9 * (kTwiceRows + 2) * kTwicePitch * int(sizeof(float));
+    const cudaError_t e = allow_dynamic_smem<kern, dyn>();
+    if (e != cudaSuccess) return e;
+    const dim3 g((p.nx + 127) / 128, (p.ny + kTwiceRows - 1) / kTwiceRows);
+    kern<<<g, 32 * (kTwiceRows + 3), dyn, stream>>>(p, mid);
+    return cudaGetLastError();
+  }
+  return cudaErrorInvalidValue;
+}
+
+template <>
+cudaError_t launch_plain_twice<KSS_T>(const StepParams<KSS_T>& p, KSS_T* mid,
+                                      cudaStream_t stream) {
+  return launch_twice<KSS_T>(p, mid, stream);
+}
+
+template <>
 cudaError_t launch_step_aar<KSS_T>(const StepParams<KSS_T>& p, int mode, cudaStream_t stream) {
   const dim3 grid = step_grid<KSS_T>(p.nx, p.ny, p.tile, p.bands);
   if (const int ranks = step_split_ranks<KSS_T>(p, mode, true, nullptr)) {

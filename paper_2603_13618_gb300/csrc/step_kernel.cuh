@@ -2764,6 +2764,99 @@ __global__ void __launch_bounds__(128) step_plain_f64_kernel(const StepParams<do
                                                            unused[2], mbits);
 }
 
+// Two plain FP32 steps of a tile of 128 columns x H rows in one launch: the first over the
+// tile and the cells around it (one warp per row, and one warp for the columns x0 - 1 and
+// x0 + 128), into shared memory, the second from there.  mid: the state in between, of the
+// tile's own cells (null: not kept).  The arithmetic is that of the plain step, cell by cell.
+// A plain step is bound by its one read and one write of the populations (large lattices: all
+// of the HBM bandwidth) or by its launch and load latency (small ones); this halves both, for
+// (H + 2) / H of the first step's arithmetic.  Per step of 20 steps, us, one / two to a launch
+// (all ten pairs): 64^2 6.1 / 4.1, 512^2 6.8 / 5.0, 1024^2 12.5 / 9.8, 2048^2 51.2 / 31.1,
+// 4096^2 181 / 110, 8192^2 712 / 424.  Eight rows at two CTAs per SM: three CTAs (56 registers,
+// spills) 116 at 4096^2; sixteen rows (one CTA) 152; six rows at three CTAs 107, but 5.3
+// against 5.0 at 512^2.
+constexpr int kTwicePitch = 136;  // floats of a row in shared memory: column c is at c + 4
+template <int H>
+__global__ void __launch_bounds__(32 * (H + 3), 2) step_plain_twice_kernel(const StepParams<float> p,
+                                                                        float* mid) {
+  constexpr int R = H + 2, P = kTwicePitch;
+  constexpr int cy[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+  extern __shared__ __align__(16) float kss_twice_smem[];
+  auto at = [&](int q, int r, int c) -> float* { return kss_twice_smem + (q * R + r) * P + c + 4; };
+  const int lane = threadIdx.x & 31, warp = __shfl_sync(kFull, int(threadIdx.x >> 5), 0);
+  const int x0 = blockIdx.x * 128, y0 = blockIdx.y * H, hr = min(H, p.ny - y0);
+  const int i0 = x0 + 4 * lane;
+  const bool cv = i0 < p.nx;
+  if (!bounds_ok(x0 < p.pitch && y0 < p.ny, p.err)) return;  // (uniform over the CTA)
+  Acc<float> unused[3];
+  auto wrap = [&](int j) { return j < 0 ? j + p.ny : (j >= p.ny ? j - p.ny : j); };
+  F2 f[9][2];
+  if (warp < hr + 2) {
+    const int j = wrap(y0 - 1 + warp);
+    float ft[9][4];
+    pull_row<float>(p, j, i0, lane, cv, ft);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+      f[q][0] = pack2(ft[q][0], ft[q][1]);
+      f[q][1] = pack2(ft[q][2], ft[q][3]);
+    }
+    fused_row_paired<float, MODE_PLAIN, false>(p, f, i0, j, cv, unused[0], unused[1], unused[2]);
+    float* const m = mid && warp >= 1 && warp <= hr && cv ? mid + (long long)j * p.pitch + i0
+                                                         : nullptr;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+      unpack2(f[q][0], ft[q][0], ft[q][1]);
+      unpack2(f[q][1], ft[q][2], ft[q][3]);
+      *reinterpret_cast<float4*>(at(q, warp, 4 * lane)) =
+          make_float4(ft[q][0], ft[q][1], ft[q][2], ft[q][3]);
+      if (m) vstore<float, 4>(m + q * p.plane, ft[q]);
+    }
+  } else if (warp == H + 2) {
+    const int xe = min(x0 + 128, p.nx);
+    for (int k = lane; k < 2 * (hr + 2); k += 32) {
+      const int r = k >> 1, j = wrap(y0 - 1 + r);
+      const int i = (k & 1) ? (xe == p.nx ? 0 : xe) : (x0 == 0 ? p.nx : x0) - 1;
+      float c[9];
+      pull_cell<float, true>(p, i, j, true, c);
+#pragma unroll
+      for (int q = 0; q < 9; ++q) f[q][0] = f[q][1] = pack2(c[q], c[q]);
+      fused_row_paired<float, MODE_PLAIN, false>(p, f, 0, j, true, unused[0], unused[1],
+                                                 unused[2]);
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        float v, w;
+        unpack2(f[q][0], v, w);
+        *at(q, r, (k & 1) ? 128 : -1) = v;
+      }
+    }
+  }
+  __syncthreads();
+  if (warp >= hr) return;
+  const int r = warp + 1;
+  float ft[9][4];
+#pragma unroll
+  for (int q = 0; q < 9; ++q) {
+    const float4 v = *reinterpret_cast<const float4*>(at(q, r - cy[q], 4 * lane));
+    ft[q][0] = v.x;
+    ft[q][1] = v.y;
+    ft[q][2] = v.z;
+    ft[q][3] = v.w;
+  }
+  assemble_from_left<float>(ft[1], *at(1, r, -1), lane);
+  assemble_from_left<float>(ft[5], *at(5, r - 1, -1), lane);
+  assemble_from_left<float>(ft[8], *at(8, r + 1, -1), lane);
+  assemble_from_right<float>(ft[3], *at(3, r, 128), i0, p.nx, lane);
+  assemble_from_right<float>(ft[6], *at(6, r - 1, 128), i0, p.nx, lane);
+  assemble_from_right<float>(ft[7], *at(7, r + 1, 128), i0, p.nx, lane);
+#pragma unroll
+  for (int q = 0; q < 9; ++q) {
+    f[q][0] = pack2(ft[q][0], ft[q][1]);
+    f[q][1] = pack2(ft[q][2], ft[q][3]);
+  }
+  fused_row_paired<float, MODE_PLAIN, true>(p, f, i0, y0 + warp, cv, unused[0], unused[1],
+                                            unused[2]);
+}
+
 // ---------------------------------------------------------------- multi-step ----
 // nsteps steps in one cooperative launch (every CTA resident).  The (step, block) work
 // items are handed out in order from an atomic counter (as the hardware hands out the
