@@ -464,7 +464,7 @@ int regrid_run(Workspace& ws, const uint8_t* d_flags, long long pitch, int nx, i
   // the outputs: device arrays are written directly; host ones go through borrowed
   // page-locked memory (16 bytes for the count, the mask, then boxes) where they fit
   static_assert(sizeof(Box) == sizeof(kss_box), "box layout");
-  const HostLease lease;
+  HostLease lease(s);
   const size_t at_boxes = 16 + (size_t(ntiles) + 15) / 16 * 16;
   unsigned char* const mail = static_cast<unsigned char*>(lease.room(at_boxes));
   int* const count_mail = static_cast<int*>(lease.room(16));
@@ -489,8 +489,9 @@ int regrid_run(Workspace& ws, const uint8_t* d_flags, long long pitch, int nx, i
     return fail_cuda(e);
   if (L) {
     if (const int r = finish(L, lease)) return r;
-  } else if ((e = cudaStreamSynchronize(s)) != cudaSuccess) {
-    return fail_cuda(e);
+  } else {
+    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return fail_cuda(e);
+    lease.settled();
   }
   if (count_mail) total = *count_mail;
   if (!on_device) {

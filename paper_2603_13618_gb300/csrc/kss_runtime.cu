@@ -508,50 +508,7 @@ cudaError_t launch_flags_out(kss_lattice* L, uint8_t* out, int32_t* tiles_out) {
 
 namespace kss_rt {
 
-// ---- borrowed page-locked memory ----
-namespace lease_pool {
-std::mutex g_mutex;
-unsigned char* g_kept[HostLease::kKeptLeases];
-int g_n = 0;
-}  // namespace lease_pool
-
-HostLease::HostLease(bool wanted) : p(nullptr) {
-  if (!wanted) return;
-  {
-    std::lock_guard<std::mutex> lock(lease_pool::g_mutex);
-    if (lease_pool::g_n > 0) {
-      p = lease_pool::g_kept[--lease_pool::g_n];
-      return;
-    }
-  }
-  // (another thread's stream capture is not disturbed by the allocation)
-  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-  cudaThreadExchangeStreamCaptureMode(&mode);
-  void* q = nullptr;
-  if (cudaHostAlloc(&q, kBytes, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
-    cudaGetLastError();
-    q = nullptr;
-  }
-  cudaThreadExchangeStreamCaptureMode(&mode);
-  p = static_cast<unsigned char*>(q);
-}
-
-HostLease::~HostLease() {
-  if (!p) return;
-  {
-    std::lock_guard<std::mutex> lock(lease_pool::g_mutex);
-    if (lease_pool::g_n < kKeptLeases) {
-      lease_pool::g_kept[lease_pool::g_n++] = p;
-      return;
-    }
-  }
-  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-  cudaThreadExchangeStreamCaptureMode(&mode);
-  if (cudaFreeHost(p) != cudaSuccess) cudaGetLastError();
-  cudaThreadExchangeStreamCaptureMode(&mode);
-}
-
-int finish(kss_lattice* L, const HostLease& lease, Status* st) {
+int finish(kss_lattice* L, HostLease& lease, Status* st) {
   unsigned char block[HostLease::kMailBytes];
   const unsigned char* b = lease.p;
   if (b) {
@@ -563,6 +520,7 @@ int finish(kss_lattice* L, const HostLease& lease, Status* st) {
     b = block;
   }
   KSS_CUDA(L, cudaStreamSynchronize(L->stream));
+  lease.settled();
   Status s;
   std::memcpy(s.sums, b + 64, sizeof(s.sums));
   std::memcpy(s.counts, b + 128, sizeof(s.counts));
@@ -582,7 +540,7 @@ int finish(kss_lattice* L, const HostLease& lease, Status* st) {
 }
 
 int device_error(kss_lattice* L) {
-  const HostLease lease;
+  HostLease lease(L->stream);
   return finish(L, lease);
 }
 
@@ -879,7 +837,7 @@ int set_fields_of(kss_lattice* L, const E* rho, const E* ux, const E* uy, int on
     u = pinned_device_view(ux);
     v = pinned_device_view(uy);
   }
-  const HostLease lease(!on_device && !(r && u && v));
+  HostLease lease(L->stream, !on_device && !(r && u && v));
   E* const mail = static_cast<E*>(lease.room(3 * n * sizeof(E)));
   if (!on_device && !(r && u && v) && mail) {  // small arrays: through page-locked memory
     std::memcpy(mail, rho, n * sizeof(E));
@@ -910,7 +868,10 @@ int set_fields_of(kss_lattice* L, const E* rho, const E* ux, const E* uy, int on
                return kss::launch_init_equilibrium<S>(r, u, v, f, L->plane, L->pitch, nx, ny,
                                                       codec_of<S>(L), L->stream);
            }));
-  if (!on_device) KSS_CUDA(L, cudaStreamSynchronize(L->stream));
+  if (!on_device) {
+    KSS_CUDA(L, cudaStreamSynchronize(L->stream));
+    lease.settled();
+  }
   return reset_after_set(L);
 }
 }  // namespace
@@ -934,7 +895,7 @@ int kss_set_populations(kss_lattice* L, const double* f, int on_device) {
   DeviceGuard g(L->device);
   const size_t n = 9 * size_t(L->cfg.nx) * L->cfg.ny;
   const double* src = on_device ? f : pinned_device_view(f);
-  const HostLease lease(!src);
+  HostLease lease(L->stream, !src);
   if (double* const mail = src ? nullptr : static_cast<double*>(lease.room(n * 8))) {
     std::memcpy(mail, f, n * 8);
     src = mail;
@@ -951,7 +912,10 @@ int kss_set_populations(kss_lattice* L, const double* f, int on_device) {
                                                  static_cast<S*>(L->f[L->cur]), codec_of<S>(L),
                                                  L->stream);
            }));
-  if (!on_device) KSS_CUDA(L, cudaStreamSynchronize(L->stream));
+  if (!on_device) {
+    KSS_CUDA(L, cudaStreamSynchronize(L->stream));
+    lease.settled();
+  }
   return reset_after_set(L);
 }
 
@@ -961,7 +925,7 @@ int kss_get_populations(kss_lattice* L, double* f, int on_device) {
   if (!f) return fail(L, KSS_ERR_ARG, "null population pointer");
   DeviceGuard g(L->device);
   const size_t n = 9 * size_t(L->cfg.nx) * L->cfg.ny;
-  const HostLease lease;
+  HostLease lease(L->stream);
   double* const mail = on_device ? nullptr : static_cast<double*>(lease.room(n * 8));
   double* dst = mail ? mail : f;
   if (!on_device && !mail) {
@@ -1046,7 +1010,7 @@ int kss_read_moments(kss_lattice* L, double* rho, double* ux, double* uy, int on
   if (!rho || !ux || !uy) return fail(L, KSS_ERR_ARG, "null field pointer");
   DeviceGuard g(L->device);
   const size_t n = size_t(L->cfg.nx) * L->cfg.ny;
-  const HostLease lease;
+  HostLease lease(L->stream);
   double* const mail = on_device ? nullptr : static_cast<double*>(lease.room(3 * n * 8));
   double *r = rho, *u = ux, *v = uy;
   if (!on_device) {
@@ -1084,7 +1048,7 @@ int kss_read_sensor(kss_lattice* L, int32_t sensor, double* out, int on_device) 
   const void* field = nullptr;
   if ((rc = ensure_outputs(L, sensor, &field))) return rc;
   const size_t n = size_t(L->cfg.nx) * L->cfg.ny;
-  const HostLease lease;
+  HostLease lease(L->stream);
   double* const mail = on_device ? nullptr : static_cast<double*>(lease.room(n * 8));
   double* dst = mail ? mail : out;
   if (!on_device && !mail) {
@@ -1115,7 +1079,7 @@ int kss_read_flags(kss_lattice* L, uint8_t* flags, int32_t* tile_counts, int64_t
   const size_t nf = flags ? size_t(L->cfg.nx) * L->cfg.ny : 0;
   const size_t nt = tile_counts ? sizeof(int32_t) * 2 * size_t(L->ntx) * L->nty : 0;
   const size_t at = (nf + 15) / 16 * 16;  // the tile counts' place after the flags
-  const HostLease lease;
+  HostLease lease(L->stream);
   unsigned char* const mail =
       on_device ? nullptr : static_cast<unsigned char*>(lease.room(at + nt));
   if (on_device || mail) {
@@ -1146,7 +1110,7 @@ int kss_read_stats(kss_lattice* L, double sums[3], int64_t counts[3], int64_t* s
   if (rc) return rc;
   DeviceGuard g(L->device);
   if ((rc = ensure_outputs(L, -1, nullptr))) return rc;
-  const HostLease lease;
+  HostLease lease(L->stream);
   Status st;
   if ((rc = finish(L, lease, &st))) return rc;
   if (sums)

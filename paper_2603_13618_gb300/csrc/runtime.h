@@ -10,6 +10,7 @@
 #include <type_traits>
 
 #include "../../include/kss.h"
+#include "host_lease.h"
 #include "launch.h"
 
 // NVTX ranges around the compute entry points (kss_step, kss_batch_step, the adjoint's
@@ -253,24 +254,6 @@ inline int enter(kss_lattice* L) {
 // Free a lattice's device buffers and stream after its stream drains (kss_runtime.cu).
 void release(kss_lattice* L);
 
-// Page-locked host memory that kernels read and write in place, borrowed for the length of
-// one call: the first kMailBytes take the lattice's status block, the rest small arrays on
-// their way from or to pageable memory.  A call that needs it takes a lease from a pool,
-// shared by all threads and lattices, which keeps at most kKeptLeases buffers between calls
-// and frees the others.  `p` is nullptr if page-locked memory could not be had (the calls
-// then copy through the driver as for large arrays).
-struct HostLease {
-  static constexpr size_t kMailBytes = 256, kBytes = size_t(1) << 20;
-  static constexpr int kKeptLeases = 4;
-  unsigned char* p;
-  explicit HostLease(bool wanted = true);
-  ~HostLease();
-  HostLease(const HostLease&) = delete;
-  HostLease& operator=(const HostLease&) = delete;
-  // room for `bytes` of array data, or nullptr
-  void* room(size_t bytes) const { return p && bytes <= kBytes - kMailBytes ? p + kMailBytes : nullptr; }
-};
-
 // A lattice's status block (kss_lattice::small) as of a stream synchronisation.
 struct Status {
   double sums[3];
@@ -280,7 +263,7 @@ struct Status {
 // Wait for the lattice's stream and read its status block, in one synchronisation: a kernel
 // at the end of the queued work writes the block into the lease.  Did a bounded device wait
 // run out?  (sticky)
-int finish(kss_lattice* L, const HostLease& lease, Status* st = nullptr);
+int finish(kss_lattice* L, HostLease& lease, Status* st = nullptr);
 // The same without a status to return.
 int device_error(kss_lattice* L);
 // Evaluate the flags, tile counts, sums and counts of the current step if it had no outputs.
