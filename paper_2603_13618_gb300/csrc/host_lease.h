@@ -11,16 +11,17 @@ namespace kss_rt {
 
 // The first kMailBytes take the lattice's status block, the rest small arrays on their way
 // from or to pageable memory.  A call that needs it takes a lease from a pool, shared by all
-// threads and lattices, which keeps at most kKeptLeases buffers between calls and frees the
-// others.  `p` is nullptr if page-locked memory could not be had (the calls then copy through
-// the driver as for large arrays).
+// threads and lattices, of at most kLeases buffers, made as they are first needed and kept.
+// `p` is nullptr if all are borrowed or page-locked memory could not be had: the call then
+// copies through the driver as for large arrays.  (Making and freeing a buffer in such a call
+// would cost it more than the copies, and freeing one can wait for other streams' work.)
 //
 // Kernels of `stream` use the buffer until the call has waited for the stream (settled).  A
 // call that returns before that, on an error, waits when the lease ends: the next borrower
 // must not find a kernel still writing.  A buffer that cannot be waited for is not handed on.
 struct HostLease {
   static constexpr size_t kMailBytes = 256, kBytes = size_t(1) << 20;
-  static constexpr int kKeptLeases = 4;
+  static constexpr int kLeases = 8;
   unsigned char* p = nullptr;
 
   explicit HostLease(cudaStream_t stream, bool wanted = true) : stream_(stream) {
@@ -32,6 +33,8 @@ struct HostLease {
         p = pool.kept[--pool.n];
         return;
       }
+      if (pool.made == kLeases) return;
+      ++pool.made;
     }
     // (another thread's stream capture is not disturbed by the allocation)
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
@@ -43,22 +46,17 @@ struct HostLease {
     }
     cudaThreadExchangeStreamCaptureMode(&mode);
     p = static_cast<unsigned char*>(q);
+    if (!p) {
+      std::lock_guard<std::mutex> lock(pool.mutex);
+      --pool.made;
+    }
   }
   ~HostLease() {
     if (!p) return;
     if (!settled_ && cudaStreamSynchronize(stream_) != cudaSuccess) return;
     Pool& pool = the_pool();
-    {
-      std::lock_guard<std::mutex> lock(pool.mutex);
-      if (pool.n < kKeptLeases) {
-        pool.kept[pool.n++] = p;
-        return;
-      }
-    }
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    if (cudaFreeHost(p) != cudaSuccess) cudaGetLastError();
-    cudaThreadExchangeStreamCaptureMode(&mode);
+    std::lock_guard<std::mutex> lock(pool.mutex);
+    pool.kept[pool.n++] = p;
   }
   HostLease(const HostLease&) = delete;
   HostLease& operator=(const HostLease&) = delete;
@@ -73,8 +71,8 @@ struct HostLease {
  private:
   struct Pool {
     std::mutex mutex;
-    unsigned char* kept[kKeptLeases] = {};
-    int n = 0;
+    unsigned char* kept[kLeases] = {};
+    int n = 0, made = 0;
   };
   static Pool& the_pool() {
     static Pool pool;

@@ -70,5 +70,28 @@ int main() {
               !a.room(HostLease::kBytes - HostLease::kMailBytes + 1));
     a.settled();
   }
+  // more calls at once than the pool has buffers, three times over
+  constexpr int kCalls = 40;
+  for (int round = 0; round < 3; ++round) {
+    HostLease* lease[kCalls];
+    std::set<unsigned char*> lent;
+    int without = 0;
+    for (auto& l : lease) {
+      l = new HostLease(s);
+      if (l->p) lent.insert(l->p);
+      else ++without;
+      l->settled();
+    }
+    const std::string what = "no buffer is lent twice (" + std::to_string(round) + ")";
+    check(what.c_str(), int(lent.size()) + without == kCalls && without < kCalls);
+    for (auto& l : lease) delete l;
+  }
+  check("calls beyond the pool's size make and free no memory", g_allocs <= 16 && g_frees == 0);
+  g_no_memory = true;
+  {
+    HostLease a(s);
+    check("kept buffers need no new memory", a.p != nullptr);
+    a.settled();
+  }
   return 0;
 }

@@ -30,3 +30,11 @@ def _checks(tmp_path, defines=()):
 def test_buffers_are_handed_on_only_when_nothing_uses_them(tmp_path):
     checks = _checks(tmp_path)
     assert len(checks) >= 6 and set(checks.values()) == {"ok"}, checks
+
+
+def test_the_pool_is_bounded_and_calls_beyond_it_make_and_free_no_memory(tmp_path):
+    checks = _checks(tmp_path)
+    for r in range(3):
+        assert checks[f"no buffer is lent twice ({r})"] == "ok", checks
+    assert checks["calls beyond the pool's size make and free no memory"] == "ok", checks
+    assert checks["kept buffers need no new memory"] == "ok", checks
