@@ -460,6 +460,19 @@ int ensure_outputs(kss_lattice* L, int sensor, const void** field) {
   return KSS_OK;
 }
 
+// kernel<<<grid, threads, 0, stream>>>(args...), returning this launch's own status: the calls
+// below copied through the driver before they had kernels, and an error that the caller's own
+// CUDA calls left behind (cudaGetLastError) is none of theirs.
+template <class... P, class... A>
+cudaError_t launch_alone(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t stream,
+                         A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(unsigned(threads));
+  cfg.stream = stream;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // The status block into page-locked host memory (one CTA of 64 threads, one word each).
 __global__ void status_kernel(const uint32_t* __restrict__ block, uint32_t* __restrict__ mail) {
   mail[threadIdx.x] = block[threadIdx.x];
@@ -494,9 +507,8 @@ cudaError_t launch_flags_out(kss_lattice* L, uint8_t* out, int32_t* tiles_out) {
   auto go = [&](auto width) {
     constexpr int V = decltype(width)::value;
     const dim3 g((nx + 256 * V - 1) / (256 * V), ny < 65535 ? ny : 65535);
-    flags_out_kernel<V><<<g, 256, 0, L->stream>>>(L->flags, L->pitch, nx, ny, out, L->tiles, n,
-                                                  tiles_out);
-    return cudaGetLastError();
+    return launch_alone(flags_out_kernel<V>, g, 256, L->stream, (const uint8_t*)L->flags, L->pitch,
+                        nx, ny, out, (const int32_t*)L->tiles, n, tiles_out);
   };
   // (rows of the pitched plane are 16-byte aligned: its pitch is a multiple of 16 elements)
   if (nx % 16 == 0 && at % 16 == 0) return go(std::integral_constant<int, 16>{});
@@ -512,9 +524,9 @@ int finish(kss_lattice* L, HostLease& lease, Status* st) {
   unsigned char block[HostLease::kMailBytes];
   const unsigned char* b = lease.p;
   if (b) {
-    status_kernel<<<1, 64, 0, L->stream>>>(reinterpret_cast<const uint32_t*>(L->small),
-                                           reinterpret_cast<uint32_t*>(lease.p));
-    KSS_CUDA(L, cudaGetLastError());
+    KSS_CUDA(L, launch_alone(status_kernel, dim3(1), 64, L->stream,
+                             reinterpret_cast<const uint32_t*>(L->small),
+                             reinterpret_cast<uint32_t*>(lease.p)));
   } else {
     KSS_CUDA(L, cudaMemcpyAsync(block, L->small, sizeof(block), cudaMemcpyDeviceToHost, L->stream));
     b = block;
