@@ -188,7 +188,9 @@ int kss_read_sensor(kss_lattice* lat, int32_t sensor, double* out, int on_device
  * tile_counts (int32 [2][nty][ntx], nty = ceil(ny/tile), ntx = ceil(nx/tile): refine
  * then switch tags per tile; ragged edge tiles are partial) and counts[3] = {refine,
  * switch, non-positive}.  Any output pointer may be NULL.  on_device applies to flags
- * and tile_counts; counts is always host memory. */
+ * and tile_counts; counts is always host memory.  Neither pointer needs an alignment
+ * (arrays of this device, tile_counts on a 4-byte boundary, are written by a kernel, any
+ * other by the driver's copy). */
 int kss_read_flags(kss_lattice* lat, uint8_t* flags, int32_t* tile_counts, int64_t counts[3],
                    int on_device);
 
@@ -380,8 +382,8 @@ typedef struct {
 /* On the lattice's flags of its current step (evaluated first if that step had no
  * outputs).  tile_mask: [nty][ntx] bytes or NULL; boxes: up to max_boxes boxes or NULL;
  * *nboxes: the number of boxes (may exceed max_boxes: only max_boxes are written).
- * on_device applies to tile_mask and boxes.  buffer in [0, 1024], efficiency in [0, 1];
- * the tile grid is at most 8192 tiles per side (KSS_ERR_UNSUPPORTED beyond). */
+ * on_device applies to tile_mask and boxes, which need no alignment.  buffer in [0, 1024],
+ * efficiency in [0, 1]; the tile grid is at most 8192 tiles per side (KSS_ERR_UNSUPPORTED beyond). */
 int kss_regrid(kss_lattice* lat, int32_t buffer, double efficiency, uint8_t* tile_mask,
                kss_box* boxes, int32_t max_boxes, int32_t* nboxes, int on_device);
 

@@ -461,8 +461,9 @@ int regrid_run(Workspace& ws, const uint8_t* d_flags, long long pitch, int nx, i
                          efficiency, ws.level[0], ws.level[1], ws.acc, ws.kids, ws.result, ws.cap,
                          ws.count);
   if (e != cudaSuccess) return fail_cuda(e);
-  // the outputs: device arrays are written directly; host ones go through borrowed
-  // page-locked memory (16 bytes for the count, the mask, then boxes) where they fit
+  // the outputs: this device's arrays are written directly; host ones go through borrowed
+  // page-locked memory (16 bytes for the count, the mask, then boxes) where they fit; the
+  // rest through the driver's copy
   static_assert(sizeof(Box) == sizeof(kss_box), "box layout");
   HostLease lease(s);
   const size_t at_boxes = 16 + (size_t(ntiles) + 15) / 16 * 16;
@@ -472,10 +473,14 @@ int regrid_run(Workspace& ws, const uint8_t* d_flags, long long pitch, int nx, i
   int room = wanted;
   uint8_t* mo = nullptr;
   kss_box* bo = nullptr;
-  if (on_device) {
+  int device = 0;
+  if (on_device && (e = cudaGetDevice(&device)) != cudaSuccess) return fail_cuda(e);
+  const bool direct = on_device && kernel_may_write(tile_mask, 1, device) &&
+                      kernel_may_write(boxes, alignof(kss_box), device);
+  if (direct) {
     mo = tile_mask;
     bo = boxes;
-  } else if (mail) {
+  } else if (mail && !on_device) {
     room = std::min<size_t>(wanted, (HostLease::kBytes - HostLease::kMailBytes - at_boxes) / sizeof(Box));
     mo = tile_mask ? mail + 16 : nullptr;
     bo = boxes ? reinterpret_cast<kss_box*>(mail + at_boxes) : nullptr;
@@ -494,18 +499,17 @@ int regrid_run(Workspace& ws, const uint8_t* d_flags, long long pitch, int nx, i
     lease.settled();
   }
   if (count_mail) total = *count_mail;
-  if (!on_device) {
-    const int ncopy = std::min(total, wanted), have = mail ? std::min(ncopy, room) : 0;
+  if (!direct) {
+    const int ncopy = std::min(total, wanted), have = bo ? std::min(ncopy, room) : 0;
     if (mo) std::memcpy(tile_mask, mail + 16, size_t(ntiles));
     if (bo) std::memcpy(boxes, mail + at_boxes, sizeof(Box) * size_t(have));
+    const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     const bool more = boxes && ncopy > have;
-    if (more &&
-        (e = cudaMemcpyAsync(boxes + have, ws.result + have, sizeof(Box) * size_t(ncopy - have),
-                             cudaMemcpyDeviceToHost, s)) != cudaSuccess)
+    if (more && (e = cudaMemcpyAsync(boxes + have, ws.result + have,
+                                     sizeof(Box) * size_t(ncopy - have), kind, s)) != cudaSuccess)
       return fail_cuda(e);
     if (tile_mask && !mo &&
-        (e = cudaMemcpyAsync(tile_mask, ws.mask, size_t(ntiles), cudaMemcpyDeviceToHost, s)) !=
-            cudaSuccess)
+        (e = cudaMemcpyAsync(tile_mask, ws.mask, size_t(ntiles), kind, s)) != cudaSuccess)
       return fail_cuda(e);
     if ((more || (tile_mask && !mo)) && (e = cudaStreamSynchronize(s)) != cudaSuccess)
       return fail_cuda(e);

@@ -520,6 +520,17 @@ cudaError_t launch_flags_out(kss_lattice* L, uint8_t* out, int32_t* tiles_out) {
 
 namespace kss_rt {
 
+bool kernel_may_write(const void* p, size_t align, int device) {
+  if (!p) return true;
+  if (reinterpret_cast<uintptr_t>(p) % align != 0) return false;
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == device;
+}
+
 int finish(kss_lattice* L, HostLease& lease, Status* st) {
   unsigned char block[HostLease::kMailBytes];
   const unsigned char* b = lease.p;
@@ -1094,19 +1105,20 @@ int kss_read_flags(kss_lattice* L, uint8_t* flags, int32_t* tile_counts, int64_t
   HostLease lease(L->stream);
   unsigned char* const mail =
       on_device ? nullptr : static_cast<unsigned char*>(lease.room(at + nt));
-  if (on_device || mail) {
+  if (mail || (on_device && kernel_may_write(flags, 1, L->device) &&
+               kernel_may_write(tile_counts, alignof(int32_t), L->device))) {
     uint8_t* const fo = !flags ? nullptr : mail ? mail : flags;
     int32_t* const to = !tile_counts ? nullptr
                         : mail       ? reinterpret_cast<int32_t*>(mail + at)
                                      : tile_counts;
     if (fo || to) KSS_CUDA(L, launch_flags_out(L, fo, to));
   } else {
+    const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     if (flags)
       KSS_CUDA(L, cudaMemcpy2DAsync(flags, size_t(L->cfg.nx), L->flags, size_t(L->pitch),
-                                    size_t(L->cfg.nx), size_t(L->cfg.ny), cudaMemcpyDeviceToHost,
-                                    L->stream));
+                                    size_t(L->cfg.nx), size_t(L->cfg.ny), kind, L->stream));
     if (tile_counts)
-      KSS_CUDA(L, cudaMemcpyAsync(tile_counts, L->tiles, nt, cudaMemcpyDeviceToHost, L->stream));
+      KSS_CUDA(L, cudaMemcpyAsync(tile_counts, L->tiles, nt, kind, L->stream));
   }
   Status st;
   if ((rc = finish(L, lease, &st))) return rc;

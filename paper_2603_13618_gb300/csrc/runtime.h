@@ -266,6 +266,10 @@ struct Status {
 int finish(kss_lattice* L, HostLease& lease, Status* st = nullptr);
 // The same without a status to return.
 int device_error(kss_lattice* L);
+// May a kernel on `device` write an output of elements of `align` bytes to p (nullptr: not
+// wanted)?  Memory of that device, aligned to its elements; outputs anywhere else (another
+// device's memory, off an element's boundary) go through the driver's copy.
+bool kernel_may_write(const void* p, size_t align, int device);
 // Evaluate the flags, tile counts, sums and counts of the current step if it had no outputs.
 int ensure_flags(kss_lattice* L);
 
