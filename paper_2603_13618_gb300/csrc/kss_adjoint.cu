@@ -383,12 +383,8 @@ int kss_adjoint_create(const kss_adjoint_config* cfg, kss_adjoint** out) {
   A->adj_rows = KSS_ADJ_ROWS ? KSS_ADJ_ROWS : kss::fill_rows(cfg->nx, cfg->ny, 32 * kss::kAdjV, nsm);
   A->step_rows = kss::fill_rows(cfg->nx, cfg->ny, 32 * (A->fp32 ? kss::Vec<float>::N : kss::Vec<double>::N), nsm);
   const dim3 g = kss::adj_grid(cfg->nx, cfg->ny, A->adj_rows);
-  // one row per warp, or up to four where the reverse step still has four waves of warps (28
-  // per SM)
   A->twice = cfg->precision == KSS_FP32 && kss::can_step_twice<float>(cfg->nx, cfg->ny);
-  while (A->rev_rows < 4 &&
-         kss::adj_reverse_parts(cfg->nx, cfg->ny, 2 * A->rev_rows) >= 4LL * 28 * nsm)
-    A->rev_rows *= 2;
+  A->rev_rows = kss::adj_reverse_rows(cfg->nx, cfg->ny, nsm);
   A->nparts = kss::adj_reverse_parts(cfg->nx, cfg->ny, A->rev_rows);
   struct {
     void** p;

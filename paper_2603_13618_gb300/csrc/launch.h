@@ -138,12 +138,21 @@ cudaError_t launch_adj_objective(const AdjParams<T>& p, cudaStream_t stream);
 // reverse step of the segment, and nothing else writes the state p.f.
 inline dim3 adj_reverse_grid(int nx, int ny, int rows) {
   return dim3((unsigned)((nx + 32 * kAdjV - 1) / (32 * kAdjV)),
-              (unsigned)((ny + kAdjWarps * rows - 1) / (kAdjWarps * rows)), 1u);
+              (unsigned)((ny - 1) / (kAdjWarps * rows) + 1), 1u);
 }
 // (the partials of one step: a double per warp)
 inline long long adj_reverse_parts(int nx, int ny, int rows) {
   const dim3 g = adj_reverse_grid(nx, ny, rows);
   return (long long)g.x * g.y * kAdjWarps;
+}
+// Rows per warp of a reverse step: one, or up to four where that still leaves four waves of
+// warps (28 per SM); more only where the grid's 65535 CTAs along y would not hold the rows
+// (four: 1 048 560).
+inline int adj_reverse_rows(int nx, int ny, int nsm) {
+  int rows = 1;
+  while (rows < 4 && adj_reverse_parts(nx, ny, 2 * rows) >= 4LL * 28 * nsm) rows *= 2;
+  while (adj_reverse_grid(nx, ny, rows).y > 65535u) rows *= 2;
+  return rows;
 }
 template <class T>
 cudaError_t launch_adj_reverse(const AdjParams<T>& p, bool chained, cudaStream_t stream);
