@@ -301,11 +301,13 @@ cudaError_t launch_step<KSS_T>(const StepParams<KSS_T>& p, int mode, bool pull, 
 
 template <>
 bool can_step_twice<KSS_T>(int nx, int ny) {
-  return std::is_same<KSS_T, float>::value && (ny + kTwiceRows - 1) / kTwiceRows <= 65535 && nx > 0;
+  return KSS_STEP_TWICE && std::is_same<KSS_T, float>::value &&
+         (ny + kTwiceRows - 1) / kTwiceRows <= 65535 && nx > 0;
 }
 
 template <class S>
 cudaError_t launch_twice(const StepParams<S>& p, S* mid, cudaStream_t stream) {
+#if KSS_STEP_TWICE
   if constexpr (std::is_same<S, float>::value) {
     constexpr auto kern = step_plain_twice_kernel<kTwiceRows>;
     constexpr int dyn = 9 * (kTwiceRows + 2) * kTwicePitch * int(sizeof(float));
@@ -315,6 +317,7 @@ cudaError_t launch_twice(const StepParams<S>& p, S* mid, cudaStream_t stream) {
     kern<<<g, 32 * (kTwiceRows + 3), dyn, stream>>>(p, mid);
     return cudaGetLastError();
   }
+#endif
   return cudaErrorInvalidValue;
 }
 

@@ -2448,7 +2448,10 @@ __device__ __forceinline__ void split_block(const StepParams<S>& p, const int bx
   constexpr bool kH8 = VC == 8, FULL = MODE == MODE_FULL, kF64 = std::is_same<S, double>::value;
   constexpr bool kHalfPaired = KSS_ROW_PAIRED && std::is_same<S, __half>::value && !FULL &&
                                !AAR && PULL && V == 4;
-  static_assert(MODE != MODE_PLAIN && (VC == V || (kH8 && kHalfPaired && STORE)), "split steps");
+  static_assert(MODE != MODE_PLAIN &&
+                    (VC == V || (kH8 && std::is_same<S, __half>::value && MODE == MODE_STD &&
+                                 PULL && STORE && !AAR && KSS_ROW_PAIRED)),
+                "split steps");
   constexpr int kVals = split_vals<S, MODE, VC>();
   constexpr int kCells = kF64 ? 1 : VC;   // cells per lane of a row
   constexpr int kShare = VC / kCells;     // warps per row
@@ -2764,6 +2767,10 @@ __global__ void __launch_bounds__(128) step_plain_f64_kernel(const StepParams<do
                                                            unused[2], mbits);
 }
 
+// The kernel below is written for the paired row of four cells per lane; builds that choose
+// another (KSS_ROW_PAIRED=0, KSS_F32_VEC=2) step once per launch.
+#define KSS_STEP_TWICE (KSS_ROW_PAIRED && KSS_F32_VEC == 4)
+#if KSS_STEP_TWICE
 // Two plain FP32 steps of a tile of 128 columns x H rows in one launch: the first over the
 // tile and the cells around it (one warp per row, and one warp for the columns x0 - 1 and
 // x0 + 128), into shared memory, the second from there.  mid: the state in between, of the
@@ -2856,6 +2863,7 @@ __global__ void __launch_bounds__(32 * (H + 3), 2) step_plain_twice_kernel(const
   fused_row_paired<float, MODE_PLAIN, true>(p, f, i0, y0 + warp, cv, unused[0], unused[1],
                                             unused[2]);
 }
+#endif  // KSS_STEP_TWICE
 
 // ---------------------------------------------------------------- multi-step ----
 // nsteps steps in one cooperative launch (every CTA resident).  The (step, block) work
