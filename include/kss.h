@@ -175,13 +175,19 @@ int kss_get_populations(kss_lattice* lat, double* f, int on_device);
  * stream; errors of the launches are reported here or by the next call. */
 int kss_step(kss_lattice* lat, int32_t nsteps);
 
-/* rho, ux, uy of the stored state (Eqs. eq_quadratur1-2), nx*ny doubles each. */
+/* rho, ux, uy of the stored state (Eqs. eq_quadratur1-2), nx*ny doubles each: FP64 sums
+ * of the stored populations and their quotients (of FP32 and FP16 states each quotient is
+ * the IEEE one or, in about one of 2^32 cases, its neighbour). */
 int kss_read_moments(kss_lattice* lat, double* rho, double* ux, double* uy, int on_device);
 
 /* Sensor field (nx*ny doubles) of the pre-collision populations of the most recent
  * step, or of the stored populations if no step was taken since the last set.  A
  * field recorded on that step is returned as stored; any other is evaluated on
- * demand from the population buffer the step read. */
+ * demand from the population buffer the step read.
+ * The same calls on the same lattice give the same bits.  On FP64 lattices the terms of the
+ * KL field's series that are summed depend on the largest |f^neq / f^eq| among the 64
+ * columns around the cell, those left out being below 2^-54 of what is summed: the same cell
+ * in a lattice of another width, or shifted in x, may differ in the last bits. */
 int kss_read_sensor(kss_lattice* lat, int32_t sensor, double* out, int on_device);
 
 /* Tags of the same state as kss_read_sensor: flags (nx*ny bytes, KSS_FLAG_*),
@@ -435,10 +441,10 @@ int kss_adjoint_forward(kss_adjoint* adj, const double* rho0, const double* ux0,
 int kss_adjoint_backward(kss_adjoint* adj, double* grad_rho0, double* grad_tau, int on_device);
 
 const char* kss_adjoint_last_error(const kss_adjoint* adj);
-/* How the reverse sweep runs (no counterpart in the paper): on = 1 (the default)
- * recomputes each segment's states beside the reverse steps of the segment before it, on a
- * branch of its own of the recorded graph; on = 0 after them.  The gradients are the same
- * bit for bit.  KSS_ERR_ARG for another value. */
+/* How the reverse sweep runs (no counterpart in the paper), always one launch per reverse
+ * step (the name is older than that): on = 1 (the default) recomputes each segment's states
+ * beside the reverse steps of the segment before it, on a branch of its own of the recorded
+ * graph; on = 0 after them.  The gradients are the same bit for bit.  KSS_ERR_ARG for another value. */
 int kss_adjoint_set_multistep(kss_adjoint* adj, int on);
 
 /* ---- Allocation-free fused step (no counterpart in the paper) ----------------------

@@ -398,11 +398,10 @@ __device__ __forceinline__ void adj_step_row(const AdjParams<T>& p, int j, int i
 // chained (launch_chained): a warp pulls the forward state, which no launch of the segment
 // writes, before it waits for the previous reverse step, so that only the adjoint's own
 // loads follow that wait.  The sums are added after the segment (adj_iteration_totals).
-// FP32 takes 72 registers, so that the 4096 warps of a 512^2 step run at once (28 per SM).
+// FP32 takes 69 registers, so that the 4096 warps of a 512^2 step run at once (28 per SM).
 // One launch for a whole segment, whose blocks waited on their neighbours' previous step
 // through counters in memory, took 8.1 us per 512^2 step (the chain of a block's waits,
-// loads, stores, fence and release); a chained launch
-// takes 4.0.
+// loads, stores, fence and release); a chained launch takes 4.0.
 constexpr int kAdjWarps = 4;
 template <class T>
 __global__ void __launch_bounds__(32 * kAdjWarps, std::is_same<T, float>::value ? 7 : 4)

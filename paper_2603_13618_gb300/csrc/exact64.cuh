@@ -2,7 +2,10 @@
 // FP64 operations per clock (conversions to and from FP64 included) against 64 integer and
 // 128 FP32 ones, so the boundary kernels, which hand FP32 and FP16 states out as FP64
 // arrays, are bound by that pipe and not by memory when they convert, add and divide in FP64.
-// Everything here gives the value that the FP64 instruction sequence gives.
+// Conversions and sums here give the value that the FP64 instructions give.  Quotients and
+// reciprocals are rounded once, from a value within 2^-86 of the exact one: they are the IEEE
+// result except where the exact value lies within 2^-33 of a unit in the last place from the
+// middle of two FP64 numbers (about one in 2^32 of them), where they may be the other of the two.
 #pragma once
 
 #include <cstdint>
@@ -20,7 +23,7 @@ __device__ __forceinline__ double widen(float x) {
 }
 __device__ __forceinline__ double widen(double x) { return x; }
 
-// The rounded quotient j / r of two integers, |j| and 0 < r below 2^53 (jd, rd: the
+// The quotient j / r (rounded as above) of two integers, |j| and 0 < r below 2^53 (jd, rd: the
 // magnitudes scaled into [1, 2), yd about 1 / rd): q0 = jd yd, then one correction by the
 // remainder (Markstein, "Computation of elementary functions on the IBM RISC System/6000
 // processor", 1990).  yd is within 2^-43 of 1 / rd, so the corrected quotient is within
@@ -47,7 +50,7 @@ __device__ __forceinline__ double reciprocal46(uint64_t frac) {
   return __longlong_as_double((y & ((1ll << 52) - 1)) | (1022ll << 52));
 }
 
-// 1 / x rounded: reciprocal46 and one FP64 Newton step, which leaves 2^-86 before its
+// 1 / x (rounded as above): reciprocal46 and one FP64 Newton step, which leaves 2^-86 before its
 // rounding (two operations of the FP64 pipe; the compiler's division takes about ten).
 // Exponents near the ends of the range, zero, infinities and NaN take the division.
 __device__ __forceinline__ double rcp64(double x) {
@@ -63,7 +66,7 @@ __device__ __forceinline__ double rcp64(double x) {
                           __double2loint(y));
 }
 
-// n / d rounded, for d positive and of ordinary size (2^-1000 < d < 2^1000; other d give
+// n / d (rounded as above), for d positive and of ordinary size (2^-1000 < d < 2^1000; other d give
 // some number or NaN): three operations of the FP64 pipe.
 __device__ __forceinline__ double ratio64(double n, double d) {
   const uint64_t b = uint64_t(__double_as_longlong(d));
@@ -73,8 +76,8 @@ __device__ __forceinline__ double ratio64(double n, double d) {
                                          __double2loint(y)));
 }
 
-// rho = sum v, ux = jx / rho and uy = jy / rho of nine FP32 populations as FP64 arithmetic
-// gives them.  Where the populations are positive and their exponents span at most 25, the
+// rho = sum v, ux = jx / rho and uy = jy / rho of nine FP32 populations: the sums of FP64
+// arithmetic, and their quotients rounded as above.  Where the populations are positive and their exponents span at most 25, the
 // moments are integers below 2^53 in units of the smallest population's last place: every
 // FP64 partial sum is exact, and so are these integer sums.  Other cells return false.
 __device__ __forceinline__ bool moments_exact(const float (&v)[9], double& rho, double& ux,

@@ -403,7 +403,9 @@ int steps_graph(kss_lattice* L, int nsteps) {
 // launches) rather than as one multi-step launch?  Where each block is shared out to several
 // CTAs; and with FP32 storage where the blocks are at most one wave of two CTAs per SM, so
 // that the multi-step launch has no wave of its own to overlap and only its waits to pay:
-// 1024^2 (256 blocks) 20.3 against 22.2 us per step, 1280^2 (400) 30.9 against 28.2.
+// 1024^2 (256 blocks) 20.3 against 22.2 us per step, 1280^2 (400) 30.9 against 28.2; with the
+// two-relaxation model 800^2 (175 blocks) 20.8 against 23.9, 1024^2 21.6 against 24.5, 1536x800
+// (300) 22.3 against 25.1.
 bool one_launch_per_step(const kss_lattice* L) {
   if (L->cfg.precision == KSS_FP32 && L->nblocks <= 2 * L->nsm) return true;
   return with_storage(L->cfg.precision, [&](auto tag) {
@@ -979,8 +981,8 @@ int kss_step(kss_lattice* L, int32_t nsteps) {
     return fail(L, KSS_ERR_CUDA, "injected launch failure (kss_testing_fail_after)");
   DeviceGuard g(L->device);
   // several output steps of the {Kn, KL, neq} set on FP32 or FP64 storage, of a lattice above
-  // the line of one_launch_per_step: one multi-step launch (measured on GB300 at 4096^2 FP32: 0.232 vs 0.244 ms per step; plain steps and
-  // FP16-deviation storage gain nothing from it: 0.179 vs 0.179, 0.224 vs 0.221 ms)
+  // the line of one_launch_per_step: one multi-step launch (4096^2 FP32: 0.203 vs 0.216 ms per step;
+  // FP16-deviation storage gains nothing from it: 0.224 vs 0.221 ms)
   const int every = L->cfg.output_every;
   const int mode =
       every == 1 ? mode_for(needed_mask(L, L->cfg.record_mask), L->region != nullptr) : MODE_PLAIN;

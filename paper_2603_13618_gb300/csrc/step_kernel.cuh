@@ -558,6 +558,9 @@ struct StdAcc {
 // N = 6 for |x| < 2^-10, 8 for 2^-7, 15 for 2^-4, 24 for 2^-2.  keep[k] returns whether cell
 // k has |x| < 1/4 throughout; the others are deferred (with cells up to Kn = 1/16 only, the
 // exact recomputation of the cells around a density step took 20 to 30 us per 64^2 step).
+// A cell's last bits so depend on the other cells of its group of 64 columns.  With an order
+// per cell they would not, but the warps of a density step then run several of the series: 64^2
+// 26.8 -> 33.7 us per step, 512^2 211 -> 440.
 constexpr int kPhiF64Orders[4] = {6, 8, 15, 24};
 template <int N, int V>
 __device__ __forceinline__ void kl_sum_f64(StdAcc<double, V>& a) {
