@@ -399,15 +399,27 @@ int steps_graph(kss_lattice* L, int nsteps) {
   return KSS_OK;
 }
 
-// Do runs of output steps of this lattice go as one launch per step (a graph of chained
-// launches) rather than as one multi-step launch?  Where each block is shared out to several
-// CTAs; and with FP32 storage where the blocks are at most one wave of two CTAs per SM, so
-// that the multi-step launch has no wave of its own to overlap and only its waits to pay:
-// 1024^2 (256 blocks) 20.3 against 22.2 us per step, 1280^2 (400) 30.9 against 28.2; with the
-// two-relaxation model 800^2 (175 blocks) 20.8 against 23.9, 1024^2 21.6 against 24.5, 1536x800
-// (300) 22.3 against 25.1.
-bool one_launch_per_step(const kss_lattice* L) {
-  if (L->cfg.precision == KSS_FP32 && L->nblocks <= 2 * L->nsm) return true;
+// Does a run of nsteps output steps of this lattice go as one launch per step (a graph of
+// chained launches) rather than as one multi-step launch?  Where each block is shared out to
+// several CTAs; and with FP32 storage where the blocks are at most one wave of two CTAs per SM,
+// so that the multi-step launch has no wave of its own to overlap and only its waits to pay
+// (us per step of 20, one launch per step / multi-step): 1024^2 (256 blocks) 20.0 / 22.2,
+// 768x1344 in 64-row blocks (126) 26.6 / 26.9, above the line 1280^2 (400) 30.9 / 28.2; with the
+// two-relaxation model 800^2 (175) 20.8 / 23.9, 1024^2 21.1 / 24.4, 1536x800 (300) 22.3 / 25.1.
+// Longer runs (from 8 steps; 2 and 4 are faster as launches everywhere) of lattices whose blocks
+// wait on few others keep the multi-step launch where a step has more blocks than SMs, of which
+// its launch would wait for the few SMs with two: one row of blocks (20000x20, 157 blocks, 14.8 /
+// 12.0; 38000x16, 297, 13.5 / 12.3), and tall lattices of up to 9/8 blocks per SM (1x4900, 154
+// blocks, 15.6 / 12.8; 768x832, 156, 21.4 / 19.0; 832x768, 168, 19.8 / 20.0; 640x1216, 190, 21.8 /
+// 22.0), with the two-relaxation model one column of blocks (100x5000 30.4 / 27.9; 768x832 22.1 /
+// 22.8).
+bool one_launch_per_step(const kss_lattice* L, int nsteps) {
+  if (L->cfg.precision == KSS_FP32 && L->nblocks <= 2 * L->nsm) {
+    const int gx = int(kss::step_grid<float>(L->cfg.nx, L->cfg.ny, L->cfg.tile, L->bands).x);
+    const int gy = L->nblocks / gx;
+    const bool few = 8 * L->nblocks <= 9 * L->nsm && (L->region ? gx == 1 : gy >= 4 * gx);
+    return nsteps < 8 || L->nblocks <= L->nsm || !(gy == 1 || few);
+  }
   return with_storage(L->cfg.precision, [&](auto tag) {
     return kss::split_ranks<typename decltype(tag)::type>(L->nblocks, L->cfg.tile * L->bands) > 0;
   });
@@ -988,7 +1000,7 @@ int kss_step(kss_lattice* L, int32_t nsteps) {
       every == 1 ? mode_for(needed_mask(L, L->cfg.record_mask), L->region != nullptr) : MODE_PLAIN;
   if (KSS_MULTISTEP && nsteps >= 2 && every == 1 && mode == MODE_STD &&
       (KSS_MULTISTEP_F16 || L->cfg.precision != KSS_FP16DEV) &&
-      (L->region || !use_tma(L, mode)) && !one_launch_per_step(L) &&
+      (L->region || !use_tma(L, mode)) && !one_launch_per_step(L, nsteps) &&
       (long long)nsteps * L->nblocks < (1LL << 30)) {
     KSS_CUDA(L, with_storage(L->cfg.precision, [&](auto tag) {
                return launch_multi<typename decltype(tag)::type>(L, mode, nsteps);

@@ -158,6 +158,32 @@ def test_multi_step_launch_of_ragged_lattices(kss, sms, precision, nx, ny, switc
     b.close()
 
 
+@pytest.mark.parametrize("nx,ny", [(33, 4987), (1, 4900), (20011, 17), (38000, 1), (765, 832)])
+@pytest.mark.parametrize("tau2", [0.0, 1.4])
+def test_long_runs_of_strips(kss, sms, nx, ny, tau2):
+    """FP32 lattices of one row of blocks, or tall ones of slightly more blocks than SMs: runs of
+    8 steps and more are one multi-step launch, shorter ones a launch per step."""
+    from paper_2603_13618_gb300 import inputs
+
+    n = blocks("fp32", nx, ny)
+    assert sms < n <= 2 * sms and not splits("fp32", n, 32, sms)
+    assert -(-ny // 32) == 1 or (8 * n <= 9 * sms and -(-ny // 32) >= 4 * -(-nx // 128))
+    fields = inputs.smooth_jump(nx, ny, seed=9, kmax=1)
+    kw = dict(precision="fp32", tau=0.62, record=("kl",), tau2=tau2)
+    a, b = kss.Lattice(nx, ny, **kw), kss.Lattice(nx, ny, **kw)
+    for x in (a, b):
+        x.set_fields(*fields)
+    for steps in (9, 7, 8):
+        a.step(steps)
+        for _ in range(steps):
+            b.step(1)
+        assert_equal(outputs(a), outputs(b))
+        if tau2:
+            np.testing.assert_array_equal(a.get_aar_region(), b.get_aar_region())
+    a.close()
+    b.close()
+
+
 # ---- multi-step launches of a batch against one launch per step ----
 MEMBERS = [dict(nx=37, ny=21, tau=0.7), dict(nx=130, ny=67, tau=1.0), dict(nx=1, ny=5, tau=0.8),
            dict(nx=200, ny=9, tau=0.6), dict(nx=1021, ny=1037, tau=0.9), dict(nx=5, ny=1, tau=1.3),
