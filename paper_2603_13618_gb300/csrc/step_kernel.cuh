@@ -54,7 +54,10 @@ namespace kss {
 //   KSS_F64_MIN_BLOCKS   FP64 {Kn, KL, neq} steps, which keep all nine ratios of a row: two
 //                        (2048^2: 1.88 / 1.75 / 1.81 ms at one / two / three).
 //   KSS_F16_MIN_BLOCKS   FP16-deviation {Kn, KL, neq} steps: three (0.659 ms per 8192^2 step
-//                        against 0.706 ms at two: its 8-byte rows need more warps in flight).
+//                        against 0.706 ms at two: its 8-byte rows need more warps in flight);
+//                        two with the two-relaxation model, whose rows spill 200 to 340 bytes at
+//                        three (us per step at three / two: 700x1500 32.5 / 23.2, 2048^2 75.5 /
+//                        67.5, a batch of four 1021x1037 lattices 88.4 / 77.3).
 //   KSS_FULL_MIN_BLOCKS  the all-sensor steps with FP32 arithmetic: four CTAs at 64 registers
 //                        (2048^2 FP32, all of Table 1: 217 / 189 / 179 / 195 us at two /
 //                        three / four / five; the strain sensor alone: 114 / 96 / 80 / 86 us).
@@ -86,10 +89,11 @@ namespace kss {
 #define KSS_H8_MIN_BLOCKS (KSS_H8_WARPS == 4 ? 5 : 2)
 #endif
 
-// The knob of a step kernel with storage S and sensor set MODE.
-template <class S, int MODE>
+// The knob of a step kernel with storage S and sensor set MODE (AAR: two-relaxation steps).
+template <class S, int MODE, bool AAR = false>
 __host__ __device__ constexpr int step_min_blocks() {
-  return MODE == MODE_FULL ? (std::is_same<S, double>::value ? 2 : KSS_FULL_MIN_BLOCKS)
+  return AAR && MODE == MODE_STD ? 2
+         : MODE == MODE_FULL ? (std::is_same<S, double>::value ? 2 : KSS_FULL_MIN_BLOCKS)
          : std::is_same<S, float>::value ? KSS_F32_MIN_BLOCKS
          : (std::is_same<S, double>::value && MODE == MODE_STD) ? KSS_F64_MIN_BLOCKS
          : (std::is_same<S, __half>::value && MODE == MODE_STD) ? KSS_F16_MIN_BLOCKS
@@ -2262,7 +2266,7 @@ __device__ __forceinline__ void step_cta(const StepParams<S>& p, const int bx, c
 template <class S, int MODE, bool PULL, bool STORE, bool AAR = false, bool PF = false,
           int VC = Vec<S>::N, int NW = kWarps>
 __global__ void __launch_bounds__(32 * NW, VC == 8 ? KSS_H8_MIN_BLOCKS
-                                                   : step_min_blocks<S, MODE>())
+                                                   : step_min_blocks<S, MODE, AAR>())
 step_kernel(const StepParams<S> p) {
   if (MODE != MODE_PLAIN) {
     previous_done();
@@ -3019,7 +3023,7 @@ struct BatchItem {
 // AAR: members with a region take the two-relaxation collision there (members without
 // one step as BGK).
 template <class S, int MODE, bool AAR = false>
-__global__ void __launch_bounds__(kThreads, MODE == MODE_FULL ? 2 : step_min_blocks<S, MODE>())
+__global__ void __launch_bounds__(kThreads, MODE == MODE_FULL ? 2 : step_min_blocks<S, MODE, AAR>())
 batch_step_kernel(const StepParams<S>* __restrict__ table, const BatchItem* __restrict__ items,
                   int nitems) {
   static_assert(sizeof(StepParams<S>) % 8 == 0, "parameter copy in 8-byte words");
