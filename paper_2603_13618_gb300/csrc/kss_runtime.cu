@@ -413,7 +413,10 @@ int steps_graph(kss_lattice* L, int nsteps) {
 // blocks, 15.6 / 12.8; 768x832, 156, 21.4 / 19.0; 832x768, 168, 19.8 / 20.0; 640x1216, 190, 21.8 /
 // 22.0), with the two-relaxation model one column of blocks (100x5000 30.4 / 27.9; 768x832 22.1 /
 // 22.8).
+// FP64 lattices of at most one block per SM, all of whose blocks run at once: a launch per step
+// (per step of 40, 144 blocks of a developed density step, 226 / 290; smooth fields 127 / 125).
 bool one_launch_per_step(const kss_lattice* L, int nsteps) {
+  if (L->cfg.precision == KSS_FP64 && L->nblocks <= L->nsm) return true;
   if (L->cfg.precision == KSS_FP32 && L->nblocks <= 2 * L->nsm) {
     const int gx = int(kss::step_grid<float>(L->cfg.nx, L->cfg.ny, L->cfg.tile, L->bands).x);
     const int gy = L->nblocks / gx;

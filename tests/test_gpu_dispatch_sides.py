@@ -36,10 +36,13 @@ def blocks(precision, nx, ny, rows=32):
 
 def splits(precision, nblocks, rows, sms):
     """Do `nblocks` blocks of `rows` rows go as split blocks?  Their ranks of eight rows (FP32
-    arithmetic: or sixteen, at two rows per warp) must fit at two CTAs per SM."""
+    arithmetic: or sixteen, at two rows per warp) must fit at two CTAs per SM; of FP64, half as
+    many again."""
+    if precision == "fp64":
+        return nblocks * (rows // 8) <= 3 * sms
     if nblocks * (rows // 8) <= 2 * sms:
         return rows > 8
-    return precision != "fp64" and rows > 16 and nblocks * (rows // 16) <= 2 * sms
+    return rows > 16 and nblocks * (rows // 16) <= 2 * sms
 
 
 def outputs(lat, sums=True):
@@ -57,11 +60,15 @@ def assert_equal(a, b):
 # ---- split blocks of a lone lattice against one CTA per block ----
 @pytest.mark.parametrize("precision", ["fp32", "fp64", "fp16dev"])
 @pytest.mark.parametrize("tile", [8, 16, 32, 64])
-@pytest.mark.parametrize("nx,ny", [(1, 1), (33, 2), (128, 8), (130, 31), (257, 33), (300, 65)])
+@pytest.mark.parametrize("nx,ny", [(1, 1), (33, 2), (128, 8), (130, 31), (257, 33), (300, 65),
+                                   (600, 320)])
 def test_split_lattice_against_unsplit_blocks(kss, sms, precision, tile, nx, ny):
     from paper_2603_13618_gb300 import inputs
 
-    assert splits(precision, blocks(precision, nx, ny, max(32, tile)), max(32, tile), sms)
+    n = blocks(precision, nx, ny, max(32, tile))
+    if (nx, ny) == (600, 320) and precision == "fp64" and tile < 64:
+        assert 2 * sms < n * 4 <= 3 * sms  # (beyond the line of the other storage types)
+    assert splits(precision, n, max(32, tile), sms)
     fields = inputs.smooth_jump(nx, ny, seed=5, kmax=2)
     kw = dict(precision=precision, tau=0.56, tile=tile, record=("kl",))
     batch = kss.Batch([dict(nx=nx, ny=ny)], **kw)
@@ -121,7 +128,7 @@ def test_sums_of_split_fp16_blocks(kss, nx, ny):
 
 # ---- multi-step launches of a lone lattice against single steps ----
 @pytest.mark.parametrize("precision,nx,ny", [("fp32", 1537, 1203), ("fp32", 2051, 1037),
-                                             ("fp64", 515, 389)])
+                                             ("fp64", 515, 719), ("fp64", 515, 445)])
 @pytest.mark.parametrize("switch", ["neq", "qe", None])
 def test_multi_step_launch_of_ragged_lattices(kss, sms, precision, nx, ny, switch):
     """Ragged widths, partial last blocks, the seam of an odd width.  switch: the sensor that
@@ -130,7 +137,11 @@ def test_multi_step_launch_of_ragged_lattices(kss, sms, precision, nx, ny, switc
     from paper_2603_13618_gb300 import inputs
 
     n = blocks(precision, nx, ny)
-    assert not splits(precision, n, 32, sms) and (precision != "fp32" or n > 2 * sms)
+    assert not splits(precision, n, 32, sms)
+    if precision == "fp32":
+        assert n > 2 * sms
+    else:  # (FP64 lattices of at most one block per SM take a launch per step)
+        assert n > sms if ny == 719 else n <= sms
     fields = inputs.smooth_jump(nx, ny, seed=nx, kmax=6)
     kw = dict(precision=precision, tau=0.62, record=("kl",) if switch is None else ("kl", "qe"))
     if switch:
