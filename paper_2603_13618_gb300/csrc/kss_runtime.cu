@@ -343,6 +343,13 @@ cudaError_t launch_steps(kss_lattice* L, int nsteps, cudaStream_t s) {
   return e;
 }
 
+// Is the lattice's stream under capture?
+bool under_capture(const kss_lattice* L) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(L->stream, &st) != cudaSuccess) cudaGetLastError();
+  return st == cudaStreamCaptureStatusActive;
+}
+
 // The next nsteps >= 2 steps from buffer L->cur, one launch each, as one replayed CUDA
 // graph: a small lattice's steps are a few microseconds each, about the launch overhead.
 // The graph is recorded on the lattice's capture stream for a (step count, buffer, output
@@ -353,13 +360,9 @@ cudaError_t launch_steps(kss_lattice* L, int nsteps, cudaStream_t s) {
 // A stream under capture takes no graph launch, and its caller keeps the launches anyway: a
 // run of output steps is launched directly into it.
 int steps_graph(kss_lattice* L, int nsteps) {
-  if (L->cfg.output_every == 1) {
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(L->stream, &st) != cudaSuccess) cudaGetLastError();
-    if (st == cudaStreamCaptureStatusActive) {
-      KSS_CUDA(L, launch_steps(L, nsteps, L->stream));
-      return KSS_OK;
-    }
+  if (L->cfg.output_every == 1 && under_capture(L)) {
+    KSS_CUDA(L, launch_steps(L, nsteps, L->stream));
+    return KSS_OK;
   }
   const int64_t phase = L->cfg.output_every > 0 ? L->step % L->cfg.output_every : 0;
   kss_lattice::PlainGraph* slot = nullptr;
@@ -421,7 +424,9 @@ bool one_launch_per_step(const kss_lattice* L, int nsteps) {
     const int gx = int(kss::step_grid<float>(L->cfg.nx, L->cfg.ny, L->cfg.tile, L->bands).x);
     const int gy = L->nblocks / gx;
     const bool few = 8 * L->nblocks <= 9 * L->nsm && (L->region ? gx == 1 : gy >= 4 * gx);
-    return nsteps < 8 || L->nblocks <= L->nsm || !(gy == 1 || few);
+    if (nsteps < 8 || L->nblocks <= L->nsm || !(gy == 1 || few)) return true;
+    // (the multi-step launch's workspace cannot be made while the stream is captured)
+    return !L->multi && under_capture(L);
   }
   return with_storage(L->cfg.precision, [&](auto tag) {
     return kss::split_ranks<typename decltype(tag)::type>(L->nblocks, L->cfg.tile * L->bands) > 0;

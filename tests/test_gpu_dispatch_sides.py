@@ -253,3 +253,31 @@ def test_autotune_times_the_multi_step_launch(kss, sms, tmp_path):
         assert_equal(outputs(a[k]), outputs(b[k]))
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("precision,nx,ny", [("fp32", 20011, 17), ("fp32", 33, 4987),
+                                             ("fp64", 515, 445), ("fp64", 600, 320)])
+@pytest.mark.parametrize("long_before", [False, True])
+def test_long_runs_under_capture(kss, precision, nx, ny, long_before):
+    """A run recorded into the caller's graph equals the call, whether or not the lattice has
+    taken a run of that length before (whose workspace could not be made under capture)."""
+    import torch
+    from paper_2603_13618_gb300 import inputs
+
+    fields = inputs.smooth_jump(nx, ny, seed=9, kmax=1)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        a = kss.Lattice(nx, ny, precision=precision, tau=0.6, record=("kl",))
+        b = kss.Lattice(nx, ny, precision=precision, tau=0.6, record=("kl",))
+        for x in (a, b):
+            x.set_fields(*fields)
+            x.step(10 if long_before else 3)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            a.step(10)
+        graph.replay()
+        b.step(10)
+        assert_equal(outputs(a), outputs(b))
+        a.close()
+        b.close()
