@@ -389,7 +389,8 @@ typedef struct {
  * outputs).  tile_mask: [nty][ntx] bytes or NULL; boxes: up to max_boxes boxes or NULL;
  * *nboxes: the number of boxes (may exceed max_boxes: only max_boxes are written).
  * on_device applies to tile_mask and boxes, which need no alignment.  buffer in [0, 1024],
- * efficiency in [0, 1]; the tile grid is at most 8192 tiles per side (KSS_ERR_UNSUPPORTED beyond). */
+ * efficiency in [0, 1]; the tile grid is at most 8192 tiles per side (KSS_ERR_UNSUPPORTED
+ * beyond). */
 int kss_regrid(kss_lattice* lat, int32_t buffer, double efficiency, uint8_t* tile_mask,
                kss_box* boxes, int32_t max_boxes, int32_t* nboxes, int on_device);
 
@@ -444,7 +445,8 @@ const char* kss_adjoint_last_error(const kss_adjoint* adj);
 /* How the reverse sweep runs (no counterpart in the paper), always one launch per reverse
  * step (the name is older than that): on = 1 (the default) recomputes each segment's states
  * beside the reverse steps of the segment before it, on a branch of its own of the recorded
- * graph; on = 0 after them.  The gradients are the same bit for bit.  KSS_ERR_ARG for another value. */
+ * graph; on = 0 after them.  The gradients are the same bit for bit.  KSS_ERR_ARG for
+ * another value. */
 int kss_adjoint_set_multistep(kss_adjoint* adj, int on);
 
 /* ---- Allocation-free fused step (no counterpart in the paper) ----------------------

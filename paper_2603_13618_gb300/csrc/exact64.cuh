@@ -77,9 +77,10 @@ __device__ __forceinline__ double ratio64(double n, double d) {
 }
 
 // rho = sum v, ux = jx / rho and uy = jy / rho of nine FP32 populations: the sums of FP64
-// arithmetic, and their quotients rounded as above.  Where the populations are positive and their exponents span at most 25, the
-// moments are integers below 2^53 in units of the smallest population's last place: every
-// FP64 partial sum is exact, and so are these integer sums.  Other cells return false.
+// arithmetic, and their quotients rounded as above.  Where the populations are positive and
+// their exponents span at most 25, the moments are integers below 2^53 in units of the smallest
+// population's last place: every FP64 partial sum is exact, and so are these integer sums.
+// Other cells return false.
 __device__ __forceinline__ bool moments_exact(const float (&v)[9], double& rho, double& ux,
                                               double& uy) {
   uint32_t lo = 0xffffffffu, hi = 0u, b[9];

@@ -46,12 +46,13 @@ cudaError_t launch_step(const StepParams<T>& p, int mode, bool pull, bool store,
 // cost more than the idle SMs.  FP64 rows, bound by the FP64 pipes that unsplit blocks leave
 // idle, are shared out to half as many blocks again (in 32-row blocks, 114 on 152 SMs):
 // density step of 90 blocks 234 / 123 us, of smooth fields 126 / 98, of 112 blocks 260 / 145 and
-// 126 / 123; of 144 blocks 232 / 177, but of smooth fields 126 / 145.  {Kn, KL, neq} steps of the density step, unsplit / split,
-// us: FP32 256^2 (16 blocks) 15.4 / 6.8, 512^2 (64) 17.5 / 8.4, 768^2 (144) 18.4 / 11.2 (20.5
-// at one row per warp), 1024^2 (256) 21.7 / 32.8; FP64 64^2 (2) 322 / 21, 128^2 (8) 243 / 32,
-// 512x256 (64) 227 / 100; FP16 512^2 (32 blocks of 256 columns) 21.0 / 9.0, 768^2 (72)
-// 20.2 / 11.6, 1024^2 (128) 19.9 / 17.4.  All of Table 1, FP32, before the sums of a run's
-// steps were left to the next one: 256^2 44.7 / 15.1, 512^2 44.1 / 19.1, 768^2 46.4 / 33.0.
+// 126 / 123; of 144 blocks 232 / 177, but of smooth fields 126 / 145.
+// {Kn, KL, neq} steps of the density step, unsplit / split, us: FP32 256^2 (16 blocks)
+// 15.4 / 6.8, 512^2 (64) 17.5 / 8.4, 768^2 (144) 18.4 / 11.2 (20.5 at one row per warp), 1024^2
+// (256) 21.7 / 32.8; FP64 64^2 (2) 322 / 21, 128^2 (8) 243 / 32, 512x256 (64) 227 / 100; FP16
+// 512^2 (32 blocks of 256 columns) 21.0 / 9.0, 768^2 (72) 20.2 / 11.6, 1024^2 (128)
+// 19.9 / 17.4.  All of Table 1, FP32, before the sums of a run's steps were left to the next
+// one: 256^2 44.7 / 15.1, 512^2 44.1 / 19.1, 768^2 46.4 / 33.0.
 template <class T>
 int split_ranks(long long nblocks, int rows);
 // The same for the step that launch_step (pull + store) or launch_step_aar takes with these
