@@ -44,9 +44,9 @@ cudaError_t launch_step(const StepParams<T>& p, int mode, bool pull, bool store,
 // shared where the ranks, at one row per warp of eight (FP32 arithmetic: or two), all fit on
 // the GPU at once (two CTAs of 256 threads per SM); beyond that line the cluster's barriers
 // cost more than the idle SMs.  FP64 rows, bound by the FP64 pipes that unsplit blocks leave
-// idle, are shared out to half as many blocks again (in 32-row blocks, 114 on 152 SMs):
-// density step of 90 blocks 234 / 123 us, of smooth fields 126 / 98, of 112 blocks 260 / 145 and
-// 126 / 123; of 144 blocks 232 / 177, but of smooth fields 126 / 145.
+// idle, are shared out to 10/7 times as many blocks (in 32-row blocks, 108 on 152 SMs; single
+// steps, unsplit / split): density step of 90 blocks 168 / 115 us, of smooth fields 125 / 102, of
+// 108 blocks 167 / 131 and 120 / 118; of 112 blocks 168 / 144, but of smooth fields 120 / 127.
 // {Kn, KL, neq} steps of the density step, unsplit / split, us: FP32 256^2 (16 blocks)
 // 15.4 / 6.8, 512^2 (64) 17.5 / 8.4, 768^2 (144) 18.4 / 11.2 (20.5 at one row per warp), 1024^2
 // (256) 21.7 / 32.8; FP64 64^2 (2) 322 / 21, 128^2 (8) 243 / 32, 512x256 (64) 227 / 100; FP16

@@ -142,7 +142,7 @@ int split_ranks<KSS_T>(long long nblocks, int rows) {
   const long long slots = 2LL * sm_count();
   int ranks = std::min(rows / split_rows<KSS_T>(), 16);
   if (std::is_same<KSS_T, double>::value) {
-    if (2 * nblocks * (rows / kWarps) > 3 * slots) return 0;
+    if (7 * nblocks * (rows / kWarps) > 10 * slots) return 0;
   } else if (nblocks * (rows / kWarps) > slots) {
     // (two rows per warp where one each would not fit)
     if (nblocks * (rows / (2 * kWarps)) > slots) return 0;
